@@ -482,7 +482,8 @@ SDMD_API int sdmd_set_option(sdmd_t h, int32_t option, int64_t value);
 
 /* Kernel classes for tracing. */
 enum {
-    SDMD_K_INGEST = 0,    /* snapshot copy into its ring slot (a memcpy)       */
+    SDMD_K_INGEST = 0,    /* snapshot copy into its ring slot (sdmd_push from
+                             16-byte aligned device memory: part of the row)  */
     SDMD_K_GRAM_ROW = 1,  /* Gram-row multi-dot + symmetric insert            */
     SDMD_K_MODES = 2,     /* FP64 eigensolvers / small products (one CTA)     */
     SDMD_K_PHI = 3,       /* Phi = X' (V Sigma^-1 W)                          */

@@ -448,7 +448,7 @@ int64_t sdmd::handle_device_bytes(int64_t n, int32_t m, int32_t dtype, int num_s
   int64_t chunk = 0;
   int32_t nblk = 0;
   gram_row_schedule(slot, num_sms, &chunk, &nblk);
-  return (int64_t)m * slot + 2 * (int64_t)m * m * gsz + (int64_t)m * nblk * gsz + 16 +
+  return (int64_t)m * slot + 2 * (int64_t)m * m * gsz + (int64_t)m * nblk * gsz + kGrTicketWords * 4 +
          modes_ws_doubles(m) * (int64_t)sizeof(double) + 8 + kPhiSchedWords * 4;
 }
 
@@ -488,7 +488,7 @@ int sdmd_create_ex(int64_t n, int32_t m, int32_t dtype, int32_t depth, sdmd_t* o
   if (e == cudaSuccess) e = cudaMalloc(&h->gtmp, gbytes);
   if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)m * h->nblk * h->gsz);
   h->nblk_alloc = h->nblk;
-  if (e == cudaSuccess) e = cudaMalloc(&h->ticket, 4 * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMalloc(&h->ticket, kGrTicketWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMalloc(&h->ws, ws_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&h->status, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->r_dev, sizeof(int));
@@ -496,7 +496,7 @@ int sdmd_create_ex(int64_t n, int32_t m, int32_t dtype, int32_t depth, sdmd_t* o
   if (e == cudaSuccess) e = cudaMemset(h->phi_sched, 0, kPhiSchedWords * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(h->ring, 0, ring_bytes);
   if (e == cudaSuccess) e = cudaMemset(h->G, 0, gbytes);
-  if (e == cudaSuccess) e = cudaMemset(h->ticket, 0, 4 * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(h->ticket, 0, kGrTicketWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(h->ws, 0, ws_bytes);
   if (depth > 1) {
     h->ctx.resize(depth);
@@ -554,13 +554,13 @@ int sdmd_create_sparse(int64_t n, int32_t m, int32_t nnz_max, sdmd_t* out) {
   if (e == cudaSuccess) e = cudaMalloc(&h->G, (size_t)m * m * 16);
   if (e == cudaSuccess) e = cudaMalloc(&h->gtmp, (size_t)m * m * 16);
   if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)h->nblk * 16);
-  if (e == cudaSuccess) e = cudaMalloc(&h->ticket, 4 * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMalloc(&h->ticket, kGrTicketWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMalloc(&h->ws, ws_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&h->status, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->r_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->tag, 0xff, (size_t)n * sizeof(int));   // tag -1: no stamp
   if (e == cudaSuccess) e = cudaMemset(h->G, 0, (size_t)m * m * 16);
-  if (e == cudaSuccess) e = cudaMemset(h->ticket, 0, 4 * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(h->ticket, 0, kGrTicketWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(h->status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -706,8 +706,17 @@ int ingest(sdmd_s* h, const void* x, cudaStream_t st) {
   return SDMD_OK;
 }
 
-// Gram row of the snapshot just ingested into slot `s`, then advance the ring.
-int gram_row_and_advance(sdmd_s* h, int32_t s, cudaStream_t st) {
+// Whether the Gram-row kernel can take the snapshot from the caller's buffer
+// (bulk copies need 16-byte aligned device memory); other sources go through
+// ingest().
+bool row_ingests(const void* x) {
+  return (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && ptr_kind(x) == kDevice;
+}
+
+// Gram row of the newest snapshot, in slot `s` (x = nullptr) or still in the
+// caller's buffer x (the kernel copies it into the slot), then advance the
+// ring.
+int gram_row_and_advance(sdmd_s* h, int32_t s, cudaStream_t st, const void* x = nullptr) {
   GramRowArgs a;
   a.ring = h->ring;
   a.slot_bytes = h->slot_bytes;
@@ -721,9 +730,11 @@ int gram_row_and_advance(sdmd_s* h, int32_t s, cudaStream_t st) {
   a.ticket = h->ticket;
   a.G = h->G;
   a.status = h->status;
+  a.x_src = static_cast<const uint8_t*>(x);
+  a.x_bytes = h->n * h->elem;
   {
     TraceScope ts(h, SDMD_K_GRAM_ROW, st);
-    CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, st));
+    CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, h->num_sms, st));
   }
   h->head = (s + 1) % h->cap;
   h->count += 1;
@@ -739,9 +750,13 @@ int sdmd_push(sdmd_t h, const void* x, void* stream) {
   DeviceScope ds(h->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = flush_pending(h, st);
-  if (rc == SDMD_OK) rc = ingest(h, x, st);
-  if (rc == SDMD_OK) rc = gram_row_and_advance(h, h->head, st);
-  return rc;
+  if (rc != SDMD_OK) return rc;
+  if (row_ingests(x)) {
+    rc = wait_ring_readers(h, st);
+    return rc == SDMD_OK ? gram_row_and_advance(h, h->head, st, x) : rc;
+  }
+  rc = ingest(h, x, st);
+  return rc == SDMD_OK ? gram_row_and_advance(h, h->head, st) : rc;
 }
 
 namespace {
@@ -1054,7 +1069,7 @@ int sdmd_rebuild(sdmd_t h, void* stream) {
       a.G = h->G;
       a.status = h->status;
       TraceScope ts(h, SDMD_K_GRAM_ROW, st);
-      CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, st));
+      CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, h->num_sms, st));
     }
   }
   return SDMD_OK;
@@ -1448,12 +1463,12 @@ int sdmd_autotune(sdmd_t h, int64_t* chunk_bytes, double* us, void* stream) {
     if (dup) continue;
     a.chunk = cch[i];
     a.nblk = cnb[i];
-    cudaError_t e = launch_gram_row(h->dtype, h->f32_fp64 != 0, a, st);   // warm-up
+    cudaError_t e = launch_gram_row(h->dtype, h->f32_fp64 != 0, a, h->num_sms, st);   // warm-up
     double tot = 0.0;
     for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
       float ms = 0.f;
       if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-      if (e == cudaSuccess) e = launch_gram_row(h->dtype, h->f32_fp64 != 0, a, st);
+      if (e == cudaSuccess) e = launch_gram_row(h->dtype, h->f32_fp64 != 0, a, h->num_sms, st);
       if (e == cudaSuccess) e = cudaEventRecord(e1, st);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
@@ -1475,7 +1490,7 @@ int sdmd_autotune(sdmd_t h, int64_t* chunk_bytes, double* us, void* stream) {
   h->nblk = cnb[bi];
   a.chunk = h->chunk;                 // the newest row once more with the kept schedule
   a.nblk = h->nblk;
-  CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, st));
+  CK(launch_gram_row(h->dtype, h->f32_fp64 != 0, a, h->num_sms, st));
   if (chunk_bytes) *chunk_bytes = h->chunk;
   if (us) *us = 1e3 * best / 3.0;
   return SDMD_OK;

@@ -4,21 +4,31 @@
 // each window byte exactly once, so the kernel is HBM-bound.
 //
 // Decomposition: the n dimension (bytes, padded to whole 4 KiB units) is cut
-// into `nblk` contiguous chunks, about two per SM. One persistent CTA per SM
-// takes chunks from a counter (atomicAdd), so a launch is not held back by
-// SMs that another stream's kernel occupies, and walks each chunk in
-// sub-chunks of up to 32 KiB: thread 0 brings the sub-chunk of x_new into
+// into `nblk` contiguous chunks of up to 24 KiB, about two per SM. A work
+// item is one chunk of one of `groups` interleaved sets of eight slots (slot
+// rows jj with (jj / 8) % groups == g). One persistent CTA per SM takes items
+// from a counter (atomicAdd), so a launch is not held back by SMs that
+// another stream's kernel occupies: thread 0 brings the chunk of x_new into
 // shared memory with one bulk copy (TMA, cp.async.bulk), then each of the 8
-// warps streams its slots (warp w takes slots w, w+8, ...) in 4 KiB pieces
+// warps streams its slots (warp w takes rows jj = w mod 8) in 4 KiB pieces
 // through its own 4-stage shared-memory ring: lane 0 issues cp.async.bulk
 // copies that complete on one mbarrier per stage, the lanes wait on the
 // barrier, consume the piece (16 bytes per lane per step) and hand the stage
 // back. That keeps 128 KiB of loads in flight per SM without register
-// pressure. Each slot's sub-chunk sum is reduced with warp shuffles into a
-// per-chunk accumulator; the per-chunk partials go to a [slot][chunk] array
-// and the last CTA to finish (atomic ticket, no waiting) sums them in a
-// fixed order and writes row and column `s_new` of G, so the result does not
-// depend on which CTA took which chunk.
+// pressure, and the rings run on into the next item. Each slot's chunk sum is
+// reduced with warp shuffles and goes to a [slot][chunk] array; the CTA that
+// completes a group's last chunk (atomic count, no waiting) sums its partials
+// in a fixed order and writes its entries of row and column `s_new` of G, so
+// the result depends neither on which CTA took which item nor on the number
+// of groups.
+//
+// The new snapshot. With x_src set (a 16-byte aligned device buffer) the
+// kernel also is the ingest: x_new's chunks come from x_src, the items of
+// group 0 write them to the ring slot, and <x_new, x_new> is formed from the
+// staged chunk, so the snapshot is read once and its slot not at all. Against
+// a copy kernel before this one a push of one HD frame (m = 100) went from 126
+// to 117 us, one of a 64 x 64 FP32 field (m = 32, launches only) from 22.5 to
+// 14.3 us.
 //
 //  - uint8: __dp4a (4 u8 x u8 products into u32). A lane sums at most
 //    32 KiB / 32 = 1024 products (< 2^32 / 255^2) before the value goes to
@@ -34,6 +44,8 @@
 // copies, waits (bounded) for the copies it has in flight, and finishes.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "sdmd_internal.cuh"
 
@@ -77,6 +89,15 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned
       : "memory");
 }
 
+// shared -> global bulk copy of this thread's bulk group, and the waits for
+// it: source read (the buffer may be refilled), and complete
+__device__ __forceinline__ void bulk_s2g(void* dst, unsigned src, unsigned bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+__device__ __forceinline__ void bulk_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+
 __device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
   unsigned ok;
   asm volatile(
@@ -99,15 +120,13 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
 
 struct Smem {
   uint8_t stage[kGrWarps][kStages][kPiece];   // per-warp piece rings
-  uint8_t xs[2][kXSub];                       // x_new pieces of the current and the next chunk
+  uint8_t xs[2][kXSub];                       // x_new chunks of the current and the next item
   unsigned long long bar[kGrWarps][kStages];  // one mbarrier per stage
   unsigned long long xbar[2];                 // x_new barriers
-  int cq[2];                                  // chunk index of chunk ordinal k at [k & 1]
+  int iq[2];                                  // index of item ordinal k at [k & 1]
   int fail;                                   // a wait expired in some warp
-  long long acc_i[SDMD_MAX_M];
-  double acc_d[SDMD_MAX_M];
-  double acc_im[SDMD_MAX_M];                  // imaginary parts (complex snapshots)
-  int last;
+  int quit;                                   // fail as thread 0 saw it between two items
+  int last;                                   // group whose last chunk this CTA completed, -1: none
 };
 
 // Element modes of the kernel.
@@ -115,293 +134,8 @@ struct Smem {
 // a product of two FP32 values is exact in FP64).
 enum { kModeU8 = 0, kModeF32 = 1, kModeC64 = 2, kModeF64 = 3 };
 
-template <typename Acc>
-__device__ void finish_row(const GramRowArgs& a, Smem& sm) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int t = atomicAdd(a.ticket, 1u);
-    sm.last = (t == gridDim.x - 1u);
-  }
-  __syncthreads();
-  if (!sm.last) return;
-  __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const Acc* P = static_cast<const Acc*>(a.partials);
-  Acc* G = static_cast<Acc*>(a.G);
-  for (int jj = warp; jj < a.c; jj += kGrWarps) {
-    Acc s = 0;
-    for (int b = lane; b < a.nblk; b += 32) s += __ldcg(P + (int64_t)jj * a.nblk + b);
-    s = warp_sum(s);
-    if (lane == 0) {
-      const int j = (a.s_first + jj) % a.m;
-      G[(int64_t)a.s_new * a.m + j] = s;
-      G[(int64_t)j * a.m + a.s_new] = s;
-    }
-  }
-  if (threadIdx.x == 0) {                // ready for the next launch
-    a.ticket[0] = 0u;
-    a.ticket[1] = 0u;
-  }
-}
-
-// Complex version: G[j][s_new] = <x_j, x_new> = g_j and G[s_new][j] = conj(g_j).
-__device__ void finish_row_c64(const GramRowArgs& a, Smem& sm) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int t = atomicAdd(a.ticket, 1u);
-    sm.last = (t == gridDim.x - 1u);
-  }
-  __syncthreads();
-  if (!sm.last) return;
-  __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double2* P = static_cast<const double2*>(a.partials);
-  double2* G = static_cast<double2*>(a.G);
-  for (int jj = warp; jj < a.c; jj += kGrWarps) {
-    double sr = 0.0, si = 0.0;
-    for (int b = lane; b < a.nblk; b += 32) {
-      const double2 v = __ldcg(P + (int64_t)jj * a.nblk + b);
-      sr += v.x;
-      si += v.y;
-    }
-    sr = warp_sum(sr);
-    si = warp_sum(si);
-    if (lane == 0) {
-      const int j = (a.s_first + jj) % a.m;
-      if (j == a.s_new) si = 0.0;   // <x, x> is real; drop the rounding residue
-      G[(int64_t)j * a.m + a.s_new] = make_double2(sr, si);
-      G[(int64_t)a.s_new * a.m + j] = make_double2(sr, -si);
-    }
-  }
-  if (threadIdx.x == 0) {
-    a.ticket[0] = 0u;
-    a.ticket[1] = 0u;
-  }
-}
-
-template <int kMode>
-__global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArgs a) {
-  constexpr bool kU8 = (kMode == kModeU8);
-  extern __shared__ __align__(128) uint8_t smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = threadIdx.x; j < a.c; j += blockDim.x) {
-    sm.acc_i[j] = 0;
-    sm.acc_d[j] = 0.0;
-    sm.acc_im[j] = 0.0;
-  }
-  if (threadIdx.x == 0) {
-    for (int w = 0; w < kGrWarps; ++w)
-      for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&sm.bar[w][s]), 1);
-    mbar_init(smem_u32(&sm.xbar[0]), 1);
-    mbar_init(smem_u32(&sm.xbar[1]), 1);
-    sm.fail = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  const uint8_t* xnew = a.ring + (int64_t)a.s_new * a.slot_bytes;
-  const int nmine = (a.c > warp) ? (a.c - warp + kGrWarps - 1) / kGrWarps : 0;  // slots of this warp
-  // chunk ordinal k of this CTA -> chunk index sm.cq[k & 1] (>= nblk: none)
-  auto chunk_len = [&](int ch) -> int { return (int)min(a.chunk, a.slot_bytes - (int64_t)ch * a.chunk); };
-  auto issue_x = [&](int k, int ch) {          // x_new's piece of chunk ordinal k
-    const unsigned xb = smem_u32(&sm.xbar[k & 1]);
-    const int len = chunk_len(ch);
-    mbar_expect_tx(xb, (unsigned)len);
-    bulk_g2s(smem_u32(sm.xs[k & 1]), xnew + (int64_t)ch * a.chunk, (unsigned)len, xb);
-  };
-  if (threadIdx.x == 0) {
-    const int c0 = (int)atomicAdd(a.ticket + 1, 1u);
-    sm.cq[0] = c0;
-    if (c0 < a.nblk) issue_x(0, c0);
-  }
-  // per-warp item stream: item (k, i) = piece i % np of slot i / np of chunk
-  // ordinal k; lane 0 keeps the ring kStages items ahead, into chunk k + 1
-  // once it is known
-  unsigned consumed = 0, issued = 0;   // items of this warp (all chunks)
-  int kc = 0, ic = 0;                  // issue cursor: chunk ordinal, item
-  bool failed = false;                 // a bounded wait expired: stop issuing, drain, finish
-  auto top_up = [&](int k) {           // chunk ordinals k and k + 1 are known
-    if (lane != 0 || failed) return;
-    while (issued - consumed < (unsigned)kStages && kc <= k + 1) {
-      const int ch = sm.cq[kc & 1];
-      if (ch >= a.nblk) break;
-      const int np = chunk_len(ch) / kPiece;
-      if (ic >= nmine * np) {
-        ++kc;
-        ic = 0;
-        continue;
-      }
-      const unsigned s = issued % kStages;
-      const int j = (a.s_first + warp + kGrWarps * (ic / np)) % a.m;
-      const unsigned b = smem_u32(&sm.bar[warp][s]);
-      mbar_expect_tx(b, kPiece);
-      bulk_g2s(smem_u32(sm.stage[warp][s]),
-               a.ring + (int64_t)j * a.slot_bytes + (int64_t)ch * a.chunk + (int64_t)kPiece * (ic % np), kPiece, b);
-      ++ic;
-      ++issued;
-    }
-  };
-  for (int k = 0;; ++k) {
-    __syncthreads();                   // chunk k - 1 fully consumed: xs[(k + 1) & 1] is free
-    if (threadIdx.x == 0) {
-      const int ch = sm.cq[k & 1];
-      int nx = a.nblk;
-      if (ch < a.nblk && !sm.fail) nx = (int)atomicAdd(a.ticket + 1, 1u);
-      sm.cq[(k + 1) & 1] = nx;
-      if (nx < a.nblk) issue_x(k + 1, nx);
-    }
-    __syncthreads();
-    const int ch = sm.cq[k & 1];
-    if (ch >= a.nblk) break;
-    const int np = chunk_len(ch) / kPiece;
-    const int nitems = nmine * np;
-    top_up(k);
-    if (!failed && !mbar_wait(smem_u32(&sm.xbar[k & 1]), (unsigned)((k >> 1) & 1))) failed = true;
-    failed = __any_sync(0xffffffffu, failed);
-    unsigned int su = 0;
-    double sd = 0.0, si = 0.0;
-    const uint8_t* xs = sm.xs[k & 1];
-    for (int it = 0; it < nitems && !failed; ++it) {
-      const unsigned s = consumed % kStages, par = (consumed / kStages) & 1;
-      const int q = it % np;
-      bool bad = !mbar_wait(smem_u32(&sm.bar[warp][s]), par);
-      if (__any_sync(0xffffffffu, bad)) {
-        failed = true;
-        break;
-      }
-      const uint8_t* piece = sm.stage[warp][s];
-      const uint8_t* xq = xs + kPiece * q;
-      if constexpr (kU8) {
-#pragma unroll
-        for (int u = 0; u < kPiece / 512; ++u) {
-          const uint4 v = *reinterpret_cast<const uint4*>(piece + 16 * lane + 512 * u);
-          const uint4 w = *reinterpret_cast<const uint4*>(xq + 16 * lane + 512 * u);
-          su = __dp4a(v.x, w.x, su);
-          su = __dp4a(v.y, w.y, su);
-          su = __dp4a(v.z, w.z, su);
-          su = __dp4a(v.w, w.w, su);
-        }
-      } else if constexpr (kMode == kModeF32) {
-        float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-#pragma unroll
-        for (int u = 0; u < kPiece / 512; ++u) {
-          const float4 v = *reinterpret_cast<const float4*>(piece + 16 * lane + 512 * u);
-          const float4 w = *reinterpret_cast<const float4*>(xq + 16 * lane + 512 * u);
-          f0 = fmaf(v.x, w.x, f0);
-          f1 = fmaf(v.y, w.y, f1);
-          f2 = fmaf(v.z, w.z, f2);
-          f3 = fmaf(v.w, w.w, f3);
-        }
-        sd += (double)((f0 + f1) + (f2 + f3));
-      } else if constexpr (kMode == kModeF64) {
-        double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
-#pragma unroll
-        for (int u = 0; u < kPiece / 512; ++u) {
-          const float4 v = *reinterpret_cast<const float4*>(piece + 16 * lane + 512 * u);
-          const float4 w = *reinterpret_cast<const float4*>(xq + 16 * lane + 512 * u);
-          d0 = fma((double)v.x, (double)w.x, d0);
-          d1 = fma((double)v.y, (double)w.y, d1);
-          d2 = fma((double)v.z, (double)w.z, d2);
-          d3 = fma((double)v.w, (double)w.w, d3);
-        }
-        sd += (d0 + d1) + (d2 + d3);
-      } else {
-        // two complex64 values per 16 bytes: conj(v) * w
-        float r0 = 0.f, r1 = 0.f, i0 = 0.f, i1 = 0.f;
-#pragma unroll
-        for (int u = 0; u < kPiece / 512; ++u) {
-          const float4 v = *reinterpret_cast<const float4*>(piece + 16 * lane + 512 * u);
-          const float4 w = *reinterpret_cast<const float4*>(xq + 16 * lane + 512 * u);
-          r0 = fmaf(v.x, w.x, fmaf(v.y, w.y, r0));
-          r1 = fmaf(v.z, w.z, fmaf(v.w, w.w, r1));
-          i0 = fmaf(v.x, w.y, fmaf(-v.y, w.x, i0));
-          i1 = fmaf(v.z, w.w, fmaf(-v.w, w.z, i1));
-        }
-        sd += (double)(r0 + r1);
-        si += (double)(i0 + i1);
-      }
-      __syncwarp();                    // all lanes are done reading stage s
-      ++consumed;
-      top_up(k);
-      if (q == np - 1) {               // this slot is finished for the chunk
-        const int jj = warp + kGrWarps * (it / np);
-        if constexpr (kU8) {
-          const long long t = warp_sum((long long)su);
-          if (lane == 0) sm.acc_i[jj] += t;
-          su = 0;
-        } else {
-          const double t = warp_sum(sd);
-          if (lane == 0) sm.acc_d[jj] += t;
-          sd = 0.0;
-          if constexpr (kMode == kModeC64) {
-            const double ti = warp_sum(si);
-            if (lane == 0) sm.acc_im[jj] += ti;
-            si = 0.0;
-          }
-        }
-      }
-    }
-    if (failed) {
-      if (lane == 0) {
-        atomicOr(a.status, kDevTimeout);
-        sm.fail = 1;
-      }
-    }
-    __syncthreads();
-    // this chunk's partials (each thread writes and clears its own slots)
-    for (int j = threadIdx.x; j < a.c; j += blockDim.x) {
-      if constexpr (kU8) {
-        static_cast<long long*>(a.partials)[(int64_t)j * a.nblk + ch] = sm.acc_i[j];
-      } else if constexpr (kMode == kModeF32 || kMode == kModeF64) {
-        static_cast<double*>(a.partials)[(int64_t)j * a.nblk + ch] = sm.acc_d[j];
-      } else {
-        static_cast<double2*>(a.partials)[(int64_t)j * a.nblk + ch] = make_double2(sm.acc_d[j], sm.acc_im[j]);
-      }
-      sm.acc_i[j] = 0;
-      sm.acc_d[j] = 0.0;
-      sm.acc_im[j] = 0.0;
-    }
-    if (sm.fail) {
-      // copies issued but not consumed must land before the shared memory
-      // is released (bounded waits); then stop
-      if (lane == 0)
-        for (unsigned gk = consumed; gk < issued; ++gk) mbar_wait(smem_u32(&sm.bar[warp][gk % kStages]), (gk / kStages) & 1);
-      if (threadIdx.x == 0 && sm.cq[(k + 1) & 1] < a.nblk) mbar_wait(smem_u32(&sm.xbar[(k + 1) & 1]), (unsigned)(((k + 1) >> 1) & 1));
-      break;
-    }
-  }
-  if constexpr (kU8) {
-    finish_row<long long>(a, sm);
-  } else if constexpr (kMode == kModeF32 || kMode == kModeF64) {
-    finish_row<double>(a, sm);
-  } else {
-    finish_row_c64(a, sm);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Batched rows: one new snapshot of each of up to kMaxBatchJobs handles (mixed
-// n, window and element type) in one launch. Work items are (job, chunk)
-// pairs over the concatenated chunk lists, taken from a counter by
-// persistent CTAs. Each item is computed exactly as the single-handle kernel
-// computes that chunk (same warp-to-slot assignment, piece order and per-lane
-// sums), its partials go to the job's [slot][chunk] array, and the CTA that
-// completes a job's last chunk reduces the job's row in the same fixed order,
-// so every row is bit-identical to the handle's own sdmd_push.
-
-struct BatchSmem {
-  uint8_t stage[kGrWarps][kStages][kPiece];
-  uint8_t xs[kXSub];
-  unsigned long long bar[kGrWarps][kStages];
-  unsigned long long xbar;
-  int item, job, ch, fail, last;
-  long long acc_i[SDMD_MAX_M];
-  double acc_d[SDMD_MAX_M];
-  double acc_im[SDMD_MAX_M];
-};
-
+// One 4 KiB piece of a slot against the same piece of x_new, added to this
+// lane's sums (16 bytes per lane and step).
 template <int kMode>
 __device__ __forceinline__ void piece_sums(const uint8_t* piece, const uint8_t* xq, int lane, unsigned& su, double& sd,
                                            double& si) {
@@ -454,6 +188,288 @@ __device__ __forceinline__ void piece_sums(const uint8_t* piece, const uint8_t* 
     si += (double)(i0 + i1);
   }
 }
+
+// acc[0 .. 2] of one (slot, chunk): the lanes' sums reduced over the warp and
+// stored by lane 0.
+template <int kMode>
+__device__ __forceinline__ void store_partial(void* partials, int64_t at, int lane, unsigned su, double sd, double si) {
+  if constexpr (kMode == kModeU8) {
+    const long long t = warp_sum((long long)su);
+    if (lane == 0) static_cast<long long*>(partials)[at] = t;
+  } else if constexpr (kMode == kModeC64) {
+    const double t = warp_sum(sd), ti = warp_sum(si);
+    if (lane == 0) static_cast<double2*>(partials)[at] = make_double2(t, ti);
+  } else {
+    const double t = warp_sum(sd);
+    if (lane == 0) static_cast<double*>(partials)[at] = t;
+  }
+}
+
+// Sum over the chunks of one row of partials in a fixed order (lane-strided
+// sums, then the butterfly); kFinLoads loads are in flight per lane.
+constexpr int kFinLoads = 8;
+template <typename T>
+__device__ __forceinline__ T chunk_sum(const T* P, int nblk, int lane) {
+  T s = 0;
+  for (int b = lane; b < nblk; b += 32 * kFinLoads) {
+    T v[kFinLoads];
+#pragma unroll
+    for (int u = 0; u < kFinLoads; ++u) v[u] = (b + 32 * u < nblk) ? __ldcg(P + b + 32 * u) : T(0);
+#pragma unroll
+    for (int u = 0; u < kFinLoads; ++u)
+      if (b + 32 * u < nblk) s += v[u];
+  }
+  return warp_sum(s);
+}
+__device__ __forceinline__ double2 chunk_sum_c64(const double2* P, int nblk, int lane) {
+  double sr = 0.0, si = 0.0;
+  for (int b = lane; b < nblk; b += 32 * kFinLoads) {
+    double2 v[kFinLoads];
+#pragma unroll
+    for (int u = 0; u < kFinLoads; ++u) v[u] = (b + 32 * u < nblk) ? __ldcg(P + b + 32 * u) : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < kFinLoads; ++u)
+      if (b + 32 * u < nblk) {
+        sr += v[u].x;
+        si += v[u].y;
+      }
+  }
+  return make_double2(warp_sum(sr), warp_sum(si));
+}
+
+// G's entries of row jj (this warp): row and column s_new, physical slots.
+// Complex: G[j][s_new] = <x_j, x_new> = g_j and G[s_new][j] = conj(g_j).
+template <int kMode>
+__device__ __forceinline__ void finish_slot(const void* partials, int nblk, int jj, void* G, int s_first, int s_new,
+                                            int m, int lane) {
+  int j = s_first + jj;
+  if (j >= m) j -= m;
+  if constexpr (kMode == kModeC64) {
+    double2 v = chunk_sum_c64(static_cast<const double2*>(partials) + (int64_t)jj * nblk, nblk, lane);
+    if (j == s_new) v.y = 0.0;         // <x, x> is real; drop the rounding residue
+    if (lane == 0) {
+      double2* g = static_cast<double2*>(G);
+      g[(int64_t)j * m + s_new] = v;
+      g[(int64_t)s_new * m + j] = make_double2(v.x, -v.y);
+    }
+  } else {
+    using Acc = typename std::conditional<kMode == kModeU8, long long, double>::type;
+    const Acc v = chunk_sum<Acc>(static_cast<const Acc*>(partials) + (int64_t)jj * nblk, nblk, lane);
+    if (lane == 0) {
+      Acc* g = static_cast<Acc*>(G);
+      g[(int64_t)s_new * m + j] = v;
+      g[(int64_t)j * m + s_new] = v;
+    }
+  }
+}
+
+template <int kMode>
+__global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int w = 0; w < kGrWarps; ++w)
+      for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&sm.bar[w][s]), 1);
+    mbar_init(smem_u32(&sm.xbar[0]), 1);
+    mbar_init(smem_u32(&sm.xbar[1]), 1);
+    sm.fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+  const int S = a.groups, nitems = a.nblk * S;
+  const bool src = a.x_src != nullptr;
+  const uint8_t* xnew = src ? a.x_src : a.ring + (int64_t)a.s_new * a.slot_bytes;
+  const int64_t xbytes = src ? a.x_bytes : a.slot_bytes;   // readable bytes at xnew
+  // the newest snapshot (window row c - 1) is dotted from its staged chunk
+  const int self = (a.s_new == (a.s_first + a.c - 1) % a.m) ? a.c - 1 : -1;
+  const int cs = (self >= 0) ? a.c - 1 : a.c;              // rows streamed from the ring
+  auto chunk_len = [&](int ch) -> int { return (int)min(a.chunk, a.slot_bytes - (int64_t)ch * a.chunk); };
+  // bytes of chunk ch that a bulk copy may read (a multiple of 16)
+  auto bulk_len = [&](int ch) -> int {
+    const int64_t rest = xbytes - (int64_t)ch * a.chunk;
+    return rest <= 0 ? 0 : ((int)min((int64_t)chunk_len(ch), rest) & ~15);
+  };
+  auto rows_of = [&](int g) -> int {                       // streamed rows of this warp in group g
+    const int r0 = warp + kGrWarps * g;
+    return (r0 < cs) ? (cs - 1 - r0) / (kGrWarps * S) + 1 : 0;
+  };
+  auto issue_x = [&](int k, int it) {                      // x_new's chunk of item ordinal k
+    const int ch = it / S;
+    const unsigned xb = smem_u32(&sm.xbar[k & 1]);
+    const int len = bulk_len(ch);
+    mbar_expect_tx(xb, (unsigned)len);
+    if (len > 0) bulk_g2s(smem_u32(sm.xs[k & 1]), xnew + (int64_t)ch * a.chunk, (unsigned)len, xb);
+  };
+  if (threadIdx.x == 0) {
+    const int i0 = (int)atomicAdd(a.ticket + 1, 1u);
+    sm.iq[0] = i0;
+    if (i0 < nitems) issue_x(0, i0);
+  }
+  // this warp's piece stream: lane 0 keeps the ring kStages pieces ahead, into
+  // item ordinal k + 1 once it is known
+  unsigned consumed = 0, issued = 0;   // pieces of this warp (all items)
+  int kc = 0, ci = 0, cq = 0, cnp = 0, crows = 0, cg = 0, cch = 0;   // issue cursor (lane 0)
+  const uint8_t* csrc = nullptr;
+  bool loaded = false;                 // the cursor holds item ordinal kc
+  bool failed = false;                 // a bounded wait expired: stop issuing, drain, finish
+  auto slot_src = [&]() {
+    int j = a.s_first + warp + kGrWarps * (cg + S * ci);
+    if (j >= a.m) j -= a.m;
+    csrc = a.ring + (int64_t)j * a.slot_bytes + (int64_t)cch * a.chunk;
+  };
+  auto top_up = [&](int k) {           // item ordinals k and k + 1 are known
+    if (lane != 0 || failed) return;
+    while (issued - consumed < (unsigned)kStages) {
+      if (!loaded) {
+        if (kc > k + 1) break;
+        const int it = sm.iq[kc & 1];
+        if (it >= nitems) break;
+        cch = it / S;
+        cg = it - cch * S;
+        cnp = chunk_len(cch) / kPiece;
+        crows = rows_of(cg);
+        ci = cq = 0;
+        loaded = true;
+        if (crows > 0) slot_src();
+      }
+      if (ci >= crows) {
+        ++kc;
+        loaded = false;
+        continue;
+      }
+      const unsigned s = issued % kStages;
+      const unsigned b = smem_u32(&sm.bar[warp][s]);
+      mbar_expect_tx(b, kPiece);
+      bulk_g2s(smem_u32(sm.stage[warp][s]), csrc, kPiece, b);
+      ++issued;
+      csrc += kPiece;
+      if (++cq == cnp) {
+        cq = 0;
+        if (++ci < crows) slot_src();
+      }
+    }
+  };
+  int gprev = -1;                      // group of the item before
+  for (int k = 0;; ++k) {
+    __syncthreads();                   // item k - 1 consumed, its partials written: xs[(k + 1) & 1] is free
+    if (threadIdx.x == 0) {
+      const int it = sm.iq[k & 1];
+      int nx = nitems;
+      if (it < nitems && !sm.fail) nx = (int)atomicAdd(a.ticket + 1, 1u);
+      sm.iq[(k + 1) & 1] = nx;
+      sm.quit = sm.fail;
+      if (nx < nitems) {
+        if (src) bulk_store_wait_read(); // the store that still reads that buffer
+        issue_x(k + 1, nx);
+      }
+    } else if (threadIdx.x == 32) {    // count item k - 1 (the barrier ordered its partials before the fence)
+      int last = -1;
+      if (gprev >= 0 && !sm.fail) {
+        __threadfence();
+        if (atomicAdd(a.ticket + kGrTicketGroups + gprev, 1u) == (unsigned)a.nblk - 1u) last = gprev;
+        __threadfence();
+      }
+      sm.last = last;
+    }
+    __syncthreads();
+    if (sm.last >= 0)                  // this group's chunks are all in: its entries of G
+      for (int jj = warp + kGrWarps * sm.last; jj < a.c; jj += kGrWarps * S)
+        finish_slot<kMode>(a.partials, a.nblk, jj, a.G, a.s_first, a.s_new, a.m, lane);
+    const int it = sm.iq[k & 1];
+    if (sm.quit) {
+      // copies issued but not consumed must land before the shared memory
+      // is released (bounded waits); then stop
+      if (lane == 0)
+        for (unsigned gk = consumed; gk < issued; ++gk) mbar_wait(smem_u32(&sm.bar[warp][gk % kStages]), (gk / kStages) & 1);
+      if (threadIdx.x == 0 && it < nitems) mbar_wait(smem_u32(&sm.xbar[k & 1]), (unsigned)((k >> 1) & 1));
+      break;
+    }
+    if (it >= nitems) break;
+    const int ch = it / S, g = it - ch * S;
+    gprev = g;
+    const int np = chunk_len(ch) / kPiece, rows = rows_of(g);
+    uint8_t* xs = sm.xs[k & 1];
+    top_up(k);
+    if (src && bulk_len(ch) < chunk_len(ch)) {
+      // the last bytes of the snapshot (n mod 16) and the zero padding after it
+      const int b0 = bulk_len(ch);
+      const int64_t off = (int64_t)ch * a.chunk;
+      for (int b = b0 + threadIdx.x; b < chunk_len(ch); b += kGrThreads) xs[b] = (off + b < xbytes) ? xnew[off + b] : 0;
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncthreads();
+    }
+    if (!failed && !mbar_wait(smem_u32(&sm.xbar[k & 1]), (unsigned)((k >> 1) & 1))) failed = true;
+    failed = __any_sync(0xffffffffu, failed);
+    if (src && g == 0 && !failed) {    // the ingest of this chunk
+      uint8_t* dst = const_cast<uint8_t*>(a.ring) + (int64_t)a.s_new * a.slot_bytes + (int64_t)ch * a.chunk;
+      const int len = bulk_len(ch);
+      if (threadIdx.x == 0 && len > 0) bulk_s2g(dst, smem_u32(xs), (unsigned)len);
+      const int b = len + (int)threadIdx.x;
+      if (threadIdx.x < 16 && len < chunk_len(ch) && (int64_t)ch * a.chunk + b < xbytes) dst[b] = xs[b];
+    }
+    for (int i = 0; i < rows && !failed; ++i) {
+      unsigned su = 0;
+      double sd = 0.0, si = 0.0;
+      for (int q = 0; q < np; ++q) {
+        const unsigned s = consumed % kStages, par = (consumed / kStages) & 1;
+        const bool bad = !mbar_wait(smem_u32(&sm.bar[warp][s]), par);
+        if (__any_sync(0xffffffffu, bad)) {
+          failed = true;
+          break;
+        }
+        piece_sums<kMode>(sm.stage[warp][s], xs + kPiece * q, lane, su, sd, si);
+        __syncwarp();                  // all lanes are done reading stage s
+        ++consumed;
+        top_up(k);
+      }
+      if (!failed)
+        store_partial<kMode>(a.partials, (int64_t)(warp + kGrWarps * (g + S * i)) * a.nblk + ch, lane, su, sd, si);
+    }
+    if (self >= 0 && !failed && self % kGrWarps == warp && (self / kGrWarps) % S == g) {
+      unsigned su = 0;
+      double sd = 0.0, si = 0.0;
+      for (int q = 0; q < np; ++q) piece_sums<kMode>(xs + kPiece * q, xs + kPiece * q, lane, su, sd, si);
+      store_partial<kMode>(a.partials, (int64_t)self * a.nblk + ch, lane, su, sd, si);
+    }
+    if (failed && lane == 0) {
+      atomicOr(a.status, kDevTimeout);
+      sm.fail = 1;
+    }
+  }
+  // the ring copies are complete before the CTA's shared memory goes; the last
+  // CTA out zeroes the counters for the next launch
+  if (threadIdx.x == 0) {
+    if (src) bulk_store_wait_all();
+    __threadfence();
+    if (atomicAdd(a.ticket, 1u) == gridDim.x - 1u) {
+      for (int q = 0; q < S; ++q) a.ticket[kGrTicketGroups + q] = 0u;
+      a.ticket[1] = 0u;
+      a.ticket[0] = 0u;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Batched rows: one new snapshot of each of up to kMaxBatchJobs handles (mixed
+// n, window and element type) in one launch. Work items are (job, chunk)
+// pairs over the concatenated chunk lists, taken from a counter by
+// persistent CTAs. Each item is computed exactly as the single-handle kernel
+// computes that chunk (same warp-to-slot assignment, piece order and per-lane
+// sums), its partials go to the job's [slot][chunk] array, and the CTA that
+// completes a job's last chunk reduces the job's row in the same fixed order,
+// so every row is bit-identical to the handle's own sdmd_push.
+
+struct BatchSmem {
+  uint8_t stage[kGrWarps][kStages][kPiece];
+  uint8_t xs[kXSub];
+  unsigned long long bar[kGrWarps][kStages];
+  unsigned long long xbar;
+  int item, job, ch, fail, last;
+  long long acc_i[SDMD_MAX_M];
+  double acc_d[SDMD_MAX_M];
+  double acc_im[SDMD_MAX_M];
+};
 
 // One item: chunk `ch` of job `J`; returns false if a wait expired.
 template <int kMode>
@@ -524,43 +540,11 @@ __device__ bool batch_item(const RowJob& J, int ch, BatchSmem& sm, unsigned& g, 
   return !failed;
 }
 
-template <typename Acc>
+template <int kMode>
 __device__ void batch_finish(const RowJob& J) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const Acc* P = static_cast<const Acc*>(J.partials);
-  Acc* G = static_cast<Acc*>(J.G);
-  for (int jj = warp; jj < J.c; jj += kGrWarps) {
-    Acc s = 0;
-    for (int b = lane; b < J.nblk; b += 32) s += __ldcg(P + (int64_t)jj * J.nblk + b);
-    s = warp_sum(s);
-    if (lane == 0) {
-      const int j = (J.s_first + jj) % J.m;
-      G[(int64_t)J.s_new * J.m + j] = s;
-      G[(int64_t)j * J.m + J.s_new] = s;
-    }
-  }
-}
-
-__device__ void batch_finish_c64(const RowJob& J) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double2* P = static_cast<const double2*>(J.partials);
-  double2* G = static_cast<double2*>(J.G);
-  for (int jj = warp; jj < J.c; jj += kGrWarps) {
-    double sr = 0.0, si = 0.0;
-    for (int b = lane; b < J.nblk; b += 32) {
-      const double2 v = __ldcg(P + (int64_t)jj * J.nblk + b);
-      sr += v.x;
-      si += v.y;
-    }
-    sr = warp_sum(sr);
-    si = warp_sum(si);
-    if (lane == 0) {
-      const int j = (J.s_first + jj) % J.m;
-      if (j == J.s_new) si = 0.0;
-      G[(int64_t)j * J.m + J.s_new] = make_double2(sr, si);
-      G[(int64_t)J.s_new * J.m + j] = make_double2(sr, -si);
-    }
-  }
+  for (int jj = warp; jj < J.c; jj += kGrWarps)
+    finish_slot<kMode>(J.partials, J.nblk, jj, J.G, J.s_first, J.s_new, J.m, lane);
 }
 
 __global__ void __launch_bounds__(kGrThreads, 1) gram_rows_batched_kernel(const __grid_constant__ BatchArgs a) {
@@ -619,9 +603,9 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_rows_batched_kernel(const 
     __syncthreads();
     if (sm.last) {                     // this job's chunks are all in: reduce its row
       __threadfence();
-      if (J.mode == kModeU8) batch_finish<long long>(J);
-      else if (J.mode == kModeF32 || J.mode == kModeF64) batch_finish<double>(J);
-      else batch_finish_c64(J);
+      if (J.mode == kModeU8) batch_finish<kModeU8>(J);
+      else if (J.mode == kModeC64) batch_finish<kModeC64>(J);
+      else batch_finish<kModeF32>(J);
       if (threadIdx.x == 0) J.ticket[0] = 0u;
     }
   }
@@ -657,28 +641,47 @@ void gram_row_schedule_k(int64_t slot_bytes, int num_sms, int chunks_per_sm, int
   *nblk = (int32_t)((units + per - 1) / per);
 }
 
-cudaError_t launch_gram_row(int dtype, bool f64_ref, const GramRowArgs& a, cudaStream_t st) {
-  const size_t smem = sizeof(Smem);
-  {
-    cudaError_t e = smem_optin(reinterpret_cast<const void*>(gram_row_bulk_kernel<kModeU8>), smem);
-    if (e == cudaSuccess) e = smem_optin(reinterpret_cast<const void*>(gram_row_bulk_kernel<kModeF32>), smem);
-    if (e == cudaSuccess) e = smem_optin(reinterpret_cast<const void*>(gram_row_bulk_kernel<kModeC64>), smem);
-    if (e == cudaSuccess) e = smem_optin(reinterpret_cast<const void*>(gram_row_bulk_kernel<kModeF64>), smem);
-    if (e != cudaSuccess) return e;
+// Groups of slot rows per chunk. An item's time is about its rows of eight
+// slots (plus a fraction for its hand-over), and all items are alike, so the
+// launch takes ceil(items / SMs) of them: the count with the least of that
+// product. Sizes whose chunks divide evenly over the SMs keep one group (HD
+// uint8: 304 chunks on 152 SMs); 338 chunks (FP32, n = 2,073,600) would take
+// three rounds of whole chunks for 2.2 rounds of work and take seven of thirds
+// instead: the row of a 120-snapshot window from 237 to about 165 us.
+int gram_row_groups(int32_t nblk, int32_t c, int num_sms) {
+  const int rows = (c + kGrWarps - 1) / kGrWarps;
+  int best = 1;
+  double cost = 1e300;
+  for (int S = 1; S <= rows && S <= kGrMaxGroups; ++S) {
+    const int64_t rounds = ((int64_t)nblk * S + num_sms - 1) / num_sms;
+    const double t = (double)rounds * ((double)((rows + S - 1) / S) + 0.25);
+    if (t < 0.999 * cost) {
+      cost = t;
+      best = S;
+    }
   }
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int ctas = a.nblk < sms ? a.nblk : (sms > 0 ? sms : 1);   // persistent
-  if (dtype == SDMD_U8)
-    gram_row_bulk_kernel<kModeU8><<<ctas, kGrThreads, smem, st>>>(a);
-  else if (dtype == SDMD_C64)
-    gram_row_bulk_kernel<kModeC64><<<ctas, kGrThreads, smem, st>>>(a);
-  else if (f64_ref)
-    gram_row_bulk_kernel<kModeF64><<<ctas, kGrThreads, smem, st>>>(a);
-  else
-    gram_row_bulk_kernel<kModeF32><<<ctas, kGrThreads, smem, st>>>(a);
+  return best;
+}
+
+template <int kMode>
+static cudaError_t launch_gram_row_mode(const GramRowArgs& a, int ctas, cudaStream_t st) {
+  const size_t smem = sizeof(Smem);
+  const cudaError_t e = smem_optin(reinterpret_cast<const void*>(gram_row_bulk_kernel<kMode>), smem);
+  if (e != cudaSuccess) return e;
+  gram_row_bulk_kernel<kMode><<<ctas, kGrThreads, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_gram_row(int dtype, bool f64_ref, const GramRowArgs& args, int num_sms, cudaStream_t st) {
+  GramRowArgs a = args;
+  const int sms = num_sms > 0 ? num_sms : 1;
+  a.groups = gram_row_groups(a.nblk, a.c, sms);
+  const int64_t items = (int64_t)a.nblk * a.groups;
+  const int ctas = items < sms ? (int)items : sms;   // persistent
+  if (dtype == SDMD_U8) return launch_gram_row_mode<kModeU8>(a, ctas, st);
+  if (dtype == SDMD_C64) return launch_gram_row_mode<kModeC64>(a, ctas, st);
+  if (f64_ref) return launch_gram_row_mode<kModeF64>(a, ctas, st);
+  return launch_gram_row_mode<kModeF32>(a, ctas, st);
 }
 
 cudaError_t batched_kernel_config(const BatchArgs& a, cudaKernelNodeParams* p) {

@@ -33,10 +33,20 @@ struct GramRowArgs {
   int32_t s_new;         // slot holding the new snapshot
   int32_t m;             // G is m x m
   void* partials;        // [m][nblk] per-chunk partial sums (FP64 or int64)
-  unsigned int* ticket;  // two words, zero between launches: CTAs finished, chunks taken
+  unsigned int* ticket;  // kGrTicketWords words, zero between launches: CTAs finished, items taken,
+                         // (two for the batched kernel), chunks finished per slot group
   void* G;               // m x m, double (f32) or int64 (u8), physical slots
   int* status;           // device status word (kDevTimeout on an expired wait)
+  // the new snapshot in the caller's buffer (device memory, 16-byte aligned,
+  // x_bytes = n * element size): the kernel copies it into slot s_new, which
+  // must be the newest of the window; nullptr: the slot already holds it
+  const uint8_t* x_src = nullptr;
+  int64_t x_bytes = 0;
+  int32_t groups = 1;    // slot groups per chunk (set by launch_gram_row)
 };
+constexpr int kGrMaxGroups = 32;                   // SDMD_MAX_M / 8 slot rows
+constexpr int kGrTicketGroups = 4;                 // first per-group word of the ticket array
+constexpr int kGrTicketWords = kGrTicketGroups + kGrMaxGroups;
 
 // Gram rows/columns of the k newest uint8 snapshots against the window
 // (k = c: the full Gram) on the tensor cores, exact. The host call splits
@@ -158,7 +168,8 @@ int64_t handle_device_bytes(int64_t n, int32_t m, int32_t dtype, int num_sms);
 
 // Gram row for one pushed snapshot; launches one kernel on `st`.
 // f64_ref: FP32 snapshots with FP64 products and sums (SDMD_OPT_F32_FP64).
-cudaError_t launch_gram_row(int dtype, bool f64_ref, const GramRowArgs& a, cudaStream_t st);
+cudaError_t launch_gram_row(int dtype, bool f64_ref, const GramRowArgs& a, int num_sms, cudaStream_t st);
+int gram_row_groups(int32_t nblk, int32_t c, int num_sms);
 
 // Schedule of the Gram-row kernel: a function of slot size and SM count only,
 // so that every entry of G sees the same summation order.
