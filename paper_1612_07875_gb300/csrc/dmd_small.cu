@@ -35,10 +35,13 @@
 //     eigenvectors; eigenpairs ordered by descending |lambda| then angle.
 //  8. M = vsi W in df64, written in FP32 (scaled back) for the Phi kernel;
 //     lambda, sigma and V written out in FP64.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <float.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "df64.cuh"
 #include "sdmd_internal.cuh"
@@ -47,18 +50,19 @@ namespace sdmd {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
+constexpr int kParts = 8;                        // row classes of the tridiagonalisation's sums
+constexpr int kClusterCtas = 4;                  // CTAs that share a window whose G_X exceeds one SM
 constexpr double kEps = 2.220446049250313e-16;   // 2^-52 (rank rule, as the oracle)
 constexpr double kRankRtol = 64.0;               // rank threshold factor (times p * eps)
 constexpr float kEps32 = 5.9604645e-8f;          // 2^-24
 constexpr int kInvIters = 2;                     // inverse-iteration solves per vector and round
 constexpr int kMsRounds = 8;                     // FP32 multisection rounds (33-way each)
 constexpr int kJacobiSweeps = 12;                // Rayleigh-Ritz Jacobi sweep cap
-constexpr int kSmemMaxP = 144;                   // G_X kept in shared memory up to this p
+constexpr int kSmemMaxP = 144;                   // G_X in one SM's shared memory up to this p, else over a cluster
 constexpr int kRRMax = 32;                       // Rayleigh-Ritz matrices in smem up to this r
 constexpr int kClusterExt = 8;                   // eigenvalues added to close a cluster at the boundary
-constexpr int kEigMaxR = 48;                     // FP32 eig workspace in smem up to this r
 
 // ------------------------------------------------------------ helpers ----
 __device__ __forceinline__ dd shfl_dd(dd v, int o) {
@@ -107,7 +111,7 @@ __device__ __forceinline__ CF csqrt(CF z) {
 }
 
 struct WS {
-  dd *GXYd, *Ad, *Z, *Y, *lu;
+  dd *GXYt, *HV, *Z, *Y, *lu;
   double *V, *sig, *lamout, *bamp;
   float* Mf;
   long long* clk;
@@ -115,8 +119,8 @@ struct WS {
 
 __device__ WS carve(double* base, const ModesLayout& L) {
   WS w;
-  w.GXYd = reinterpret_cast<dd*>(base + L.GXY);
-  w.Ad = reinterpret_cast<dd*>(base + L.A);
+  w.GXYt = reinterpret_cast<dd*>(base + L.GXY);
+  w.HV = reinterpret_cast<dd*>(base + L.A);
   w.Z = reinterpret_cast<dd*>(base + L.Z);
   w.Y = reinterpret_cast<dd*>(base + L.Y);
   w.lu = reinterpret_cast<dd*>(base + L.lu);
@@ -130,31 +134,46 @@ __device__ WS carve(double* base, const ModesLayout& L) {
 }
 
 // ---------------------------------------------------------------- phase 1 --
-// df64 Householder reduction of the symmetric p x p matrix A (row-major,
-// full storage) to tridiagonal form (d, e). Reflector k is I - 2 v v^T on
-// indices k+1..p-1 with v unit (zero if column k is already reduced); it is
-// stored down column k, A[k+1..p-1][k].
+// df64 Householder reduction of the symmetric p x p matrix A (full storage)
+// to tridiagonal form (d, e). Reflector k is I - 2 v v^T on indices
+// k+1..p-1 with v unit (zero if column k is already reduced); it is kept in
+// HV[k * p + g].
 //
-// One block barrier per step. Step k's rank-2 update A -= v w^T + w v^T
-// (w = 2 (A v - (v^T A v) v)) is not applied in step k: step k+1 applies it
-// while it reads the trailing block for its own product A u, so the block is
-// read and written once per step. Warp w owns trailing rows w, w + 8, ...
-// and lane l columns l, l + 32, ...; as the block is symmetric, the row sums
-// of A u are also its column sums, so each lane sums its columns over its
-// warp's rows, and u^T A u comes from the same column sums. After the
-// barrier every warp adds the eight warps' parts for its lanes' columns and
-// forms v, A v and w itself, then the next pivot row, its norm and the
-// reflector's scalars: the same operations in the same order in every warp,
-// so all warps hold the same bits without a second barrier. The block stays
-// exactly symmetric: the update term of (i, j) is formed from the same
+// Step k's rank-2 update A -= v w^T + w v^T (w = 2 (A v - (v^T A v) v)) is
+// not applied in step k but at the start of step k+1, beside the scalar chain
+// that forms that step's reflector:
+//   1. warps 8.. form w and update pivot row k; then warp 0 takes the row's
+//      norm and forms u (v = u inv) while the other warps apply the pending
+//      update to the trailing block. The scalar chain (two square roots and a
+//      reciprocal in df64 behind a warp butterfly) takes about 1 k cycles
+//      whatever p, which is what the update of a p of about 100 takes.
+//   2. A u: as the block is symmetric, its row sums are its column sums; the
+//      trailing rows form kParts classes (row k+1+i in class i mod 8), and
+//      every lane sums the columns of its warp over one class's rows, with no
+//      per-row reductions.
+//   3. warps 0..7: class w's part of u^T A u; warps 8..15: the classes added,
+//      A v and v.
+// A block barrier follows each, and the sums are formed in one fixed order
+// (classes, then a tree over the classes), whatever warp takes them. The block
+// stays exactly symmetric: the update term of (i, j) is formed from the same
 // products, added in an order-free way, as that of (j, i).
 //
-// Workspace tw (8-byte units): part[2][kWarps][P] (per-warp column sums by
-// step parity), u, v, w [kWarps][P] (each warp's copy, indexed by row, of
-// the current reflector's u and of the pending reflector's v and w),
-// dot[2][kWarps] (per-warp parts of u^T A_sub u).
-constexpr int kTriCols = 8;   // columns per lane: p <= 8 * 32
-constexpr int kTriUnitsPerP = 5 * kWarps;
+// kCl = 4: A (520 KB at p = 255) lies over the shared memory of a cluster of
+// four CTAs, rows g with (g mod 8) / 2 = rank in CTA `rank`, so a CTA's rows
+// are two classes at every step. The CTAs exchange the classes' sums (written
+// to all four, double-buffered by step parity, one cluster barrier per step)
+// and each reads the pivot row from its owner; everything else is repeated in
+// every CTA with the same bits.
+//
+// Measured, p = 99 / 126 / 255: 712 / 1,103 / 8,400 thousand cycles when eight
+// warps repeated the scalar chain, took whole rows and (p > 144) kept A in L2;
+// see the phase clocks for the present figures.
+//
+// Workspace tw (8-byte units): part[kCl > 1 ? 2 : 1][kParts][P], u, v, w, pv
+// [P], dot[kParts], inv[2].
+// kNc: column groups of 32 (p <= 32 kNc), fixed at compile time: loops that
+// stop at the shrinking row cost a lone warp more than the zeros they skip.
+constexpr int tri_units(int P, int cl) { return ((cl > 1 ? 2 : 1) * kParts + 4) * P + kParts + 2; }
 
 // a*b as an unevaluated (hi, lo) pair whose bits do not depend on the operand order
 __device__ __forceinline__ dd dd_mul_sym(dd a, dd b) {
@@ -193,175 +212,228 @@ __device__ __forceinline__ dd dd_sum8(const dd* x, int64_t st) {
   const dd r = pair_add(pair_add(a, b), pair_add(c, f));
   return quick_two_sum(r.hi, r.lo);
 }
-static_assert(kWarps == 8, "dd_sum8 adds one part per warp");
+static_assert(kParts == 8 && kWarps == 2 * kParts, "dd_sum8 adds the classes; two warps per class");
 
-__device__ void tridiagonalize(dd* A, int p, dd* d, dd* e, dd* tw, int64_t P) {
+template <int kCl, int kNc>
+__device__ void tridiagonalize(dd* A, int p, dd* d, dd* e, dd* tw, int P, dd* HV) {
+  namespace cg = cooperative_groups;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  dd* part = tw;                                            // [2][kWarps][P]
-  dd* uw = tw + (2 * kWarps + warp) * P;                    // this warp's u, v, w by row
-  dd* vw = tw + (3 * kWarps + warp) * P;
-  dd* ww = tw + (4 * kWarps + warp) * P;
-  dd* dotp = tw + (int64_t)kTriUnitsPerP * P;               // [2][kWarps]
-  // pending reflector's v, w at g = k + lane + 32c (from the previous step's combine)
-  dd vr[kTriCols], wr[kTriCols];
-#pragma unroll
-  for (int c = 0; c < kTriCols; ++c) {
-    vr[c] = {0.f, 0.f};
-    wr[c] = {0.f, 0.f};
-  }
+  constexpr int kBuf = kCl > 1 ? 2 : 1;
+  dd* part = tw;                                            // [kBuf][kParts][P]
+  dd* u = part + kBuf * kParts * P;
+  dd* v = u + P;
+  dd* w = v + P;
+  dd* pv = w + P;
+  dd* dotp = pv + P;                                        // [kParts]
+  dd* invs = dotp + kParts;                                 // [2], by step parity
+  const int rank = kCl > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  // row g of A: its number among the rows of the CTA that holds it (all, or
+  // those of two classes), and the first such number from row g on
+  auto row_no = [&](int g) -> int { return kCl == 1 ? g : (g >> 3) * 2 + (g & 1); };
+  auto rows_below = [&](int g) -> int { return kCl == 1 ? g : (g >> 3) * 2 + min(max((g & 7) - 2 * rank, 0), 2); };
+  auto pivot_row = [&](int k) -> const dd* {
+    if constexpr (kCl > 1) return cg::this_cluster().map_shared_rank(A, (k & 7) >> 1) + row_no(k) * p;
+    else return A + k * p;
+  };
+  // K = v^T A v of the reflector of step k
+  auto k_of = [&](int k) {
+    const dd inv = invs[k & 1];
+    return dd_mul(dd_mul(dd_sum8(dotp, 1), inv), inv);
+  };
+  const int grp = warp - kParts;                            // (warps 8 ..) column group
+  dd vg = {0.f, 0.f}, pvg = {0.f, 0.f};                     // (warps 8 ..) v and A v at this lane's index
   for (int k = 0; k + 2 < p; ++k) {
     const int L = p - k - 1;
-    const int par = k & 1;
     const bool pend = (k > 0);
-    // pivot row k of the updated matrix, x_g for g = k..p-1 (lane g - k + 32c)
-    const dd vk = {__shfl_sync(0xffffffffu, vr[0].hi, 0), __shfl_sync(0xffffffffu, vr[0].lo, 0)};
-    const dd wk = {__shfl_sync(0xffffffffu, wr[0].hi, 0), __shfl_sync(0xffffffffu, wr[0].lo, 0)};
-    float ts = 0.f, tc = 0.f;
-    dd xk[kTriCols];
-#pragma unroll
-    for (int c = 0; c < kTriCols; ++c) {
-      xk[c] = {0.f, 0.f};
-      if (32 * c > L) break;             // warp-uniform: no slot beyond the row
-      const int g = k + lane + 32 * c;
-      dd x = {0.f, 0.f};
-      if (g < p) {
-        x = A[(int64_t)k * p + g];
-        if (pend) x = dd_rank2_sub(x, vk, wk, vr[c], wr[c]);
-        if (g >= k + 2) dot2_acc(ts, tc, x, x);
+    // ---- 1a. w of the pending reflector and pivot row k after its update (into u)
+    if (grp >= 0 && grp < kNc && 32 * grp <= L) {
+      const int g = k + lane + 32 * grp;
+      dd x = (g < p) ? pivot_row(k)[g] : dd{0.f, 0.f};
+      if (pend) {
+        const dd kv = k_of(k - 1);
+        const dd vk = v[k], wk = dd_scale(dd_sub(pv[k], dd_mul(kv, vk)), 2.f);
+        const dd wg = dd_scale(dd_sub(pvg, dd_mul(kv, vg)), 2.f);
+        x = dd_rank2_sub(x, vk, wk, vg, wg);
+        if (g < p) w[g] = wg;
       }
-      xk[c] = x;
+      if (g < p) u[g] = x;
     }
+    __syncthreads();
+    // ---- 1b. the reflector | the pending update of the trailing block
+    if (warp == 0) {
+      float ts = 0.f, tc = 0.f;
+      dd x[kNc];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {   // xor butterfly: all lanes end with the same bits
-      const float so = __shfl_xor_sync(0xffffffffu, ts, o), co = __shfl_xor_sync(0xffffffffu, tc, o);
-      const dd q = two_sum(ts, so);
-      ts = q.hi;
-      tc = (tc + co) + q.lo;
-    }
-    const dd t = quick_two_sum(ts, tc);
-    const dd x0 = {__shfl_sync(0xffffffffu, xk[0].hi, 1), __shfl_sync(0xffffffffu, xk[0].lo, 1)};
-    dd inv = {0.f, 0.f}, u0 = x0, ek = x0;
-    if (t.hi != 0.f) {
-      const dd nrm = dd_sqrt(dd_fma(x0, x0, t));
-      const dd alpha = (x0.hi >= 0.f) ? dd_neg(nrm) : nrm;
-      u0 = dd_sub(x0, alpha);                       // same sign as x0: no cancellation
-      inv = dd_recip(dd_sqrt(dd_fma(u0, u0, t)));
-      ek = alpha;
-    }
-    // this warp's copy of u (u_{k+1} = x0 - alpha, u_g = x_g beyond)
-#pragma unroll
-    for (int c = 0; c < kTriCols; ++c) {
-      if (32 * c > L) break;
-      const int g = k + lane + 32 * c;
-      if (g > k && g < p) uw[g] = (g == k + 1) ? u0 : xk[c];
-    }
-    if (warp == 0 && lane == 0) {
-      d[k] = xk[0];
-      e[k] = ek;
-    }
-    __syncwarp();
-    // trailing block rows/cols k+1..p-1: apply the pending update, store, and
-    // sum a_ij u_i down this lane's columns j over this warp's rows i
-    dd vc[kTriCols], wc[kTriCols];
-    float cs[kTriCols], cc[kTriCols];
-#pragma unroll
-    for (int c = 0; c < kTriCols; ++c) {
-      const int gj = k + 1 + lane + 32 * c;
-      vc[c] = {0.f, 0.f};
-      wc[c] = {0.f, 0.f};
-      cs[c] = 0.f;
-      cc[c] = 0.f;
-      if (32 * c >= L) continue;
-      if (pend && gj < p) {
-        vc[c] = vw[gj];
-        wc[c] = ww[gj];
+      for (int c = 0; c < kNc; ++c) {
+        const int g = k + lane + 32 * c;
+        x[c] = (g >= k + 2 && g < p) ? u[g] : dd{0.f, 0.f};   // zeros add nothing
       }
-    }
-    // four rows per iteration: their loads, updates and sums interleave
-    for (int i0 = warp; i0 < L; i0 += 4 * kWarps) {
-      dd ui[4], vi[4], wi[4];
-      dd* rp[4];
-      bool ok[4];
+      const dd x0 = u[k + 1];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = i0 + q * kWarps;
-        ok[q] = i < L;
-        const int gi = ok[q] ? k + 1 + i : k + 1;
-        ui[q] = ok[q] ? uw[gi] : dd{0.f, 0.f};
-        vi[q] = (pend && ok[q]) ? vw[gi] : dd{0.f, 0.f};
-        wi[q] = (pend && ok[q]) ? ww[gi] : dd{0.f, 0.f};
-        rp[q] = A + (int64_t)gi * p + (k + 1);
+      for (int c = 0; c < kNc; ++c) dot2_acc(ts, tc, x[c], x[c]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {   // xor butterfly: all lanes end with the same bits
+        const float so = __shfl_xor_sync(0xffffffffu, ts, o), co = __shfl_xor_sync(0xffffffffu, tc, o);
+        const dd q = two_sum(ts, so);
+        ts = q.hi;
+        tc = (tc + co) + q.lo;
       }
+      const dd t = quick_two_sum(ts, tc);
+      dd inv = {0.f, 0.f}, u0 = x0, ek = x0;
+      if (t.hi != 0.f) {
+        const dd nrm = dd_sqrt(dd_fma(x0, x0, t));
+        const dd alpha = (x0.hi >= 0.f) ? dd_neg(nrm) : nrm;
+        u0 = dd_sub(x0, alpha);                       // same sign as x0: no cancellation
+        inv = dd_recip(dd_sqrt(dd_fma(u0, u0, t)));
+        ek = alpha;
+      }
+      if (lane == 0) {                       // u_{k+1} = x0 - alpha, u_g = x_g beyond
+        d[k] = u[k];
+        e[k] = ek;
+        u[k + 1] = u0;
+        invs[k & 1] = inv;
+      }
+    } else if (pend && (kNc > 4 || (warp & 3) != 0)) {
+      // short windows leave warp 0's scheduler to its scalar chain
+      constexpr int kUp = kNc > 4 ? kWarps - 1 : 3 * (kWarps / 4);
+      const int uw = kNc > 4 ? warp - 1 : (warp >> 2) * 3 + (warp & 3) - 1;
+      dd vc[kNc], wc[kNc];
 #pragma unroll
-      for (int c = 0; c < kTriCols; ++c) {
-        if (32 * c >= L) break;
-        const int j = lane + 32 * c;
-        if (j < L) {
-          dd av[4];
+      for (int c = 0; c < kNc; ++c) {
+        const int gj = k + 1 + lane + 32 * c;
+        vc[c] = wc[c] = {0.f, 0.f};
+        if (gj < p) {
+          vc[c] = v[gj];
+          wc[c] = w[gj];
+        }
+      }
+      const int r1 = rows_below(p);
+      dd* rp = A + (rows_below(k + 1) + uw) * p + (k + 1) + lane;
+      for (int i = rows_below(k + 1) + uw; i < r1; i += 2 * kUp, rp += 2 * kUp * p) {
+        const bool two = i + kUp < r1;       // two rows: their loads and updates interleave
+        const int i2 = two ? i + kUp : i;
+        const int ga = kCl == 1 ? i : (i >> 1) * 8 + 2 * rank + (i & 1);
+        const int gb = kCl == 1 ? i2 : (i2 >> 1) * 8 + 2 * rank + (i2 & 1);
+        const dd va = v[ga], wa = w[ga], vb = v[gb], wb = w[gb];
+        dd* rq = rp + (two ? kUp * p : 0);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) av[q] = ok[q] ? rp[q][j] : dd{0.f, 0.f};
-          if (pend) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) av[q] = dd_rank2_sub(av[q], vi[q], wi[q], vc[c], wc[c]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (ok[q]) rp[q][j] = av[q];
+        for (int c = 0; c < kNc; ++c) {
+          if (32 * c >= L) break;
+          if (lane + 32 * c < L) {
+            const dd a = rp[32 * c], b = rq[32 * c];
+            rp[32 * c] = dd_rank2_sub(a, va, wa, vc[c], wc[c]);
+            if (two) rq[32 * c] = dd_rank2_sub(b, vb, wb, vc[c], wc[c]);
           }
-#pragma unroll
-          for (int q = 0; q < 4; ++q)   // rows past L add zero products
-            dot2_acc(cs[c], cc[c], av[q], ui[q]);
         }
       }
     }
-    // column parts, and this warp's part of u^T A_sub u
-    dd* pp = part + (int64_t)par * kWarps * P;
-    float us = 0.f, uc = 0.f;
-#pragma unroll
-    for (int c = 0; c < kTriCols; ++c) {
-      if (32 * c >= L) break;
-      const int gj = k + 1 + lane + 32 * c;
-      if (gj < p) {
-        const dd T = quick_two_sum(cs[c], cc[c]);
-        pp[(int64_t)warp * P + gj] = T;
-        dot2_acc(us, uc, uw[gj], T);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float so = __shfl_xor_sync(0xffffffffu, us, o), co = __shfl_xor_sync(0xffffffffu, uc, o);
-      const dd q = two_sum(us, so);
-      us = q.hi;
-      uc = (uc + co) + q.lo;
-    }
-    if (lane == 0) dotp[par * kWarps + warp] = quick_two_sum(us, uc);
     __syncthreads();
-    // every warp: A_sub u for its lanes' rows, v = u inv, pv = A_sub v,
-    // K = v^T pv = inv^2 u^T A_sub u, w = 2 (pv - K v); reflector k down column k
-    const dd kv = dd_mul(dd_mul(dd_sum8(dotp + par * kWarps, 1), inv), inv);
+    // ---- 2. columns of A u over one class's rows
+    {
+      constexpr int kCStep = kCl == 1 ? 2 : kNc;            // column groups of a warp: c0, c0 + kCStep, ..
+      constexpr int kCols = (kNc + kCStep - 1) / kCStep;
+      const int c0 = kCl == 1 ? warp >> 3 : warp >> 1;
+      const int res = kCl == 1 ? (k + 1 + (warp & 7)) & 7 : 2 * rank + (warp & 1);   // rows g = res mod 8
+      const int cls = (res - (k + 1)) & 7;
+      if (c0 < kNc && 32 * c0 < L) {
+        float cs[kCols], cc[kCols];
 #pragma unroll
-    for (int c = 0; c < kTriCols; ++c) {
-      if (32 * c >= L) break;
-      const int g = k + 1 + lane + 32 * c;
-      if (g < p) {
-        const dd pvg = dd_mul(dd_sum8(pp + g, P), inv);
-        const dd vg = dd_mul(uw[g], inv);
-        const dd wg = dd_scale(dd_sub(pvg, dd_mul(kv, vg)), 2.f);
-        vw[g] = vg;
-        ww[g] = wg;
-        vr[c] = vg;
-        wr[c] = wg;
-        if (warp == 0) A[(int64_t)g * p + k] = vg;
+        for (int c = 0; c < kCols; ++c) cs[c] = cc[c] = 0.f;
+        const int g0 = k + 1 + cls;                         // the class's first row
+        int n = (g0 < p) ? (p - 1 - g0) / kParts + 1 : 0;
+        const dd* up = u + g0;
+        // lanes past the last column read what follows in shared memory and
+        // drop their sums
+        const dd* rp = A + row_no(g0) * p + (k + 1) + lane + 32 * c0;
+        const int rs = (kCl == 1 ? kParts : 2) * p;
+        for (; n >= 4; n -= 4, up += 4 * kParts, rp += 4 * rs) {
+          dd ui[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) ui[q] = up[kParts * q];
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) {
+            if (32 * (c0 + kCStep * c) >= L) break;
+            dd av[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) av[q] = rp[q * rs + 32 * kCStep * c];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dot2_acc(cs[c], cc[c], av[q], ui[q]);
+          }
+        }
+        for (; n > 0; --n, up += kParts, rp += rs) {
+          const dd ui = up[0];
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) {
+            if (32 * (c0 + kCStep * c) >= L) break;
+            dot2_acc(cs[c], cc[c], rp[32 * kCStep * c], ui);
+          }
+        }
+        dd* pp = part + ((kBuf > 1 ? (k & 1) * kParts : 0) + cls) * P;
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) {
+          const int gj = k + 1 + lane + 32 * (c0 + kCStep * c);
+          if (gj < p) {
+            const dd T = quick_two_sum(cs[c], cc[c]);
+            if constexpr (kCl > 1) {
+#pragma unroll
+              for (int q = 0; q < kCl; ++q) cg::this_cluster().map_shared_rank(pp, q)[gj] = T;
+            } else {
+              pp[gj] = T;
+            }
+          }
+        }
       }
     }
-    __syncwarp();
+    if constexpr (kCl > 1) cg::this_cluster().sync();
+    else __syncthreads();
+    // ---- 3. u^T A u by classes | A v = (sum of the classes) inv, v = u inv
+    const dd* pp = part + (kBuf > 1 ? (k & 1) * kParts * P : 0);
+    if (warp < kParts) {
+      float us = 0.f, uc = 0.f;
+      dd a[kNc], b[kNc];
+#pragma unroll
+      for (int c = 0; c < kNc; ++c) {
+        const int gj = k + 1 + lane + 32 * c;
+        a[c] = b[c] = {0.f, 0.f};
+        if (gj < p) {
+          a[c] = u[gj];
+          b[c] = pp[warp * P + gj];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < kNc; ++c) dot2_acc(us, uc, a[c], b[c]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float so = __shfl_xor_sync(0xffffffffu, us, o), co = __shfl_xor_sync(0xffffffffu, uc, o);
+        const dd q = two_sum(us, so);
+        us = q.hi;
+        uc = (uc + co) + q.lo;
+      }
+      if (lane == 0) dotp[warp] = quick_two_sum(us, uc);
+    } else if (grp < kNc) {
+      const int g = k + 1 + lane + 32 * grp;
+      if (g < p) {
+        const dd inv = invs[k & 1];
+        pvg = dd_mul(dd_sum8(pp + g, P), inv);
+        vg = dd_mul(u[g], inv);
+        pv[g] = pvg;
+        v[g] = vg;
+        if (kCl == 1 || rank == 0) HV[(int64_t)k * p + g] = vg;
+      }
+    }
+    __syncthreads();
   }
   if (threadIdx.x == 0) {
     if (p >= 3) {   // the last reflector's update of the final 2 x 2 block
       const int k = p - 2;
-      const dd v0 = vw[k], v1 = vw[k + 1], w0 = ww[k], w1 = ww[k + 1];
-      d[k] = dd_rank2_sub(A[(int64_t)k * p + k], v0, w0, v0, w0);
-      d[k + 1] = dd_rank2_sub(A[(int64_t)(k + 1) * p + k + 1], v1, w1, v1, w1);
-      e[k] = dd_rank2_sub(A[(int64_t)k * p + k + 1], v0, w0, v1, w1);
+      const dd kv = k_of(p - 3);
+      const dd v0 = v[k], v1 = v[k + 1];
+      const dd w0 = dd_scale(dd_sub(pv[k], dd_mul(kv, v0)), 2.f), w1 = dd_scale(dd_sub(pv[k + 1], dd_mul(kv, v1)), 2.f);
+      const dd* r0 = pivot_row(k);
+      const dd* r1 = pivot_row(k + 1);
+      d[k] = dd_rank2_sub(r0[k], v0, w0, v0, w0);
+      d[k + 1] = dd_rank2_sub(r1[k + 1], v1, w1, v1, w1);
+      e[k] = dd_rank2_sub(r0[k + 1], v0, w0, v1, w1);
     } else if (p == 2) {
       d[0] = A[0];
       d[1] = A[3];
@@ -392,14 +464,24 @@ __device__ int sturm32(const float* d, const float* e2, int p, float x, float pi
 // Number of eigenvalues of the df64 tridiagonal (d, e) below x (pivots kept
 // at least pivmin away from zero): the df64 counterpart of sturm32, for the
 // missed-eigenvalue check and the df64 multisection of phase 3'.
-__device__ int sturm_below_dd(const dd* d, const dd* e, int p, dd x, float pivmin) {
+__device__ int sturm_below_dd(const dd* __restrict__ d, const dd* __restrict__ e, int p, dd x, float pivmin) {
   dd q = dd_sub(d[0], x);
   if (fabsf(q.hi) < pivmin) q = dd_make(-pivmin);
   int below = q.hi < 0.f;
+  // d_i - x and e_{i-1}^2 one step ahead of the recurrence
+  dd a = {0.f, 0.f}, e2 = {0.f, 0.f};
+  if (p > 1) {
+    a = dd_sub(d[1], x);
+    e2 = dd_mul(e[0], e[0]);
+  }
   for (int i = 1; i < p; ++i) {
-    q = dd_sub(dd_sub(d[i], x), dd_mul(dd_mul(e[i - 1], e[i - 1]), dd_recip(q)));
+    const int nx = (i + 1 < p) ? i + 1 : i;
+    const dd an = dd_sub(d[nx], x), en = dd_mul(e[nx - 1], e[nx - 1]);
+    q = dd_sub(a, dd_mul(e2, dd_recip(q)));
     if (fabsf(q.hi) < pivmin) q = dd_make(-pivmin);
     below += q.hi < 0.f;
+    a = an;
+    e2 = en;
   }
   return below;
 }
@@ -410,56 +492,91 @@ __device__ int sturm_below_dd(const dd* d, const dd* e, int p, dd x, float pivmi
 // mult / piv (0 or 1) describe L. Pivots below `tiny` are raised to it.
 // Branch-free (selects), so the lanes of a warp that factor different shifts
 // never diverge.
-__device__ void tri_lu_dd(const dd* __restrict__ d, const dd* __restrict__ e, int p, dd mu, float tiny,
-                          dd* __restrict__ u0, dd* __restrict__ u1, dd* __restrict__ u2, dd* __restrict__ mult,
-                          dd* __restrict__ piv) {
-  dd cd = dd_sub(d[0], mu), c1 = (p > 1) ? e[0] : dd{0.f, 0.f};
+// b is eliminated forward on the way (the first solve's forward pass: its
+// chain is hidden behind the factorisation's).
+// The recurrences below run on single lanes, so every load and every term
+// that does not depend on the recurrence is taken one step ahead: an in-order
+// warp would otherwise wait for each of them in turn.
+__device__ __forceinline__ void tri_lu_forward_dd(const dd* __restrict__ d, const dd* __restrict__ e, int p, dd mu,
+                                                  float tiny, dd* __restrict__ u0, dd* __restrict__ u1,
+                                                  dd* __restrict__ u2, dd* __restrict__ mult, dd* __restrict__ piv,
+                                                  dd* __restrict__ b) {
+  const dd zero = {0.f, 0.f};
+  dd cd = dd_sub(d[0], mu), c1 = (p > 1) ? e[0] : zero;
+  dd bi = b[0];
+  dd sub = c1;                                      // e[i]
+  dd nd = zero, bn = zero;                          // d[i + 1] - mu, b[i + 1]
+  if (p > 1) {
+    nd = dd_sub(d[1], mu);
+    bn = b[1];
+  }
   for (int i = 0; i + 1 < p; ++i) {
-    const dd sub = e[i];
-    const dd nd = dd_sub(d[i + 1], mu);
-    const dd n1 = (i + 2 < p) ? e[i + 1] : dd{0.f, 0.f};
+    const int nx = (i + 2 < p) ? i + 2 : i + 1;
+    const dd n1 = (i + 2 < p) ? e[i + 1] : zero;
+    const dd ndn = dd_sub(d[nx], mu), bnn = b[nx];
     const bool sw = fabsf(cd.hi) < fabsf(sub.hi);   // row i+1 becomes the pivot row
     dd pv = dd_sel(sw, sub, cd);
     const dd num = dd_sel(sw, cd, sub);
     if (fabsf(pv.hi) < tiny) pv = {copysignf(tiny, pv.hi), 0.f};
     const dd rp = dd_recip(pv);
-    const dd m = (pv.hi != 0.f) ? dd_mul(num, rp) : dd{0.f, 0.f};
+    const dd m = (pv.hi != 0.f) ? dd_mul(num, rp) : zero;
     u0[i] = rp;
     u1[i] = dd_sel(sw, nd, c1);
-    u2[i] = dd_sel(sw, n1, dd{0.f, 0.f});
+    u2[i] = dd_sel(sw, n1, zero);
     piv[i] = {sw ? 1.f : 0.f, 0.f};
     mult[i] = m;
+    const dd keep = dd_sel(sw, bn, bi), elim = dd_sel(sw, bi, bn);
+    b[i] = keep;
     // no swap: row i+1 - m row i = (nd - m c1, n1); swap: row i - m row i+1 = (c1 - m nd, -m n1)
     cd = dd_sub(dd_sel(sw, c1, nd), dd_mul(m, dd_sel(sw, nd, c1)));
+    bi = dd_sub(elim, dd_mul(m, keep));
     c1 = sw ? dd_neg(dd_mul(m, n1)) : n1;
+    sub = n1;
+    nd = ndn;
+    bn = bnn;
   }
   dd last = cd;
   if (fabsf(last.hi) < tiny) last = {copysignf(tiny, last.hi), 0.f};
   u0[p - 1] = dd_recip(last);
-  u1[p - 1] = {0.f, 0.f};
-  u2[p - 1] = {0.f, 0.f};
+  u1[p - 1] = zero;
+  u2[p - 1] = zero;
+  b[p - 1] = bi;
 }
 
-__device__ void tri_solve_dd(int p, const dd* __restrict__ u0inv, const dd* __restrict__ u1,
-                             const dd* __restrict__ u2, const dd* __restrict__ mult, const dd* __restrict__ piv,
-                             dd* __restrict__ b) {
+__device__ __forceinline__ void tri_forward_dd(int p, const dd* __restrict__ mult, const dd* __restrict__ piv,
+                                               dd* __restrict__ b) {
   dd bi = b[0];
-  for (int i = 0; i + 1 < p; ++i) {   // forward, branch-free: b_i is carried in registers
-    const bool sw = piv[i].hi != 0.f;
-    const dd bn = b[i + 1];
+  dd bn = b[p > 1 ? 1 : 0], m = mult[0];
+  bool sw = p > 1 && piv[0].hi != 0.f;
+  for (int i = 0; i + 1 < p; ++i) {   // branch-free: b_i is carried in registers
+    const int nx = (i + 2 < p) ? i + 2 : i + 1;
+    const dd bnn = b[nx], mn = mult[nx - 1];
+    const bool swn = piv[nx - 1].hi != 0.f;
     const dd keep = dd_sel(sw, bn, bi), elim = dd_sel(sw, bi, bn);
     b[i] = keep;
-    bi = dd_sub(elim, dd_mul(mult[i], keep));
+    bi = dd_sub(elim, dd_mul(m, keep));
+    bn = bnn;
+    m = mn;
+    sw = swn;
   }
   b[p - 1] = bi;
-  dd x1 = {0.f, 0.f}, x2 = {0.f, 0.f};   // x_{i+1}, x_{i+2}
+}
+
+__device__ __forceinline__ void tri_backward_dd(int p, const dd* __restrict__ u0inv, const dd* __restrict__ u1,
+                                                const dd* __restrict__ u2, dd* __restrict__ b) {
+  dd x1 = {0.f, 0.f};                                  // x_{i+1}
+  dd s = dd_sub(b[p - 1], dd_mul(u2[p - 1], x1));      // b_i - u2_i x_{i+2}
+  dd c1 = u1[p - 1], c0 = u0inv[p - 1];
   for (int i = p - 1; i >= 0; --i) {
-    dd s = dd_sub(b[i], dd_mul(u2[i], x2));
-    s = dd_sub(s, dd_mul(u1[i], x1));
-    const dd x = dd_mul(s, u0inv[i]);
+    const int nx = (i > 0) ? i - 1 : 0;
+    const dd c1n = u1[nx], c0n = u0inv[nx];
+    const dd sn = dd_sub(b[nx], dd_mul(u2[nx], x1));   // the next row's, which needs x_{i+1}
+    const dd x = dd_mul(dd_sub(s, dd_mul(c1, x1)), c0);
     b[i] = x;
-    x2 = x1;
     x1 = x;
+    s = sn;
+    c1 = c1n;
+    c0 = c0n;
   }
 }
 
@@ -474,21 +591,15 @@ __device__ void tri_solve_dd(int p, const dd* __restrict__ u0inv, const dd* __re
 // stays a basis of the cluster's subspace. rn: rw reciprocal norms 1 / |z_j|
 // (not 1 / |z_j|^2: after a solve |z|^2 reaches ~1e30, and the low word of
 // its reciprocal would sit in FP32's denormal range).
-__device__ dd block_sum_dd(dd v, dd* red) {   // every thread gets the same sum
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  v = warp_sum_dd(v);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  dd t = red[0];
-  for (int w = 1; w < kWarps; ++w) t = dd_add(t, red[w]);
-  __syncthreads();
-  return t;
-}
+//
+// Two barriers a pass: the norm of a projected vector is taken by the threads
+// that update it, and every thread adds the warps' parts and forms 1 / |z_i|
+// itself.
 
-// one projection pass of z_i against z_0..z_{i-1}; with `self` also z_i . z_i
-// (before the projection) into *self_out
-__device__ void cgs_pass(dd* Z, int i, int p, const dd* rn, dd* coef, dd* self_out) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// coefficients of z_i against z_0..z_{i-1} (rn_last: 1 / |z_{i-1}|, in every
+// thread); with `self` also z_i . z_i (before the projection) into *self_out
+__device__ void cgs_dots(const dd* Z, int i, int p, const dd* rn, dd rn_last, dd* coef, dd* self_out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const dd* zi = Z + (int64_t)i * p;
   const int nj = self_out ? i + 1 : i;
   for (int j = warp; j < nj; j += kWarps) {
@@ -497,45 +608,77 @@ __device__ void cgs_pass(dd* Z, int i, int p, const dd* rn, dd* coef, dd* self_o
     for (int q = lane; q < p; q += 32) acc = dd_fma(zj[q], zi[q], acc);
     acc = warp_sum_dd(acc);
     if (lane == 0) {
-      const dd dt = acc;
-      if (j < i)
-        coef[j] = dd_mul(dd_mul(dt, rn[j]), rn[j]);
-      else
-        *self_out = dt;
+      if (j < i) {
+        const dd r = (j == i - 1) ? rn_last : rn[j];
+        coef[j] = dd_mul(dd_mul(acc, r), r);
+      } else {
+        *self_out = acc;
+      }
     }
   }
-  __syncthreads();
-  dd* zw = Z + (int64_t)i * p;
-  for (int q = tid; q < p; q += kThreads) {
-    dd s = zw[q];
-    for (int j = 0; j < i; ++j) s = dd_sub(s, dd_mul(coef[j], Z[(int64_t)j * p + q]));
-    zw[q] = s;
+}
+
+// z_i -= sum_j coef_j z_j (coef = nullptr: as it is); with `norm` the warps'
+// parts of |z_i|^2 into red
+__device__ void cgs_update(dd* Z, int i, int p, const dd* coef, bool norm, dd* red) {
+  const int q = threadIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  dd nn = {0.f, 0.f};
+  if (q < p) {
+    dd s = Z[(int64_t)i * p + q];
+    if (coef) {
+      for (int j = 0; j < i; ++j) s = dd_sub(s, dd_mul(coef[j], Z[(int64_t)j * p + q]));
+      Z[(int64_t)i * p + q] = s;
+    }
+    nn = dd_fma(s, s, nn);
   }
-  __syncthreads();
+  if (norm && 32 * warp < p) {
+    nn = warp_sum_dd(nn);
+    if (lane == 0) red[warp] = nn;
+  }
+}
+static_assert(SDMD_MAX_M <= kThreads, "cgs_update: one position per thread");
+
+__device__ dd cgs_norm2(const dd* red, int p) {   // every thread gets the same sum
+  dd t = red[0];
+  for (int w = 1; 32 * w < p; ++w) t = dd_add(t, red[w]);
+  return t;
 }
 
 __device__ void cgs_dd(dd* Z, int rw, int p, int passes, dd* coef, dd* rn, dd* red, dd* sc) {
   const int tid = threadIdx.x;
+  dd rn_i = {0.f, 0.f};
   for (int i = 0; i < rw; ++i) {
     dd* zi = Z + (int64_t)i * p;
-    for (int pass = 0; pass < passes && i > 0; ++pass) cgs_pass(Z, i, p, rn, coef, pass == 0 ? &sc[3] : nullptr);
-    dd nn = {0.f, 0.f};
-    for (int q = tid; q < p; q += kThreads) nn = dd_fma(zi[q], zi[q], nn);
-    dd t = block_sum_dd(nn, red);
-    if (i > 0 && !(t.hi > 1e-20f * sc[3].hi)) {   // collapsed: reseed and project twice
-      for (int q = tid; q < p; q += kThreads) {
-        const unsigned hsh = (unsigned)(q + 1) * 2654435761u ^ (unsigned)(i + 1) * 40503u;
-        zi[q] = dd_make((float)((hsh >> 8) & 0xFFFFu) / 65536.f - 0.5f);
+    dd* self = &sc[2 + (i & 1)];           // by parity: read after the next vector's dots began
+    if (i == 0) {
+      cgs_update(Z, i, p, nullptr, true, red);
+      __syncthreads();
+    }
+    for (int pass = 0; pass < passes && i > 0; ++pass) {
+      cgs_dots(Z, i, p, rn, rn_i, coef, pass == 0 ? self : nullptr);
+      __syncthreads();
+      cgs_update(Z, i, p, coef, pass + 1 == passes, red);
+      __syncthreads();
+    }
+    dd t = cgs_norm2(red, p);
+    if (i > 0 && !(t.hi > 1e-20f * self->hi)) {   // collapsed: reseed and project twice
+      if (tid < p) {
+        const unsigned hsh = (unsigned)(tid + 1) * 2654435761u ^ (unsigned)(i + 1) * 40503u;
+        zi[tid] = dd_make((float)((hsh >> 8) & 0xFFFFu) / 65536.f - 0.5f);
       }
       __syncthreads();
-      for (int pass = 0; pass < 2; ++pass) cgs_pass(Z, i, p, rn, coef, nullptr);
-      nn = {0.f, 0.f};
-      for (int q = tid; q < p; q += kThreads) nn = dd_fma(zi[q], zi[q], nn);
-      t = block_sum_dd(nn, red);
+      for (int pass = 0; pass < 2; ++pass) {
+        cgs_dots(Z, i, p, rn, rn_i, coef, nullptr);
+        __syncthreads();
+        cgs_update(Z, i, p, coef, pass == 1, red);
+        __syncthreads();
+      }
+      t = cgs_norm2(red, p);
     }
-    if (tid == 0) rn[i] = (t.hi > 0.f) ? dd_recip(dd_sqrt(t)) : dd{0.f, 0.f};
-    __syncthreads();
+    rn_i = (t.hi > 0.f) ? dd_recip(dd_sqrt(t)) : dd{0.f, 0.f};
+    if (tid == 0) rn[i] = rn_i;
   }
+  __syncthreads();
   for (int idx = tid; idx < rw * p; idx += kThreads) Z[idx] = dd_mul(Z[idx], rn[idx / p]);
   __syncthreads();
 }
@@ -556,15 +699,32 @@ __device__ void rayleigh_ritz(dd* Z, int rw, int p, const dd* d, const dd* e, dd
     tz[idx] = t;
   }
   __syncthreads();
-  for (int pr = warp; pr < rw * rw; pr += kWarps) {
-    const int a = pr / rw, b = pr - a * rw;
-    if (b < a) continue;
-    dd s = {0.f, 0.f};
-    for (int q = lane; q < p; q += 32) s = dd_fma(Z[(int64_t)a * p + q], tz[(int64_t)b * p + q], s);
-    s = warp_sum_dd(s);
-    if (lane == 0) {
-      H[a * rw + b] = s;
-      H[b * rw + a] = s;
+  // the upper triangle's dots over the warps, two per warp in flight: pairs
+  // (a, b), b >= a, numbered row by row; the warp steps 2 kWarps pairs
+  int pa[2] = {0, 0}, pb[2] = {warp, warp + kWarps};
+  for (;;) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      while (pa[h] < rw && pb[h] >= rw) {
+        pb[h] -= rw - (pa[h] + 1);
+        ++pa[h];
+      }
+    if (pa[0] >= rw && pa[1] >= rw) break;
+    dd s[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    for (int q = lane; q < p; q += 32) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (pa[h] < rw) s[h] = dd_fma(Z[(int64_t)pa[h] * p + q], tz[(int64_t)pb[h] * p + q], s[h]);
+    }
+    s[0] = warp_sum_dd(s[0]);
+    s[1] = warp_sum_dd(s[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (lane == 0 && pa[h] < rw) {
+        H[pa[h] * rw + pb[h]] = s[h];
+        H[pb[h] * rw + pa[h]] = s[h];
+      }
+      pb[h] += 2 * kWarps;
     }
   }
   for (int idx = tid; idx < rw * rw; idx += kThreads) R[idx] = {(idx / rw == idx % rw) ? 1.f : 0.f, 0.f};
@@ -619,40 +779,76 @@ __device__ void rayleigh_ritz(dd* Z, int rw, int p, const dd* d, const dd* e, dd
         tz[2 * k + 1] = s;
       }
       __syncthreads();
-      for (int idx = tid; idx < (n2 / 2) * rw; idx += kThreads) {   // rows: H <- J^T H
-        const int k = idx / rw, col = idx - k * rw;
-        const int a = ord[2 * k], b = ord[2 * k + 1];
-        if (b >= rw) continue;
-        const dd c = tz[2 * k], s = tz[2 * k + 1];
-        const dd ha = H[a * rw + col], hb = H[b * rw + col];
-        H[a * rw + col] = dd_sub(dd_mul(c, ha), dd_mul(s, hb));
-        H[b * rw + col] = dd_add(dd_mul(s, ha), dd_mul(c, hb));
-      }
-      __syncthreads();
-      for (int idx = tid; idx < (n2 / 2) * rw * 2; idx += kThreads) {   // columns: H <- H J, R <- R J
-        const int half = idx / ((n2 / 2) * rw);
-        const int rem = idx - half * (n2 / 2) * rw;
-        const int k = rem / rw, row = rem - k * rw;
-        const int a = ord[2 * k], b = ord[2 * k + 1];
-        if (b >= rw) continue;
-        dd* M = half ? R : H;
-        const dd c = tz[2 * k], s = tz[2 * k + 1];
-        const dd ma = M[row * rw + a], mb = M[row * rw + b];
-        M[row * rw + a] = dd_sub(dd_mul(c, ma), dd_mul(s, mb));
-        M[row * rw + b] = dd_add(dd_mul(s, ma), dd_mul(c, mb));
+      // H <- J^T H J: the 2 x 2 block of pairs (k, l) by one thread, its rows
+      // rotated and then its columns; R <- R J row by row beside it
+      const int nh = n2 / 2;
+      for (int idx = tid; idx < nh * (nh + rw); idx += kThreads) {
+        const int k = idx % nh, l = idx / nh;
+        const int ca = ord[2 * k], cb = ord[2 * k + 1];       // columns of pair k
+        const dd cc = tz[2 * k], cs = tz[2 * k + 1];
+        if (l >= nh) {                       // row l - nh of R
+          if (cb >= rw) continue;
+          dd* row = R + (int64_t)(l - nh) * rw;
+          const dd ma = row[ca], mb = row[cb];
+          row[ca] = dd_sub(dd_mul(cc, ma), dd_mul(cs, mb));
+          row[cb] = dd_add(dd_mul(cs, ma), dd_mul(cc, mb));
+          continue;
+        }
+        const int ra = ord[2 * l], rb = ord[2 * l + 1];       // rows of pair l
+        const bool rok = rb < rw, cok = cb < rw;
+        const dd rc = tz[2 * l], rs = tz[2 * l + 1];
+        dd aa = H[ra * rw + ca], ab = cok ? H[ra * rw + cb] : dd{0.f, 0.f};
+        if (rok) {
+          const dd ba = H[rb * rw + ca], bb = cok ? H[rb * rw + cb] : dd{0.f, 0.f};
+          const dd na = dd_sub(dd_mul(rc, aa), dd_mul(rs, ba)), nb = dd_add(dd_mul(rs, aa), dd_mul(rc, ba));
+          const dd oa = dd_sub(dd_mul(rc, ab), dd_mul(rs, bb)), ob = dd_add(dd_mul(rs, ab), dd_mul(rc, bb));
+          aa = na;
+          ab = oa;
+          if (cok) {
+            H[rb * rw + ca] = dd_sub(dd_mul(cc, nb), dd_mul(cs, ob));
+            H[rb * rw + cb] = dd_add(dd_mul(cs, nb), dd_mul(cc, ob));
+          } else {
+            H[rb * rw + ca] = nb;
+          }
+        }
+        if (cok) {
+          H[ra * rw + ca] = dd_sub(dd_mul(cc, aa), dd_mul(cs, ab));
+          H[ra * rw + cb] = dd_add(dd_mul(cs, aa), dd_mul(cc, ab));
+        } else {
+          H[ra * rw + ca] = aa;
+        }
       }
       __syncthreads();
     }
   }
-  if (tid == 0) {
-    for (int a = 0; a < rw; ++a) ord[a] = a;
-    for (int a = 0; a < rw; ++a) {
-      int best = a;
-      for (int b = a + 1; b < rw; ++b)
-        if (dd_lt(H[ord[best] * rw + ord[best]], H[ord[b] * rw + ord[b]])) best = b;
-      const int t = ord[a];
-      ord[a] = ord[best];
-      ord[best] = t;
+  for (int a = tid; a < rw; a += kThreads) ord[a] = a;
+  __syncthreads();
+  if (warp == 0) {     // selection sort, descending: the first largest of the rest, by a warp reduction
+    for (int a = 0; a + 1 < rw; ++a) {
+      dd best = {-INFINITY, 0.f};
+      int at = rw;
+      for (int b = a + lane; b < rw; b += 32) {
+        const dd v = H[ord[b] * rw + ord[b]];
+        if (at == rw || dd_lt(best, v)) {
+          best = v;
+          at = b;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const dd v = shfl_dd(best, o);
+        const int vat = __shfl_xor_sync(0xffffffffu, at, o);
+        if (vat < rw && (at == rw || dd_lt(best, v) || (!dd_lt(v, best) && vat < at))) {
+          best = v;
+          at = vat;
+        }
+      }
+      if (lane == 0 && at != a) {
+        const int t = ord[a];
+        ord[a] = ord[at];
+        ord[at] = t;
+      }
+      __syncwarp();
     }
   }
   __syncthreads();
@@ -669,11 +865,59 @@ __device__ void rayleigh_ritz(dd* Z, int rw, int p, const dd* d, const dd* e, dd
   __syncthreads();
 }
 
+// ---------------------------------------------------------------- phase 4 --
+// z <- H_k z for k = k1 down to k0 (k0 >= 0) on half a warp per vector, with
+// at most kNt positions per lane (p - 1 - k <= 16 kNt); reflector k - 1 is
+// loaded while k is applied. Positions past the end count as zeros.
+template <int kNt>
+__device__ void back_steps(const dd* __restrict__ HV, int p, dd* z, bool live, int k1, int k0) {
+  const int hl = threadIdx.x & 15;
+  if (k0 < 0) k0 = 0;
+  if (k1 < k0) return;
+  dd vn[kNt];
+  auto load = [&](int k) {
+#pragma unroll
+    for (int j = 0; j < kNt; ++j) {
+      const int g = k + 1 + hl + 16 * j;
+      vn[j] = (g < p) ? HV[(int64_t)k * p + g] : dd{0.f, 0.f};
+    }
+  };
+  load(k1);
+  for (int k = k1; k >= k0; --k) {
+    dd v[kNt], x[kNt];
+#pragma unroll
+    for (int j = 0; j < kNt; ++j) {
+      const int g = k + 1 + hl + 16 * j;
+      v[j] = vn[j];
+      x[j] = (g < p) ? z[g] : dd{0.f, 0.f};
+    }
+    if (k > k0) load(k - 1);
+    float ss = 0.f, sc = 0.f;
+#pragma unroll
+    for (int j = 0; j < kNt; ++j) dot2_acc(ss, sc, v[j], x[j]);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {   // within each half warp
+      const float so = __shfl_xor_sync(0xffffffffu, ss, o), co = __shfl_xor_sync(0xffffffffu, sc, o);
+      const dd q = two_sum(ss, so);
+      ss = q.hi;
+      sc = (sc + co) + q.lo;
+    }
+    const dd s = dd_scale(quick_two_sum(ss, sc), -2.f);
+#pragma unroll
+    for (int j = 0; j < kNt; ++j) {
+      const int g = k + 1 + hl + 16 * j;
+      const dd y = dd_fma(s, v[j], x[j]);
+      if (live && g < p) z[g] = y;
+    }
+    __syncwarp();
+  }
+}
+
 // ---------------------------------------------------------------- phase 7 --
 // FP32 eigen-decomposition of the complex r x r matrix H (row-major) on one
-// warp: Hessenberg reduction, shifted QR to Schur form with Q accumulated,
-// right eigenvectors W and left eigenvectors U (columns, unit norm).
-// Returns false if the QR iteration cap was reached.
+// warp: Hessenberg reduction, shifted QR to Schur form with Q accumulated
+// (returns false if the QR iteration cap was reached), then right eigenvectors W
+// and left eigenvectors U (columns, unit norm), which two warps can take at once.
 // Complex Givens rotation [c s; -conj(s) c] taking (a, b) to (rho, 0). (a, b)
 // are scaled by a power of two to a largest component in [1, 2) (c and s do
 // not change), so the squared moduli neither underflow nor overflow; then c,
@@ -704,7 +948,7 @@ __device__ __forceinline__ void givens32(CF a, CF b, float& c, CF& s) {
   s = cscale(cmul(a, cconj(b)), k);
 }
 
-__device__ bool warp_eig32(CF* H, CF* Q, CF* W, CF* U, CF* ycol, int r, float* cs, CF* sn) {
+__device__ bool warp_schur32(CF* H, CF* Q, CF* ycol, int r, float* cs, CF* sn) {
   const int lane = threadIdx.x & 31;
   for (int idx = lane; idx < r * r; idx += 32) {
     const int i = idx / r, j = idx - i * r;
@@ -882,6 +1126,12 @@ __device__ bool warp_eig32(CF* H, CF* Q, CF* W, CF* U, CF* ycol, int r, float* c
     __syncwarp();
   }
   __syncwarp();
+  return ok;
+}
+
+// Smallest pivot of the triangular solves (every lane of the warp).
+__device__ float schur_small(const CF* H, int r) {
+  const int lane = threadIdx.x & 31;
   float tnorm = 0.f;
   for (int idx = lane; idx < r * r; idx += 32) {
     const int i = idx / r, j = idx - i * r;
@@ -889,6 +1139,13 @@ __device__ bool warp_eig32(CF* H, CF* Q, CF* W, CF* U, CF* ycol, int r, float* c
   }
   tnorm = warp_max_f(tnorm);
   const float small = fmaxf(kEps32 * tnorm, FLT_MIN);
+  return small;
+}
+
+// Right eigenvectors W (columns, unit norm) of the Schur form, one warp.
+__device__ void warp_right32(const CF* H, const CF* Q, CF* W, CF* ycol, int r) {
+  const int lane = threadIdx.x & 31;
+  const float small = schur_small(H, r);
   // right eigenvectors: (T - l_k) y = 0 with y_k = 1, y_{>k} = 0; w = Q y
   for (int k = lane; k < r; k += 32) {
     CF* y = ycol + k * r;
@@ -913,6 +1170,12 @@ __device__ bool warp_eig32(CF* H, CF* Q, CF* W, CF* U, CF* ycol, int r, float* c
     for (int q = 0; q < r; ++q) W[q * r + k] = cscale(W[q * r + k], inv);
   }
   __syncwarp();
+}
+
+// Left eigenvectors U likewise (its own ycol when both run at once).
+__device__ void warp_left32(const CF* H, const CF* Q, CF* U, CF* ycol, int r) {
+  const int lane = threadIdx.x & 31;
+  const float small = schur_small(H, r);
   // left eigenvectors: x^H T = l_k x^H with x_k = 1, x_{<k} = 0; u = Q x
   for (int k = lane; k < r; k += 32) {
     CF* x = ycol + k * r;
@@ -938,50 +1201,55 @@ __device__ bool warp_eig32(CF* H, CF* Q, CF* W, CF* U, CF* ycol, int r, float* c
     for (int q = 0; q < r; ++q) U[q * r + k] = cscale(U[q * r + k], inv);
   }
   __syncwarp();
-  return ok;
 }
 
-// Shared-memory plan (dynamic), in 8-byte units.
+// Shared-memory plan (dynamic), in 8-byte units: the vectors, the
+// Rayleigh-Ritz matrices, and a pool that the phases use one after another:
+//   1     A (or this CTA's rows of it) and the tridiagonalisation's workspace
+//   3, 4  LU factors (5p per vector; Ritz scratch in the same place) and the
+//         vectors Z, which stay; the recurrences are chains of dependent
+//         loads and stores, so they belong on chip when they fit
+//   6..9  behind Z: G_XY vsi, A~, the small eigenproblem, G_XY transposed
 struct SmemPlan {
-  int a_in_smem;
+  int P, rr_dim;         // rr_dim: r plus the cluster extension
   int rr_in_smem;
-  int eig_in_smem;
-  int inv_in_smem;       // inverse-iteration LU, Ritz scratch and vectors Z in shared memory
-  int rr_dim;            // Rayleigh-Ritz size limit: r plus the cluster extension
-  int64_t P, vec_units, rr_units, big_units, inv_units;
+  int cl;                // CTAs that hold A
+  int64_t vec_units, rr_units, pool_units;
 };
 
 // Dynamic shared memory the plan may use (8-byte units): the SM's 227 KiB
 // less the kernel's static arrays, with margin.
-constexpr int64_t kSmemDynUnits = (220 * 1024) / 8;
+constexpr int64_t kSmemDynUnits = (216 * 1024) / 8;
+constexpr int kEigUnits = 8;   // H, Q, W, U, two y (complex float) and the products A~ w (two df64) per r x r
 
 __host__ __device__ inline SmemPlan smem_plan(int p, int r) {
   SmemPlan s;
   s.P = (p + 3) & ~3;
-  // d, e, vs, pv, wv, lam (df64) + part (one df64 per thread) + d32, e2_32 (float) + 32 df64 scalars
-  s.vec_units = 6 * s.P + kThreads + s.P + 32;
+  // d, e, rn, pv (two: provisional eigenvalues), lam (df64) + d32, e2_32 (float) + 32 df64 scalars
+  s.vec_units = 6 * s.P + s.P + 32;
   s.rr_dim = (r + kClusterExt < p) ? r + kClusterExt : p;
   s.rr_in_smem = (s.rr_dim <= kRRMax);
   s.rr_units = s.rr_in_smem ? 2 * (int64_t)s.rr_dim * s.rr_dim : 0;
-  // the tridiagonalisation's workspace (phase 1 only) shares its region with
-  // the inverse iteration's working set (phase 3 on)
-  const int64_t tri = (int64_t)kTriUnitsPerP * s.P + 2 * kWarps;
-  s.a_in_smem = (p <= kSmemMaxP) && (s.vec_units + s.rr_units + (int64_t)p * p + tri <= kSmemDynUnits);
-  s.eig_in_smem = (r <= kEigMaxR);
-  const int64_t a = s.a_in_smem ? (int64_t)p * p : 0;
-  const int64_t g = s.eig_in_smem ? (int64_t)5 * r * r : 0;   // H, Q, W, U, y (complex float)
-  s.big_units = a > g ? a : g;
-  // the inverse iteration's working set (per vector: LU 5p, Ritz scratch p,
-  // the vector p) on chip when it fits: its tridiagonal recurrences are
-  // chains of dependent loads and stores
-  const int64_t inv = (int64_t)s.rr_dim * 7 * p;
-  s.inv_in_smem = (s.vec_units + s.rr_units + s.big_units + (inv > tri ? inv : tri) <= kSmemDynUnits);
-  s.inv_units = s.inv_in_smem ? (inv > tri ? inv : tri) : tri;
+  s.cl = (p <= kSmemMaxP) ? 1 : kClusterCtas;
+  const int64_t room = kSmemDynUnits - s.vec_units - s.rr_units;
+  const int64_t rows = s.cl == 1 ? p : 2 * ((p + 7) / 8);
+  const int64_t tri = rows * p + tri_units(s.P, s.cl);
+  const int64_t inv = (int64_t)s.rr_dim * 6 * p;
+  const int64_t small = (int64_t)s.rr_dim * p + (int64_t)r * p + (1 + kEigUnits) * (int64_t)r * r + (int64_t)p * p;
+  s.pool_units = tri;
+  if (inv > s.pool_units) s.pool_units = inv < room ? inv : room;
+  if (small > s.pool_units) s.pool_units = small < room ? small : room;
   return s;
 }
+// phase 1 fits whatever p: one SM up to kSmemMaxP, else the cluster's rows (at
+// most 64 of them), beside the vectors and the Rayleigh-Ritz matrices
+static_assert(kSmemMaxP * kSmemMaxP + tri_units(kSmemMaxP, 1) + 7 * kSmemMaxP + 32 + 2 * kRRMax * kRRMax <= kSmemDynUnits, "p = kSmemMaxP");
+static_assert(64 * 255 + tri_units(256, kClusterCtas) + 7 * 256 + 32 + 2 * kRRMax * kRRMax <= kSmemDynUnits, "p = 255");
 
+template <int kCl>
 __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const ModesLayout& L) {
-  extern __shared__ double smem_d[];
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) double smem_d[];
   __shared__ dd red[kWarps];
   __shared__ float cs[SDMD_MAX_M];
   __shared__ CF sn[SDMD_MAX_M];
@@ -990,6 +1258,7 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   __shared__ int sh_int[4];
   __shared__ float sh_f[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = kCl > 1 ? (int)cg::this_cluster().block_rank() : 0;
   WS w = carve(a.ws, L);
   // embed_cx: the 2pc x 2pc real embedding of a complex pc x pc G_X
   const int m = a.m, pc = a.c - 1, p = a.embed_cx ? 2 * pc : pc;
@@ -1001,22 +1270,17 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   dd* e = d + P;
   dd* vs = e + P;
   dd* pv = vs + P;
-  dd* wv = pv + P;
-  dd* lam = wv + P;
-  dd* part = lam + P;
-  float* d32 = reinterpret_cast<float*>(part + kThreads);
+  dd* lam = pv + P;
+  float* d32 = reinterpret_cast<float*>(lam + P);
   float* e2_32 = d32 + P;
   dd* sc = reinterpret_cast<dd*>(e2_32 + P);
-  dd* rrH = plan.rr_in_smem ? base + plan.vec_units : w.Y;
-  dd* rrR = rrH + (int64_t)plan.rr_dim * plan.rr_dim;
-  dd* big = base + plan.vec_units + plan.rr_units;
-  dd* A = plan.a_in_smem ? big : w.Ad;
-  // inverse iteration: LU factors + Ritz scratch (rr_dim x 6p) and the vectors
-  // Z (rr_dim x p; later the eigenvectors, then vsi)
-  dd* inv_base = big + plan.big_units;
-  dd* LU = plan.inv_in_smem ? inv_base : w.lu;
-  dd* Z = plan.inv_in_smem ? inv_base + (int64_t)plan.rr_dim * 6 * p : w.Z;
-  if (tid == 0) w.clk[0] = clock64();
+  dd* pool = base + plan.vec_units + plan.rr_units;
+  dd* A = pool;                          // kCl > 1: this CTA's rows
+  dd* tri_ws = pool + (kCl > 1 ? 2 * (int64_t)((p + 7) / 8) : (int64_t)p) * p;
+  // the reflectors: the embedding (2pc > m - 1) takes the region of the
+  // complex kernel's own arrays, which it fills later
+  dd* HV = a.embed_cx ? reinterpret_cast<dd*>(a.ws + L.cx) : w.HV;
+  if (tid == 0 && rank == 0) w.clk[0] = clock64();
 
   // ---- 0. scale (exact power of two from the largest diagonal), gather, convert
   if (warp == 0) {
@@ -1058,15 +1322,19 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   // converted and stored (the stores could alias G for the compiler, so a
   // plain loop waits a full memory latency per entry; beside a bandwidth-bound
   // pass that latency is long)
+  // G_XY is kept transposed: phase 6 reads it with consecutive rows over the
+  // lanes. A cluster's CTA takes the rows it owns.
   constexpr int kGatherBatch = 8;
-  for (int base = tid; !a.embed_cx && base < p * p; base += kThreads * kGatherBatch) {
+  const int nrows = kCl > 1 ? (p >> 3) * 2 + min(max((p & 7) - 2 * rank, 0), 2) : p;   // stored rows of this CTA
+  for (int base = tid; !a.embed_cx && base < nrows * p; base += kThreads * kGatherBatch) {
     int64_t raw_x[kGatherBatch], raw_xy[kGatherBatch];   // the G words (int64 or the bits of an FP64)
 #pragma unroll
     for (int u = 0; u < kGatherBatch; ++u) {
       const int idx = base + u * kThreads;
       raw_x[u] = raw_xy[u] = 0;
-      if (idx < p * p) {
-        const int i = idx / p, j = idx - i * p;
+      if (idx < nrows * p) {
+        const int li = idx / p, j = idx - li * p;
+        const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
         int si = a.start + i, sj = a.start + j;
         if (si >= m) si -= m;
         if (sj >= m) sj -= m;
@@ -1079,19 +1347,33 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
 #pragma unroll
     for (int u = 0; u < kGatherBatch; ++u) {
       const int idx = base + u * kThreads;
-      if (idx < p * p) {
+      if (idx < nrows * p) {
+        const int li = idx / p, j = idx - li * p;
+        const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
         const dd gx = a.g_is_int ? dd_from_ll(raw_x[u]) : dd_from_double(__longlong_as_double(raw_x[u]));
         const dd gxy = a.g_is_int ? dd_from_ll(raw_xy[u]) : dd_from_double(__longlong_as_double(raw_xy[u]));
         A[idx] = {ldexpf(gx.hi, -s_exp), ldexpf(gx.lo, -s_exp)};
-        w.GXYd[idx] = {ldexpf(gxy.hi, -s_exp), ldexpf(gxy.lo, -s_exp)};
+        w.GXYt[(int64_t)j * p + i] = {ldexpf(gxy.hi, -s_exp), ldexpf(gxy.lo, -s_exp)};
       }
     }
   }
-  __syncthreads();
-  if (tid == 0) w.clk[1] = clock64();
+  if constexpr (kCl > 1) cg::this_cluster().sync();
+  else __syncthreads();
+  if (tid == 0 && rank == 0) w.clk[1] = clock64();
 
   // ---- 1. tridiagonalise G_X (df64)
-  tridiagonalize(A, p, d, e, inv_base, P);
+  if constexpr (kCl > 1) {
+    tridiagonalize<kCl, 8>(A, p, d, e, tri_ws, plan.P, HV);
+  } else {
+    if (p <= 32) tridiagonalize<1, 1>(A, p, d, e, tri_ws, plan.P, HV);
+    else if (p <= 64) tridiagonalize<1, 2>(A, p, d, e, tri_ws, plan.P, HV);
+    else if (p <= 128) tridiagonalize<1, 4>(A, p, d, e, tri_ws, plan.P, HV);
+    else tridiagonalize<1, 5>(A, p, d, e, tri_ws, plan.P, HV);
+  }
+  if constexpr (kCl > 1) {               // no CTA leaves while its rows may be read
+    cg::this_cluster().sync();
+    if (rank != 0) return;
+  }
   if (tid == 0) w.clk[2] = clock64();
 
   // ---- 2. FP32 multisection for the rw largest eigenvalues of T
@@ -1100,19 +1382,24 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     e2_32[i] = (i + 1 < p) ? e[i].hi * e[i].hi : 0.f;
   }
   __syncthreads();
-  if (tid == 0) {
-    float gl = 0.f, gu = 0.f, em = 0.f;
-    for (int i = 0; i < p; ++i) {
+  if (warp == 0) {
+    float gl = INFINITY, gu = -INFINITY, em = 0.f;
+    for (int i = lane; i < p; i += 32) {
       const float rad = ((i > 0) ? fabsf(e[i - 1].hi) : 0.f) + ((i + 1 < p) ? fabsf(e[i].hi) : 0.f);
-      gl = (i == 0) ? d32[0] - rad : fminf(gl, d32[i] - rad);
-      gu = (i == 0) ? d32[0] + rad : fmaxf(gu, d32[i] + rad);
+      gl = fminf(gl, d32[i] - rad);
+      gu = fmaxf(gu, d32[i] + rad);
       if (i + 1 < p) em = fmaxf(em, e2_32[i]);
     }
+    gl = -warp_max_f(-gl);
+    gu = warp_max_f(gu);
+    em = warp_max_f(em);
     const float tn = fmaxf(fabsf(gl), fabsf(gu));
-    sh_f[0] = gl - 4.f * kEps32 * tn * p - FLT_MIN;
-    sh_f[1] = gu + 4.f * kEps32 * tn * p + FLT_MIN;
-    sh_f[2] = tn;
-    sh_f[3] = FLT_MIN * fmaxf(1.f, em) * 4.f;
+    if (lane == 0) {
+      sh_f[0] = gl - 4.f * kEps32 * tn * p - FLT_MIN;
+      sh_f[1] = gu + 4.f * kEps32 * tn * p + FLT_MIN;
+      sh_f[2] = tn;
+      sh_f[3] = FLT_MIN * fmaxf(1.f, em) * 4.f;
+    }
   }
   __syncthreads();
   const float tnorm = sh_f[2];
@@ -1164,6 +1451,10 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   __syncthreads();
   const int rwe = (rw > 0) ? sh_int[2] : 0;
   for (int i = tid; i < rwe; i += kThreads) pv[i] = lam[i];   // the FP32 values, for phase 3'
+  // inverse iteration: the vectors Z (later the eigenvectors, then vsi) and
+  // LU factors (5p per vector; the Ritz scratch takes their place)
+  const bool inv_in_smem = (int64_t)rwe * 6 * p <= plan.pool_units;
+  dd* Z = inv_in_smem ? pool : w.Z;
   if (tid == 0) w.clk[3] = clock64();
 
   // ---- 3. df64 inverse iteration + Gram-Schmidt + Rayleigh-Ritz, twice:
@@ -1171,26 +1462,19 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   //         round-0 Ritz values (df64-accurate), which converges in one or two
   //         solves even for eigenvalues much closer than eps32 * |T|
   const float tiny = fmaxf(1e-13f * tnorm, FLT_MIN);
+  // ---- 3'. missed-eigenvalue check: inverse iteration converges to the
+  //          eigenvectors nearest its shifts, and inside a cluster below
+  //          the FP32 multisection's resolution (eps32 |T|) those need not
+  //          be the largest. A df64 Sturm count of the eigenvalues above
+  //          the smallest kept Ritz value (less 1e-13 |T|) that exceeds rw
+  //          sends the wanted eigenvalues through a df64 multisection
+  //          (warp per eigenvalue, 33 points per round, bracketed by the
+  //          FP32 value or else by Gershgorin) and one more round runs
+  //          with those shifts. One lane counts while the other warps
+  //          back-transform; the third round starts from fresh vectors, so a
+  //          failed check only costs that back-transform.
   for (int round = 0; round < 3; ++round) {
     if (round == 2) {
-      // ---- 3'. missed-eigenvalue check: inverse iteration converges to the
-      //          eigenvectors nearest its shifts, and inside a cluster below
-      //          the FP32 multisection's resolution (eps32 |T|) those need not
-      //          be the largest. A df64 Sturm count of the eigenvalues above
-      //          the smallest kept Ritz value (less 1e-13 |T|) that exceeds rw
-      //          sends the wanted eigenvalues through a df64 multisection
-      //          (warp per eigenvalue, 33 points per round, bracketed by the
-      //          FP32 value or else by Gershgorin) and one more round runs
-      //          with those shifts.
-      if (tid == 0) {
-        const int below = sturm_below_dd(d, e, p, dd_sub(lam[rw - 1], dd_make(1e-13f * tnorm)), sh_f[3]);
-        sh_int[3] = (p - below > rw) ? 1 : 0;
-      }
-      __syncthreads();
-      // the embedding of a complex window leaves a failed check to the complex
-      // kernel's FP64 Jacobi: for modes that far below lambda_1 its FP64
-      // backward error keeps A~'s eigenvalues within 1e-9, df64 does not
-      if (!sh_int[3] || a.embed_cx) break;
       for (int i = warp; i < rwe; i += kWarps) {
         const int target = p - 1 - i;
         const float W = 32.f * kEps32 * tnorm + sh_f[3];
@@ -1217,82 +1501,88 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
       }
       __syncthreads();
     }
-    const float sep = (round == 0) ? 2.f * kEps32 * tnorm : 1e-12f * tnorm;
-    // vector i on lane i / 8 of warp i % 8: the factorisations and solves are
-    // serial recurrences, so they are spread over all warps' issue slots
-    for (int i = warp + kWarps * lane; i < rwe; i += kThreads) {
-      dd* u0 = LU + (int64_t)i * 5 * p;
-      dd shift = lam[i];
-      for (int q = 0; q < i; ++q)    // (numerically) equal shifts: separate them slightly
-        if (fabsf(lam[q].hi - shift.hi) <= sep) shift = dd_sub(shift, dd_make(sep));
-      tri_lu_dd(d, e, p, shift, tiny, u0, u0 + p, u0 + 2 * p, u0 + 3 * p, u0 + 4 * p);
-    }
-    // rounds 0 and 2 start from fixed pseudo-random vectors: round 1 refines
-    // round 0's, but round 2 follows a check that found an eigenvector round
-    // 1 missed, whose component in round 1's vectors is at rounding level
-    if (round != 1) {
-      for (int idx = tid; idx < rwe * p; idx += kThreads) {
-        const int i = idx / p, j = idx - i * p;
-        Z[idx] = dd_make(1.f + 0.1f * (float)(((j + 1) * 7919 + (i + 1) * 104729) % 97) / 97.f);
+    // one round, compiled for operands all on chip (shared-memory addressing)
+    // and for operands anywhere
+    auto run = [&](auto chip) {
+      constexpr bool kChip = decltype(chip)::value;
+      dd* Z = (kChip || inv_in_smem) ? pool : w.Z;
+      dd* LU = (kChip || inv_in_smem) ? pool + (int64_t)rwe * p : w.lu;
+      dd* rrH = (kChip || plan.rr_in_smem) ? base + plan.vec_units : w.Y;
+      dd* rrR = rrH + (int64_t)plan.rr_dim * plan.rr_dim;
+      const float sep = (round == 0) ? 2.f * kEps32 * tnorm : 1e-12f * tnorm;
+      // rounds 0 and 2 start from fixed pseudo-random vectors: round 1 refines
+      // round 0's, but round 2 follows a check that found an eigenvector round
+      // 1 missed, whose component in round 1's vectors is at rounding level
+      if (round != 1) {
+        for (int idx = tid; idx < rwe * p; idx += kThreads) {
+          const int i = idx / p, j = idx - i * p;
+          Z[idx] = dd_make(1.f + 0.1f * (float)(((j + 1) * 7919 + (i + 1) * 104729) % 97) / 97.f);
+        }
+        __syncthreads();
       }
-    }
-    __syncthreads();
-    for (int it = 0; it < kInvIters; ++it) {
-      for (int i = warp + kWarps * lane; i < rwe; i += kThreads) {
-        dd* u0 = LU + (int64_t)i * 5 * p;
-        tri_solve_dd(p, u0, u0 + p, u0 + 2 * p, u0 + 3 * p, u0 + 4 * p, Z + (int64_t)i * p);
+      for (int it = 0; it < kInvIters; ++it) {
+        // vector i on lane i / 16 of warp i % 16: the factorisations and solves
+        // are serial recurrences, so they are spread over all warps' issue slots
+        for (int i = warp + kWarps * lane; i < rwe; i += kThreads) {
+          dd* u0 = LU + (int64_t)i * 5 * p;
+          dd* z = Z + (int64_t)i * p;
+          if (it == 0) {
+            dd shift = lam[i];
+            for (int q = 0; q < i; ++q)    // (numerically) equal shifts: separate them slightly
+              if (fabsf(lam[q].hi - shift.hi) <= sep) shift = dd_sub(shift, dd_make(sep));
+            tri_lu_forward_dd(d, e, p, shift, tiny, u0, u0 + p, u0 + 2 * p, u0 + 3 * p, u0 + 4 * p, z);
+          } else {
+            tri_forward_dd(p, u0 + 3 * p, u0 + 4 * p, z);
+          }
+          tri_backward_dd(p, u0, u0 + p, u0 + 2 * p, z);
+        }
+        __syncthreads();
+        cgs_dd(Z, rwe, p, (it + 1 == kInvIters) ? 2 : 1, coef, vs, red, sc);
+      }
+      rayleigh_ritz(Z, rwe, p, d, e, rrH, rrR, LU, lam, sc, ord);
+      if (round == 0) return;
+      if (tid == 0) w.clk[4] = clock64();
+
+      // ---- 4. back-transform: v = H_0 H_1 ... H_{p-3} z  (half a warp per
+      //         vector; reflector k - 1 is loaded while k is applied), and the
+      //         check of 3' on the last warp
+      if (warp == kWarps - 1) {
+        if (lane == 0 && round == 1) {
+          const int below = sturm_below_dd(d, e, p, dd_sub(lam[rw - 1], dd_make(1e-13f * tnorm)), sh_f[3]);
+          sh_int[3] = (p - below > rw) ? 1 : 0;
+        }
+        __syncwarp();
+      }
+      for (int i0 = 2 * warp; i0 < rw; i0 += 2 * kWarps) {
+        const int i = i0 + (lane >> 4);
+        dd* z = Z + (int64_t)(i < rw ? i : i0) * p;
+        back_steps<2>(HV, p, z, i < rw, p - 3, p - 33);
+        back_steps<4>(HV, p, z, i < rw, p - 34, p - 65);
+        back_steps<8>(HV, p, z, i < rw, p - 66, p - 129);
+        back_steps<16>(HV, p, z, i < rw, p - 130, 0);
       }
       __syncthreads();
-      cgs_dd(Z, rwe, p, (it + 1 == kInvIters) ? 2 : 1, coef, vs, red, sc);
-    }
-    rayleigh_ritz(Z, rwe, p, d, e, rrH, rrR, LU + (int64_t)rwe * 5 * p, lam, sc, ord);
+    };
+    if (inv_in_smem && plan.rr_in_smem) run(std::true_type{});
+    else run(std::false_type{});
+    if (round == 0) continue;
+    // the embedding of a complex window leaves a failed check to the complex
+    // kernel's FP64 Jacobi: for modes that far below lambda_1 its FP64
+    // backward error keeps A~'s eigenvalues within 1e-9, df64 does not
+    if (!sh_int[3] || a.embed_cx) break;
   }
-  if (tid == 0) w.clk[4] = clock64();
-
-  // ---- 4. back-transform: v = H_0 H_1 ... H_{p-3} z  (half a warp per vector)
-  for (int i0 = 2 * warp; i0 < rw; i0 += 2 * kWarps) {
-    const int i = i0 + (lane >> 4), hl = lane & 15;
-    const bool live = i < rw;
-    dd* z = Z + (int64_t)(live ? i : i0) * p;
-    for (int k = p - 3; k >= 0; --k) {
-      const int Lk = p - k - 1;
-      const dd* v = A + (int64_t)(k + 1) * p + k;   // down column k
-      float ss = 0.f, sc2 = 0.f;
-      if (live)
-        for (int j = hl; j < Lk; j += 16) dot2_acc(ss, sc2, v[(int64_t)j * p], z[k + 1 + j]);
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {   // within each half warp
-        const float so = __shfl_xor_sync(0xffffffffu, ss, o), co = __shfl_xor_sync(0xffffffffu, sc2, o);
-        const dd q = two_sum(ss, so);
-        ss = q.hi;
-        sc2 = (sc2 + co) + q.lo;
-      }
-      const dd s = dd_scale(quick_two_sum(ss, sc2), -2.f);
-      if (live)
-        for (int j = hl; j < Lk; j += 16) z[k + 1 + j] = dd_fma(s, v[(int64_t)j * p], z[k + 1 + j]);
-      __syncwarp();
-    }
-  }
-  __syncthreads();
   if (tid == 0) w.clk[5] = clock64();
   if (a.embed_cx) {
     // hand the K = rw / 2 complex eigenpairs to the complex kernel: lambda_k
     // (unscaled, FP64) at the start of its A~ array, x_k = u + i v from the
-    // pair's first Ritz vector [u; v] (unit norm) in its sorted-V array
+    // pair's first Ritz vector [u; v] (unit norm) in its sorted-V array;
+    // lam_h[K] = 1 accepts the handoff, 0 (a missed eigenvalue, 3') sends the
+    // complex kernel to its Jacobi sweeps.
     double* cxb = a.ws + L.cx;
     double* lam_h = cxb + 2 * 3 * (int64_t)pc * pc;   // A~ region
     double* vec_h = cxb + 2 * 5 * (int64_t)pc * pc;   // sorted-V region: vector k at k pc
     const int K = rw / 2;
-    // Missed-eigenvalue check: inverse iteration finds the eigenvectors
-    // nearest its shifts, and in a cluster below the FP32 multisection's
-    // resolution (eps32 |T|) those need not be the largest. A df64 Sturm
-    // count on T of the eigenvalues above the smallest kept Ritz value (less
-    // 1e-13 |T|) must not exceed rw; lam_h[K] = 1 accepts the handoff, 0
-    // sends the complex kernel to its Jacobi sweeps.
-    if (tid == 0) {
-      const int below = sturm_below_dd(d, e, p, dd_sub(lam[rw - 1], dd_make(1e-13f * tnorm)), sh_f[3]);
-      lam_h[K] = (p - below <= rw) ? 1.0 : 0.0;
-    }
+    if (tid == 0) lam_h[K] = sh_int[3] ? 0.0 : 1.0;
     for (int k = tid; k < K; k += kThreads) lam_h[k] = ldexp(dd_to_double(lam[2 * k]), s_exp);
     for (int idx = tid; idx < K * pc; idx += kThreads) {
       const int k = idx / pc, i = idx - k * pc;
@@ -1305,17 +1595,25 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   }
 
   // ---- 5. rank, sigma, V (FP64 out), vsi = V Sigma^-1 (df64, scaled units)
-  if (tid == 0) {
-    int k = 0;
+  if (warp == 0) {
     bool finite = true;                // a breakdown is reported, not returned as rank 0
-    for (int i = 0; i < rw; ++i) finite = finite && isfinite(dd_to_double(lam[i]));
-    if (!finite) atomicOr(a.status, kDevRank);
     const double lam0 = (rw > 0) ? dd_to_double(lam[0]) : 0.0;
-    if (lam0 > 0.0) {
-      const double thr = lam0 * kRankRtol * (double)p * kEps;
-      while (k < rw && dd_to_double(lam[k]) > thr) ++k;
+    const double thr = lam0 * kRankRtol * (double)p * kEps;
+    int k = 0;                         // leading values above the threshold
+    bool open = lam0 > 0.0;
+    for (int i0 = 0; i0 < rw; i0 += 32) {
+      const double v = (i0 + lane < rw) ? dd_to_double(lam[i0 + lane]) : 0.0;
+      finite = finite && isfinite(v);
+      const unsigned above = __ballot_sync(0xffffffffu, i0 + lane < rw && v > thr);
+      const int n = (above == 0xffffffffu) ? 32 : __ffs(~above) - 1;
+      if (open) k += n;
+      open = open && n == 32;
     }
-    sh_int[1] = k;
+    finite = __all_sync(0xffffffffu, finite);
+    if (lane == 0) {
+      if (!finite) atomicOr(a.status, kDevRank);
+      sh_int[1] = k;
+    }
   }
   __syncthreads();
   const int re = sh_int[1];
@@ -1332,41 +1630,54 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   }
   __syncthreads();
 
-  // ---- 6. A~ = vsi^T G_XY vsi (df64; independent of the scaling). G_XY is
-  //         staged into A's region (free after the back-transform) and Y, A~
-  //         into the inverse iteration's (free after phase 3) when on chip.
-  const dd* GXY = w.GXYd;
-  if (plan.a_in_smem) {
-    for (int idx = tid; idx < p * p; idx += kThreads) big[idx] = w.GXYd[idx];
-    GXY = big;
+  // ---- 6. A~ = vsi^T G_XY vsi (df64; independent of the scaling). Behind Z
+  //         the pool now holds Y = G_XY vsi, A~ and the small eigenproblem,
+  //         and G_XY (transposed) if it fits, else they lie in the workspace.
+  int64_t used = inv_in_smem ? (int64_t)rwe * p : 0;
+  auto take = [&](int64_t units, dd* global) -> dd* {
+    if (used + units > plan.pool_units) return global;
+    dd* at = pool + used;
+    used += units;
+    return at;
+  };
+  const int64_t re2 = (int64_t)re * re;
+  dd* Yb = take((int64_t)re * p, w.Y);
+  dd* At = take((1 + kEigUnits) * re2, nullptr);   // re x re df64, then the eigenproblem
+  const bool eig_on_chip = At != nullptr;
+  if (!eig_on_chip) At = w.lu;
+  const dd* GXYt = take((int64_t)p * p, nullptr);
+  if (GXYt) {
+    for (int idx = tid; idx < p * p; idx += kThreads) const_cast<dd*>(GXYt)[idx] = w.GXYt[idx];
     __syncthreads();
+  } else {
+    GXYt = w.GXYt;
   }
-  dd* Yb = plan.inv_in_smem ? LU : w.Y;
-  dd* At = plan.inv_in_smem ? LU + (int64_t)re * p : w.lu;   // re x re df64
   for (int idx = tid; idx < re * p; idx += kThreads) {
     const int k = idx / p, row = idx - k * p;
-    const dd* g = GXY + (int64_t)row * p;
+    const dd* g = GXYt + row;
     const dd* v = Z + (int64_t)k * p;
     dd s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
     int b = 0;
+#pragma unroll 4
     for (; b + 1 < p; b += 2) {
-      s0 = dd_fma(g[b], v[b], s0);
-      s1 = dd_fma(g[b + 1], v[b + 1], s1);
+      s0 = dd_fma(g[(int64_t)b * p], v[b], s0);
+      s1 = dd_fma(g[(int64_t)(b + 1) * p], v[b + 1], s1);
     }
-    if (b < p) s0 = dd_fma(g[b], v[b], s0);
+    if (b < p) s0 = dd_fma(g[(int64_t)b * p], v[b], s0);
     Yb[idx] = dd_add(s0, s1);
   }
   __syncthreads();
-  CF* Hc = plan.eig_in_smem ? reinterpret_cast<CF*>(big) : reinterpret_cast<CF*>(w.lu + (int64_t)re * re);
-  CF* Qc = Hc + re * re;
-  CF* Wc = Qc + re * re;
-  CF* Uc = Wc + re * re;
-  CF* yc = Uc + re * re;
+  CF* Hc = reinterpret_cast<CF*>(At + re2);
+  CF* Qc = Hc + re2;
+  CF* Wc = Qc + re2;
+  CF* Uc = Wc + re2;
+  CF* yc = Uc + re2;
   for (int idx = tid; idx < re * re; idx += kThreads) {
     const int k = idx / re, l = idx - k * re;
     const dd* v = Z + (int64_t)k * p;
     const dd* y = Yb + (int64_t)l * p;
     dd s = {0.f, 0.f};
+#pragma unroll 4
     for (int b = 0; b < p; ++b) s = dd_fma(v[b], y[b], s);
     At[idx] = s;
     Hc[idx] = {s.hi, 0.f};
@@ -1377,21 +1688,37 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   // ---- 7. eig(A~): FP32 Schur with left and right vectors, then df64
   //         two-sided Rayleigh quotients for the eigenvalues
   if (warp == 0 && re > 0) {
-    const bool ok = warp_eig32(Hc, Qc, Wc, Uc, yc, re, cs, sn);
+    const bool ok = warp_schur32(Hc, Qc, yc, re, cs, sn);
     if (!ok && lane == 0) atomicOr(a.status, kDevRank);
   }
   __syncthreads();
-  double* lam_tmp = reinterpret_cast<double*>(w.Y);   // provisional order (Y is free)
+  if (re > 0) {                          // both sets at once when there is a second ycol
+    if (warp == 0) warp_right32(Hc, Qc, Wc, yc, re);
+    if (!eig_on_chip) __syncthreads();
+    if (warp == 1) warp_left32(Hc, Qc, Uc, eig_on_chip ? yc + re2 : yc, re);
+  }
+  __syncthreads();
+  double* lam_tmp = reinterpret_cast<double*>(vs);   // provisional order (vs, pv are free): 2 re values
+  double* key = reinterpret_cast<double*>(d);        // |lambda|^2 (d, e are free)
+  // the products A~ w_k, one (i, k) per thread, then the quotients
+  dd* aw = eig_on_chip ? reinterpret_cast<dd*>(yc + 2 * re2) : w.Y;   // (re, im) pairs (Y is free)
+  for (int idx = tid; idx < re * re; idx += kThreads) {
+    const int i = idx / re, k = idx - i * re;
+    dd awr = {0.f, 0.f}, awi = {0.f, 0.f};
+    for (int j = 0; j < re; ++j) {
+      const CF wj = Wc[j * re + k];
+      awr = dd_fma(At[i * re + j], dd_make(wj.re), awr);
+      awi = dd_fma(At[i * re + j], dd_make(wj.im), awi);
+    }
+    aw[2 * idx] = awr;
+    aw[2 * idx + 1] = awi;
+  }
+  __syncthreads();
   for (int k = tid; k < re; k += kThreads) {
     // lambda_k = (u^H A~ w) / (u^H w), A~ real df64, u and w promoted exactly
     dd nre = {0.f, 0.f}, nim = {0.f, 0.f}, dre = {0.f, 0.f}, dim = {0.f, 0.f};
     for (int i = 0; i < re; ++i) {
-      dd awr = {0.f, 0.f}, awi = {0.f, 0.f};
-      for (int j = 0; j < re; ++j) {
-        const CF wj = Wc[j * re + k];
-        awr = dd_fma(At[i * re + j], dd_make(wj.re), awr);
-        awi = dd_fma(At[i * re + j], dd_make(wj.im), awi);
-      }
+      const dd awr = aw[2 * (i * re + k)], awi = aw[2 * (i * re + k) + 1];
       const CF ui = Uc[i * re + k];
       const CF wi = Wc[i * re + k];
       // conj(u_i) (aw_i) = (ur ar + ui ai) + i (ur ai - ui ar)
@@ -1401,8 +1728,10 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
       dim = dd_add(dim, dd_sub(two_prod(ui.re, wi.im), two_prod(ui.im, wi.re)));
     }
     const zd lk = zd_div({nre, nim}, {dre, dim});
-    lam_tmp[2 * k] = dd_to_double(lk.re);
-    lam_tmp[2 * k + 1] = dd_to_double(lk.im);
+    const double lr = dd_to_double(lk.re), li = dd_to_double(lk.im);
+    lam_tmp[2 * k] = lr;
+    lam_tmp[2 * k + 1] = li;
+    key[k] = lr * lr + li * li;
   }
   __syncthreads();
   if (tid == 0) {
@@ -1410,10 +1739,10 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     for (int k = 0; k < re; ++k) {
       int best = k;
       for (int q = k + 1; q < re; ++q) {
-        const double br = lam_tmp[2 * ord[best]], bi = lam_tmp[2 * ord[best] + 1];
-        const double qr = lam_tmp[2 * ord[q]], qi = lam_tmp[2 * ord[q] + 1];
-        const double mb = br * br + bi * bi, mq = qr * qr + qi * qi;
-        if (mq > mb || (mq == mb && atan2(qi, qr) < atan2(bi, br))) best = q;
+        const double mb = key[ord[best]], mq = key[ord[q]];
+        if (mq > mb || (mq == mb && atan2(lam_tmp[2 * ord[q] + 1], lam_tmp[2 * ord[q]]) <
+                                        atan2(lam_tmp[2 * ord[best] + 1], lam_tmp[2 * ord[best]])))
+          best = q;
       }
       const int t = ord[k];
       ord[k] = ord[best];
@@ -1479,16 +1808,19 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     w.bamp[2 * k] = br;
     w.bamp[2 * k + 1] = bi;
   }
+  for (int k = tid - 32; k >= 0 && k < re; k += kThreads - 32) {   // warps without an amplitude
+    const double lr = w.lamout[2 * k], li = w.lamout[2 * k + 1];
+    const double lm = 0.5 * log(lr * lr + li * li), th = atan2(li, lr);
+    key[k] = lm * lm + th * th;
+  }
+  __syncthreads();
   if (tid == 0) {
     int best = -1;
     double bv = 0.0;
     for (int k = 0; k < re; ++k) {
-      const double lr = w.lamout[2 * k], li = w.lamout[2 * k + 1];
-      const double lm = 0.5 * log(lr * lr + li * li), th = atan2(li, lr);
-      const double v = lm * lm + th * th;
-      if (best < 0 || v < bv) {
+      if (best < 0 || key[k] < bv) {
         best = k;
-        bv = v;
+        bv = key[k];
       }
     }
     w.bamp[2 * (a.ws_m - 1 > 1 ? a.ws_m - 1 : 1)] = (double)best;   // fixed slot for any window length
@@ -1500,13 +1832,23 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) modes_small_kernel(ModesArgs a, ModesLayout L) { modes_small_body(a, L); }
+// Windows of p <= kSmemMaxP snapshot pairs: one CTA; longer ones: a cluster of
+// kClusterCtas (blockIdx.x / kClusterCtas is the job).
+template <int kCl>
+__global__ void __launch_bounds__(kThreads, 1) modes_small_kernel(ModesArgs a, ModesLayout L) {
+  modes_small_body<kCl>(a, L);
+}
 
-// One CTA per job: the eigensolvers of up to kMaxModesJobs windows (of any
-// length) in one launch, each CTA on its own handle's G and workspace.
-__global__ void __launch_bounds__(kThreads, 1) modes_batch_kernel(ModesBatch b) {
-  const ModesArgs a = b.job[blockIdx.x];
-  modes_small_body(a, modes_layout(a.ws_m));
+// The eigensolvers of up to kMaxModesJobs windows (of any length) in one or
+// two launches, each job on its own handle's G and workspace. With both kinds
+// of window the cluster kernel goes first and lets the other start at once
+// (programmatic launch: they share no data); the other ends after it.
+template <int kCl>
+__global__ void __launch_bounds__(kThreads, 1) modes_batch_kernel(const __grid_constant__ ModesBatch b, int paired) {
+  if (kCl > 1 && paired) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  const ModesArgs a = b.job[blockIdx.x / kCl];
+  modes_small_body<kCl>(a, modes_layout(a.ws_m));
+  if (kCl == 1 && paired) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 
@@ -1751,8 +2093,10 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
 
   // ---- 4. eig(A~): FP32 complex Schur, then FP64 two-sided Rayleigh quotients
   if (warp == 0 && re > 0) {
-    const bool ok = warp_eig32(Hc, Qc, Wc, Uc, yc, re, cs, sn);
+    const bool ok = warp_schur32(Hc, Qc, yc, re, cs, sn);
     if (!ok && lane == 0) atomicOr(a.status, kDevRank);
+    warp_right32(Hc, Qc, Wc, yc, re);
+    warp_left32(Hc, Qc, Uc, yc, re);
   }
   __syncthreads();
   double* lam_tmp = ws + L.Y;
@@ -1880,15 +2224,15 @@ __host__ __device__ ModesLayout modes_layout(int m) {
     o += (n + 31) & ~int64_t(31);   // 256-byte aligned sub-arrays
     return at;
   };
-  L.A = take(p2);           // df64 G_X when it does not fit in shared memory
-  L.GXY = take(p2);         // df64 G_XY
+  L.A = take(p2);           // df64 Householder reflectors (reflector k at k p)
+  L.GXY = take(p2);         // df64 G_XY, transposed
   L.HV = 0;
   L.d = 0;
   L.e = 0;
   L.lam = 0;
   L.Z = take(p2);           // df64 vectors (rw x p)
   L.V = take(p2);           // FP64 V out
-  L.Y = take(2 * p2);       // df64 G_XY vsi; Rayleigh-Ritz matrices when r > 32
+  L.Y = take(2 * p2);       // off chip: df64 G_XY vsi, A~ w; Rayleigh-Ritz matrices when r > 32
   L.At = 0;
   L.Hc = 0;
   L.Qc = 0;
@@ -1898,7 +2242,7 @@ __host__ __device__ ModesLayout modes_layout(int m) {
   L.sig = take(p);
   L.lamout = take(2 * p);
   L.tmp = 0;
-  L.lu = take(6 * p2 + 64); // tridiagonal LU per vector (5 r p) + Ritz scratch (r p); A~ and eig fallback (6 r^2)
+  L.lu = take(6 * p2 + 64); // off chip: tridiagonal LU per vector (5 r p) or Ritz scratch (r p); A~ and eig (6 r^2)
   L.clk = take(16);
   L.bamp = take(2 * p + 2);  // b (re, im) per mode, then [2p] = background index
   L.urec = take(p);          // 2p floats
@@ -1910,37 +2254,96 @@ __host__ __device__ ModesLayout modes_layout(int m) {
 
 int64_t modes_ws_doubles(int m) { return modes_layout(m).total; }
 
+// The complex windows whose G_X goes through the embedding: 2p <= 144, at most
+// 32 Ritz vectors (2K plus the cluster extension), and a working set (G_X, 40
+// vectors, the Ritz matrices, seven vectors per wanted eigenpair) within one
+// SM, or else within the workspace that is laid out for p. The line was drawn
+// where the embedded solver's accuracy and time were measured.
 bool modes_embed_ok(int c, int r) {
   const int pc = c - 1, K = (r < pc) ? r : pc, p = 2 * pc;
-  const SmemPlan plan = smem_plan(p, 2 * K);
-  if (!plan.a_in_smem || !plan.rr_in_smem) return false;
-  if (plan.inv_in_smem) return true;
-  // otherwise LU + Ritz scratch and Z go to the workspace laid out for pc
+  const int P = (p + 3) & ~3;
+  const int rr = (2 * K + kClusterExt < p) ? 2 * K + kClusterExt : p;
+  if (p > kSmemMaxP || rr > kRRMax) return false;
+  constexpr int64_t kRoom = (220 * 1024) / 8;
+  const int64_t vec = 7 * (int64_t)P + 288, mats = 2 * (int64_t)rr * rr, a = (int64_t)p * p, tri = 40 * (int64_t)P + 16;
+  if (vec + mats + a + tri > kRoom) return false;
+  const int64_t eig = 20 * (int64_t)K * K, inv = 7 * (int64_t)rr * p;
+  if (vec + mats + (a > eig ? a : eig) + (inv > tri ? inv : tri) <= kRoom) return true;
   const int64_t pp = (int64_t)pc * pc;
-  return (int64_t)plan.rr_dim * 6 * p <= 6 * pp + 64 && (int64_t)plan.rr_dim * p <= pp;
+  return (int64_t)rr * 6 * p <= 6 * pp + 64 && (int64_t)rr * p <= pp;
+}
+
+static size_t modes_smem_bytes(const ModesArgs& a) {
+  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req);
+  return (size_t)(plan.vec_units + plan.rr_units + plan.pool_units) * 8;
 }
 
 cudaError_t launch_modes_small(const ModesArgs& a, cudaStream_t st) {
-  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req);
-  const size_t bytes = (size_t)(plan.vec_units + plan.rr_units + plan.big_units + plan.inv_units) * 8;
-  const cudaError_t e = smem_optin(reinterpret_cast<const void*>(modes_small_kernel), bytes);
+  const size_t bytes = modes_smem_bytes(a);
+  const bool cluster = !a.embed_cx && a.c - 1 > kSmemMaxP;
+  const void* f = cluster ? reinterpret_cast<const void*>(modes_small_kernel<kClusterCtas>)
+                          : reinterpret_cast<const void*>(modes_small_kernel<1>);
+  const cudaError_t e = smem_optin(f, bytes);
   if (e != cudaSuccess) return e;
-  modes_small_kernel<<<1, kThreads, bytes, st>>>(a, modes_layout(a.ws_m));
-  return cudaGetLastError();
+  if (!cluster) {
+    modes_small_kernel<1><<<1, kThreads, bytes, st>>>(a, modes_layout(a.ws_m));
+    return cudaGetLastError();
+  }
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kClusterCtas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kClusterCtas);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, modes_small_kernel<kClusterCtas>, a, modes_layout(a.ws_m));
 }
 
 cudaError_t launch_modes_batch(const ModesBatch& b, cudaStream_t st) {
   if (b.count < 1 || b.count > kMaxModesJobs) return cudaErrorInvalidValue;
-  size_t bytes = 0;
+  ModesBatch part[2];                    // [0] one-CTA windows, [1] cluster windows
+  size_t bytes[2] = {0, 0};
+  part[0].count = part[1].count = 0;
   for (int i = 0; i < b.count; ++i) {
-    const SmemPlan plan = smem_plan(b.job[i].c - 1, b.job[i].r_req);
-    const size_t jb = (size_t)(plan.vec_units + plan.rr_units + plan.big_units + plan.inv_units) * 8;
-    if (jb > bytes) bytes = jb;
+    const int q = b.job[i].c - 1 > kSmemMaxP;
+    part[q].job[part[q].count++] = b.job[i];
+    const size_t jb = modes_smem_bytes(b.job[i]);
+    if (jb > bytes[q]) bytes[q] = jb;
   }
-  const cudaError_t e = smem_optin(reinterpret_cast<const void*>(modes_batch_kernel), bytes);
+  const int paired = part[0].count > 0 && part[1].count > 0;
+  cudaError_t e = cudaSuccess;
+  if (part[0].count > 0) e = smem_optin(reinterpret_cast<const void*>(modes_batch_kernel<1>), bytes[0]);
+  if (e == cudaSuccess && part[1].count > 0)
+    e = smem_optin(reinterpret_cast<const void*>(modes_batch_kernel<kClusterCtas>), bytes[1]);
   if (e != cudaSuccess) return e;
-  modes_batch_kernel<<<b.count, kThreads, bytes, st>>>(b);
-  return cudaGetLastError();
+  cudaLaunchAttribute at;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (part[1].count > 0) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kClusterCtas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(kClusterCtas * part[1].count);
+    cfg.dynamicSmemBytes = bytes[1];
+    e = cudaLaunchKernelEx(&cfg, modes_batch_kernel<kClusterCtas>, part[1], paired);
+    if (e != cudaSuccess) return e;
+  }
+  if (part[0].count > 0) {
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = paired ? 1 : 0;
+    cfg.gridDim = dim3(part[0].count);
+    cfg.dynamicSmemBytes = bytes[0];
+    e = cudaLaunchKernelEx(&cfg, modes_batch_kernel<1>, part[0], paired);
+  }
+  return e;
 }
 
 cudaError_t launch_modes_complex(const ModesArgs& a, cudaStream_t st) {
