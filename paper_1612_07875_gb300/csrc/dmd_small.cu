@@ -293,10 +293,11 @@ __device__ void tridiagonalize(dd* A, int p, dd* d, dd* e, dd* tw, int P, dd* HV
         u[k + 1] = u0;
         invs[k & 1] = inv;
       }
-    } else if (pend && (kNc > 4 || (warp & 3) != 0)) {
-      // short windows leave warp 0's scheduler to its scalar chain
-      constexpr int kUp = kNc > 4 ? kWarps - 1 : 3 * (kWarps / 4);
-      const int uw = kNc > 4 ? warp - 1 : (warp >> 2) * 3 + (warp & 3) - 1;
+    } else if (pend && (kNc > 2 || (warp & 3) != 0)) {
+      // short windows leave warp 0's scheduler to its scalar chain; longer
+      // ones are bound by the update's FP32 operations
+      constexpr int kUp = kNc > 2 ? kWarps - 1 : 3 * (kWarps / 4);
+      const int uw = kNc > 2 ? warp - 1 : (warp >> 2) * 3 + (warp & 3) - 1;
       dd vc[kNc], wc[kNc];
 #pragma unroll
       for (int c = 0; c < kNc; ++c) {
@@ -824,31 +825,60 @@ __device__ void rayleigh_ritz(dd* Z, int rw, int p, const dd* d, const dd* e, dd
   for (int a = tid; a < rw; a += kThreads) ord[a] = a;
   __syncthreads();
   if (warp == 0) {     // selection sort, descending: the first largest of the rest, by a warp reduction
-    for (int a = 0; a + 1 < rw; ++a) {
-      dd best = {-INFINITY, 0.f};
-      int at = rw;
-      for (int b = a + lane; b < rw; b += 32) {
-        const dd v = H[ord[b] * rw + ord[b]];
-        if (at == rw || dd_lt(best, v)) {
-          best = v;
-          at = b;
-        }
-      }
+    if (rw <= 32) {    // position b on lane b: its value and index in registers
+      int at = lane;
+      dd v = (lane < rw) ? H[lane * rw + lane] : dd{-INFINITY, 0.f};
+      for (int a = 0; a + 1 < rw; ++a) {
+        dd best = (lane >= a) ? v : dd{-INFINITY, 0.f};
+        int pos = (lane >= a && lane < rw) ? lane : 64;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const dd v = shfl_dd(best, o);
-        const int vat = __shfl_xor_sync(0xffffffffu, at, o);
-        if (vat < rw && (at == rw || dd_lt(best, v) || (!dd_lt(v, best) && vat < at))) {
-          best = v;
-          at = vat;
+        for (int o = 16; o > 0; o >>= 1) {
+          const dd x = shfl_dd(best, o);
+          const int xp = __shfl_xor_sync(0xffffffffu, pos, o);
+          const bool less = dd_lt(best, x), more = dd_lt(x, best);
+          const bool take = xp < 64 && (pos == 64 || less || (!more && xp < pos));
+          best = dd_sel(take, x, best);
+          pos = take ? xp : pos;
+        }
+        const dd va = {__shfl_sync(0xffffffffu, v.hi, a), __shfl_sync(0xffffffffu, v.lo, a)};
+        const int ia = __shfl_sync(0xffffffffu, at, a), ib = __shfl_sync(0xffffffffu, at, pos);
+        if (lane == pos) {
+          v = va;
+          at = ia;
+        }
+        if (lane == a) {
+          v = best;
+          at = ib;
         }
       }
-      if (lane == 0 && at != a) {
-        const int t = ord[a];
-        ord[a] = ord[at];
-        ord[at] = t;
+      if (lane < rw) ord[lane] = at;
+    } else {
+      for (int a = 0; a + 1 < rw; ++a) {
+        dd best = {-INFINITY, 0.f};
+        int at = rw;
+        for (int b = a + lane; b < rw; b += 32) {
+          const dd v = H[ord[b] * rw + ord[b]];
+          if (at == rw || dd_lt(best, v)) {
+            best = v;
+            at = b;
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const dd v = shfl_dd(best, o);
+          const int vat = __shfl_xor_sync(0xffffffffu, at, o);
+          if (vat < rw && (at == rw || dd_lt(best, v) || (!dd_lt(v, best) && vat < at))) {
+            best = v;
+            at = vat;
+          }
+        }
+        if (lane == 0 && at != a) {
+          const int t = ord[a];
+          ord[a] = ord[at];
+          ord[at] = t;
+        }
+        __syncwarp();
       }
-      __syncwarp();
     }
   }
   __syncthreads();
@@ -1318,41 +1348,39 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     const dd gv = dd_from_double(v);
     A[idx] = {ldexpf(gv.hi, -s_exp), ldexpf(gv.lo, -s_exp)};
   }
-  // G_X and G_XY entries, kGatherBatch per thread loaded before any is
-  // converted and stored (the stores could alias G for the compiler, so a
-  // plain loop waits a full memory latency per entry; beside a bandwidth-bound
-  // pass that latency is long)
-  // G_XY is kept transposed: phase 6 reads it with consecutive rows over the
-  // lanes. A cluster's CTA takes the rows it owns.
-  constexpr int kGatherBatch = 8;
+  // G_X and G_XY, a row per warp, kGatherBatch entries per lane loaded before
+  // any is converted and stored (the stores could alias G for the compiler, so
+  // a plain loop waits a full memory latency per entry; beside a
+  // bandwidth-bound pass that latency is long). G_XY is kept transposed: phase
+  // 6 reads it with consecutive rows over the lanes. A cluster's CTA takes the
+  // rows it owns.
+  constexpr int kGatherBatch = 4;
   const int nrows = kCl > 1 ? (p >> 3) * 2 + min(max((p & 7) - 2 * rank, 0), 2) : p;   // stored rows of this CTA
-  for (int base = tid; !a.embed_cx && base < nrows * p; base += kThreads * kGatherBatch) {
-    int64_t raw_x[kGatherBatch], raw_xy[kGatherBatch];   // the G words (int64 or the bits of an FP64)
+  for (int li = warp; !a.embed_cx && li < nrows; li += kWarps) {
+    const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
+    int si = a.start + i;
+    if (si >= m) si -= m;
+    const long long* G = static_cast<const long long*>(a.G) + (int64_t)si * m;
+    for (int j0 = lane; j0 < p; j0 += 32 * kGatherBatch) {
+      int64_t raw_x[kGatherBatch], raw_xy[kGatherBatch];   // the G words (int64 or the bits of an FP64)
 #pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u) {
-      const int idx = base + u * kThreads;
-      raw_x[u] = raw_xy[u] = 0;
-      if (idx < nrows * p) {
-        const int li = idx / p, j = idx - li * p;
-        const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
-        int si = a.start + i, sj = a.start + j;
-        if (si >= m) si -= m;
+      for (int q = 0; q < kGatherBatch; ++q) {
+        int sj = a.start + j0 + 32 * q;
         if (sj >= m) sj -= m;
         const int sj1 = (sj + 1 == m) ? 0 : sj + 1;
-        const long long* G = static_cast<const long long*>(a.G);
-        raw_x[u] = G[(int64_t)si * m + sj];
-        raw_xy[u] = G[(int64_t)si * m + sj1];
+        raw_x[q] = raw_xy[q] = 0;
+        if (j0 + 32 * q < p) {
+          raw_x[q] = G[sj];
+          raw_xy[q] = G[sj1];
+        }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u) {
-      const int idx = base + u * kThreads;
-      if (idx < nrows * p) {
-        const int li = idx / p, j = idx - li * p;
-        const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
-        const dd gx = a.g_is_int ? dd_from_ll(raw_x[u]) : dd_from_double(__longlong_as_double(raw_x[u]));
-        const dd gxy = a.g_is_int ? dd_from_ll(raw_xy[u]) : dd_from_double(__longlong_as_double(raw_xy[u]));
-        A[idx] = {ldexpf(gx.hi, -s_exp), ldexpf(gx.lo, -s_exp)};
+      for (int q = 0; q < kGatherBatch; ++q) {
+        const int j = j0 + 32 * q;
+        if (j >= p) continue;
+        const dd gx = a.g_is_int ? dd_from_ll(raw_x[q]) : dd_from_double(__longlong_as_double(raw_x[q]));
+        const dd gxy = a.g_is_int ? dd_from_ll(raw_xy[q]) : dd_from_double(__longlong_as_double(raw_xy[q]));
+        A[li * p + j] = {ldexpf(gx.hi, -s_exp), ldexpf(gx.lo, -s_exp)};
         w.GXYt[(int64_t)j * p + i] = {ldexpf(gxy.hi, -s_exp), ldexpf(gxy.lo, -s_exp)};
       }
     }
@@ -1647,7 +1675,15 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   if (!eig_on_chip) At = w.lu;
   const dd* GXYt = take((int64_t)p * p, nullptr);
   if (GXYt) {
-    for (int idx = tid; idx < p * p; idx += kThreads) const_cast<dd*>(GXYt)[idx] = w.GXYt[idx];
+    constexpr int kBatch = 8;
+    for (int i0 = tid; i0 < p * p; i0 += kThreads * kBatch) {
+      dd x[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) x[q] = (i0 + q * kThreads < p * p) ? w.GXYt[i0 + q * kThreads] : dd{0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q)
+        if (i0 + q * kThreads < p * p) const_cast<dd*>(GXYt)[i0 + q * kThreads] = x[q];
+    }
     __syncthreads();
   } else {
     GXYt = w.GXYt;
@@ -1700,6 +1736,7 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   __syncthreads();
   double* lam_tmp = reinterpret_cast<double*>(vs);   // provisional order (vs, pv are free): 2 re values
   double* key = reinterpret_cast<double*>(d);        // |lambda|^2 (d, e are free)
+  const long long* ikey = reinterpret_cast<const long long*>(d);   // >= 0: ordered as their bits
   // the products A~ w_k, one (i, k) per thread, then the quotients
   dd* aw = eig_on_chip ? reinterpret_cast<dd*>(yc + 2 * re2) : w.Y;   // (re, im) pairs (Y is free)
   for (int idx = tid; idx < re * re; idx += kThreads) {
@@ -1739,7 +1776,7 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     for (int k = 0; k < re; ++k) {
       int best = k;
       for (int q = k + 1; q < re; ++q) {
-        const double mb = key[ord[best]], mq = key[ord[q]];
+        const long long mb = ikey[ord[best]], mq = ikey[ord[q]];
         if (mq > mb || (mq == mb && atan2(lam_tmp[2 * ord[q] + 1], lam_tmp[2 * ord[q]]) <
                                         atan2(lam_tmp[2 * ord[best] + 1], lam_tmp[2 * ord[best]])))
           best = q;
