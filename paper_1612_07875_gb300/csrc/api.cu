@@ -227,6 +227,52 @@ cudaError_t copy_snapshot(void* dst, const void* src, size_t bytes, int num_sms,
   return cudaGetLastError();
 }
 
+// Ingest of several snapshots in one launch: row blockIdx.y of a [k][ld]
+// device array of any alignment into its ring slot. Sources whose rows start
+// off 16 bytes (odd n, rows back to back) are read as aligned 16-byte vectors,
+// two per stored one, and shifted; the first and last vectors of a row, which
+// the aligned reads would leave, byte by byte. A copy per row cost about 5 us
+// each, whatever its size (200 rows of a million bytes: 1.1 ms).
+__global__ void __launch_bounds__(256) ingest_rows_kernel(const uint8_t* __restrict__ src, int64_t row_bytes,
+                                                          int64_t n_bytes, uint8_t* ring, int64_t slot_bytes,
+                                                          int32_t head, int32_t cap) {
+  int32_t slot = head + (int32_t)blockIdx.y;
+  if (slot >= cap) slot -= cap;
+  const uint8_t* s = src + (int64_t)blockIdx.y * row_bytes;
+  uint8_t* d = ring + (int64_t)slot * slot_bytes;
+  const int off = (int)(reinterpret_cast<uintptr_t>(s) & 15u);
+  const int64_t nv = (n_bytes + 15) / 16, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += stride) {
+    const int64_t b = 16 * v;
+    // bytes read: [b - off, b - off + 16) and, if off, the next 16
+    if (b - off < 0 || b - off + (off ? 32 : 16) > n_bytes) {
+      for (int64_t q = b; q < n_bytes && q < b + 16; ++q) d[q] = s[q];
+      continue;
+    }
+    const uint4 x = *reinterpret_cast<const uint4*>(s + b - off);
+    uint4 o = x;
+    if (off) {
+      const uint4 y = *reinterpret_cast<const uint4*>(s + b - off + 16);
+      const unsigned w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+      unsigned r[4];
+      const int sh = 8 * (off & 3);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        unsigned lo = w[q], hi = w[q + 1];          // the words at byte q * 4 + (off & ~3)
+#pragma unroll
+        for (int t = 1; t < 4; ++t)
+          if ((off >> 2) == t) {
+            lo = w[q + t];
+            hi = w[q + t + 1 < 8 ? q + t + 1 : 7];
+          }
+        r[q] = __funnelshift_r(lo, hi, sh);
+      }
+      o = make_uint4(r[0], r[1], r[2], r[3]);
+    }
+    *reinterpret_cast<uint4*>(d + b) = o;
+  }
+}
+
 // Time-ordered copy of the physical G; `words` 8-byte words per entry.
 __global__ void gather_gram_kernel(const uint64_t* G, int m, int c, int start, int words, uint64_t* out) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -593,7 +639,9 @@ int sdmd_push_sparse(sdmd_t h, int32_t nnz, const int32_t* idx, const void* vals
   const int32_t s = h->head;
   int* sidx = h->idx_ring + (int64_t)s * h->nnz_max;
   float2* sval = h->val_ring + (int64_t)s * h->nnz_max;
-  if (nnz > 0) {
+  const bool from_device = nnz > 0 && ptr_kind(idx) == kDevice && ptr_kind(vals) == kDevice &&
+                           (reinterpret_cast<uintptr_t>(idx) & 3u) == 0 && (reinterpret_cast<uintptr_t>(vals) & 7u) == 0;
+  if (nnz > 0 && !from_device) {         // a snapshot in device memory is copied by the scatter kernel
     TraceScope ts(h, SDMD_K_INGEST, st);
     CK(cudaMemcpyAsync(sidx, idx, (size_t)nnz * sizeof(int), cudaMemcpyDefault, st));
     CK(cudaMemcpyAsync(sval, vals, (size_t)nnz * sizeof(float2), cudaMemcpyDefault, st));
@@ -624,7 +672,9 @@ int sdmd_push_sparse(sdmd_t h, int32_t nnz, const int32_t* idx, const void* vals
   a.G = h->G;
   {
     TraceScope ts(h, SDMD_K_GRAM_ROW, st);
-    CK(launch_sparse_scatter(sidx, sval, nnz, h->n, h->stamp, h->tag, h->tval, h->status, st));
+    CK(launch_sparse_scatter(from_device ? idx : sidx, from_device ? static_cast<const float2*>(vals) : sval, nnz, h->n,
+                             h->stamp, h->tag, h->tval, from_device ? sidx : nullptr, from_device ? sval : nullptr,
+                             h->status, st));
     CK(launch_sparse_row(a, st));
   }
   h->head = (s + 1) % h->cap;
@@ -846,7 +896,19 @@ int sdmd_push_batch(sdmd_t h, int32_t k, const void* X, int64_t ld, void* stream
   const int64_t count0 = h->count;
   int copied = 0;
   cudaError_t e = cudaSuccess;
-  for (int j = 0; j < k && e == cudaSuccess; ++j) {        // ingest only
+  if (ptr_kind(X) == kDevice) {                            // ingest only
+    TraceScope ts(h, SDMD_K_INGEST, st);
+    const int64_t bytes = h->n * h->elem;
+    int64_t bx = (bytes + 16 * 256 * 4 - 1) / (16 * 256 * 4);        // four vectors a thread
+    const int64_t most = (16 * (int64_t)h->num_sms + k - 1) / k;
+    if (bx > most) bx = most;
+    if (bx < 1) bx = 1;
+    ingest_rows_kernel<<<dim3((unsigned)bx, (unsigned)k), 256, 0, st>>>(src, ld * h->elem, bytes, h->ring, h->slot_bytes,
+                                                                        head0, h->cap);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) copied = k;
+  }
+  for (int j = copied; j < k && e == cudaSuccess; ++j) {
     TraceScope ts(h, SDMD_K_INGEST, st);
     e = copy_snapshot(h->ring + (int64_t)((head0 + j) % h->cap) * h->slot_bytes, src + (size_t)j * ld * elem_bytes,
                       (size_t)(h->n * h->elem), h->num_sms, st);
@@ -1052,7 +1114,7 @@ int sdmd_rebuild(sdmd_t h, void* stream) {
       a.G = h->G;
       TraceScope ts(h, SDMD_K_GRAM_ROW, st);
       CK(launch_sparse_scatter(h->idx_ring + (int64_t)s * h->nnz_max, h->val_ring + (int64_t)s * h->nnz_max,
-                               h->nnz[s], h->n, h->stamp, h->tag, h->tval, h->status, st));
+                               h->nnz[s], h->n, h->stamp, h->tag, h->tval, nullptr, nullptr, h->status, st));
       CK(launch_sparse_row(a, st));
     } else {
       GramRowArgs a;

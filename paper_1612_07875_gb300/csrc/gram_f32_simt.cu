@@ -232,10 +232,17 @@ __global__ void gram_f32_simt_finish_kernel(GramF32SimtArgs a, int ctas) {
   const int pi = (a.start + i) % a.m;
   for (int j = threadIdx.x; j < a.k; j += blockDim.x) {
     if (i >= t0 && t0 + j > i) continue;
+    // in CTA order, kFinLoads partials in flight (one at a time: 45 us for 152)
+    constexpr int kFinLoads = 16;
     double g = 0.0;
-    for (int b = 0; b < ctas; ++b) {
-      const float2 v = a.partials[((int64_t)b * kSRows + i) * kGramF32SimtMaxTargets + j];
-      g += (double)v.x + (double)v.y;
+    for (int b0 = 0; b0 < ctas; b0 += kFinLoads) {
+      float2 v[kFinLoads];
+#pragma unroll
+      for (int q = 0; q < kFinLoads; ++q)
+        v[q] = a.partials[((int64_t)(b0 + q < ctas ? b0 + q : b0) * kSRows + i) * kGramF32SimtMaxTargets + j];
+#pragma unroll
+      for (int q = 0; q < kFinLoads; ++q)
+        if (b0 + q < ctas) g += (double)v[q].x + (double)v[q].y;
     }
     const int pj = (a.start + t0 + j) % a.m;
     a.G[(int64_t)pi * a.m + pj] = g;

@@ -456,10 +456,17 @@ __global__ void gram_f32_finish_kernel(GramF32Args a, int ctas) {
   const int pi = (a.start + ti) % a.m;
   for (int j = threadIdx.x; j < kt; j += blockDim.x) {
     if (i < kt && i < j) continue;
+    // in CTA order, kFinLoads partials in flight (one at a time: 45 us for 152)
+    constexpr int kFinLoads = 16;
     double g = 0.0;
-    for (int b = 0; b < ctas; ++b) {
-      const float2 v = a.partials[((int64_t)b * kRowsM + i) * kAccCols + j];
-      g += (double)v.x + (double)v.y;
+    for (int b0 = 0; b0 < ctas; b0 += kFinLoads) {
+      float2 v[kFinLoads];
+#pragma unroll
+      for (int q = 0; q < kFinLoads; ++q)
+        v[q] = a.partials[((int64_t)(b0 + q < ctas ? b0 + q : b0) * kRowsM + i) * kAccCols + j];
+#pragma unroll
+      for (int q = 0; q < kFinLoads; ++q)
+        if (b0 + q < ctas) g += (double)v[q].x + (double)v[q].y;
     }
     const int pj = (a.start + a.t_tgt + j) % a.m;
     a.G[(int64_t)pi * a.m + pj] = g;

@@ -11,7 +11,7 @@
 // same MMAs give the column sums s_i = sum_k x'_ik and the count n, and
 //   G_ij = G'_ij + 128 (s_i + s_j) + 128^2 n        (exact int64).
 //
-// GEMM. One launch: the rows of one K-major fp16 tile T (128 rows x 256
+// GEMM. One launch: the rows of one K-major fp16 tile T (128 rows x 128
 // positions, zero rows past the used ones) are a group of k <= 64 target
 // snapshots, the ones row, then a block of older snapshots. D[128 x N] +=
 // T T_B^T, where T_B is the first N = k + 1 (rounded up to 16) rows of the
@@ -26,23 +26,30 @@
 // x positions 8 kg .. 8 kg + 7 at (kg * 16 + rg) * 128 bytes: LBO 2048 B
 // between K neighbours, SBO 128 B between row groups.
 //
-// Work: persistent CTAs take chunks of 4096 positions (16 K-steps of 256)
+// Work: persistent CTAs take chunks of 4096 positions (32 K-steps of 128)
 // from a global counter; the integer sums do not depend on which CTA took
 // which chunk. Per CTA:
-//   warps 9..11  load + convert: warp-private regions of 8 rows x 256 bytes,
-//                cp.async copies (quarter warp = 128 contiguous bytes) into
-//                a 2-deep staging ring (row pitch 272 B), conversion with a
-//                byte permute (fp16 1024 + b) and one f16x2 subtraction of
-//                1152, written into a 2-deep ring of fp16 tiles; bulk L2
-//                prefetches keep the next 1-2 KiB of every row on its way;
-//   warp 8       lane 0 issues 16 MMAs per K-step into one of two TMEM
-//                accumulators (128 x N FP32) and commits every 4 K-steps;
+//   warps 9..16  load + convert: warp-private row groups (8 rows x 128 bytes
+//                per K-step), cp.async copies (a quarter warp = one row's 128
+//                bytes) into an 8-deep staging ring (row pitch 144 B: the
+//                reads of 8 rows hit distinct banks), conversion with a byte
+//                permute (fp16 1024 + b) and one f16x2 subtraction of 1152,
+//                written into a 2-deep ring of fp16 tiles;
+//   warp 8       lane 0 issues 8 MMAs per K-step into one of two TMEM
+//                accumulators (128 x N FP32) and commits every 8 K-steps;
 //   warps 0..7   drain: each reads its 32 TMEM lanes x N/2 columns and adds
-//                the exact integers into int64 registers; at the end the
-//                CTA's partial G' goes to a [CTA][128][128] array.
+//                the exact integers into int32 registers, which go to the
+//                CTA's int64 partial G' [CTA][128][128] after at most 96
+//                periods (96 x 2^24 < 2^31).
 // A second kernel sums the partials over CTAs and writes G (physical slots).
+// What bounds it: the loads in flight, then shared memory. HBM gives one SM
+// about 22 bytes a cycle, 600 cycles for a K-step of 104 rows; the ring keeps
+// 93 KB per SM on its way. Three converter warps with one K-step of 256
+// positions in flight (and L2 prefetches issued as they were needed) took 466
+// us for 8 new HD frames (c = 100), loads straight into registers, 28 KB in
+// flight, 692.
 // Every wait is bounded; on expiry the status word gets kDevTimeout, all
-// roles stop, copies and MMAs are waited for (bounded) and TMEM is freed.
+// roles stop, MMAs are waited for (bounded) and TMEM is freed.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -58,17 +65,19 @@ using namespace tc;
 constexpr int kDrainWarps = 8;       // warps 0..7
 constexpr int kMmaWarp = 8;
 constexpr int kConvWarp0 = 9;
-constexpr int kConvWarps = 3;
-constexpr int kThreads = 32 * (kConvWarp0 + kConvWarps);   // 384
+constexpr int kConvWarps = 8;
+constexpr int kThreads = 32 * (kConvWarp0 + kConvWarps);   // 544
+constexpr int kGroups = 16 / kConvWarps;  // row groups of 8 per converter warp, at most
 constexpr int kRowsM = 128;          // MMA M
-constexpr int kKst = 256;            // positions per K-step
-constexpr int kStepsPerChunk = 16;   // scheduling unit: 4096 positions
-constexpr int kStepsPerDrain = 4;    // 1024 positions per accumulator period
-constexpr int kStages = 2;           // staging ring (u8)
+constexpr int kKst = 128;            // positions per K-step
+constexpr int kStepsPerChunk = 32;   // scheduling unit: 4096 positions
+constexpr int kStepsPerDrain = 8;    // 1024 positions per accumulator period
+constexpr int kStages = 8;           // staging ring (u8): seven K-steps in flight
+constexpr int kPitch = 144;          // staging row pitch, bytes
 constexpr int kTiles = 2;            // fp16 tile ring
-constexpr int kPitch = 272;          // staging row pitch, bytes
-constexpr int kTileBytes = kRowsM * kKst * 2;              // 65536
-constexpr int kStageBytes = kRowsM * kPitch;               // 34816
+constexpr int kFlush = 96;           // accumulator periods between flushes of the int32 sums
+constexpr int kTileBytes = kRowsM * kKst * 2;              // 32768
+constexpr int kStageBytes = kRowsM * kPitch;               // 18432
 constexpr int kTmemCols = 256;       // two accumulators of <= 128 columns
 
 struct FullShared {
@@ -162,7 +171,18 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
     const int cw = warp - kConvWarp0;
     const int ngroups = (c + 1 + 7) / 8;                       // row groups incl. the ones row
     const unsigned stg0 = smem_u32(stg);
-    // K-step sequence: chunk k covers K-steps 16 k .. 16 k + 15 of this CTA
+    // copies of group gi, half t: lane -> row 4 t + lane / 8, 16-byte chunk lane % 8
+    const uint8_t* src[kGroups][2];                            // nullptr: nothing to load
+    unsigned dst[kGroups][2];
+#pragma unroll
+    for (int gi = 0; gi < kGroups; ++gi)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int row = 8 * (cw + kConvWarps * gi) + 4 * t + (lane >> 3);
+        src[gi][t] = (row <= c && row != kt) ? a.ring + sh.tab[row] + 16 * (lane & 7) : nullptr;
+        dst[gi][t] = (unsigned)(row * kPitch + 16 * (lane & 7));
+      }
+    // K-step sequence: chunk k covers K-steps 32 k .. 32 k + 31 of this CTA
     int ld_count = 0, nvalid = 0x7fffffff, cbase = 0;
     bool ended = false;
     // fix the position of K-step number ld_count (or -1 past the end)
@@ -186,15 +206,6 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
             if (lane == 0) raise_timeout(a.status, stop);
             cbase = (int)nchunks;
           }
-          if (cbase < nchunks) {               // this chunk's first 8 K-steps (2 KiB per row) into L2
-            const int64_t x0 = (int64_t)cbase * kStepsPerChunk * kKst;
-            for (int q = cw * 32 + lane; q <= c; q += kConvWarps * 32)
-              if (q != kt) bulk_prefetch_l2(a.ring + sh.tab[q] + x0, 8 * kKst);
-          }
-        } else if (o == 8 && cbase < nchunks) {  // the second half
-          const int64_t x0 = ((int64_t)cbase * kStepsPerChunk + 8) * kKst;
-          for (int q = cw * 32 + lane; q <= c; q += kConvWarps * 32)
-            if (q != kt) bulk_prefetch_l2(a.ring + sh.tab[q] + x0, 8 * kKst);
         }
         if (cbase < nchunks) {
           p0 = ((int64_t)cbase * kStepsPerChunk + o) * kKst;
@@ -207,37 +218,32 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
       return p0;
     };
     int ld_stage = 0;
-    int64_t pos0 = -1, pos1 = -1;            // first position of the K-step in stage 0 / 1
     auto load_next = [&]() {
       const int64_t p0 = fix_next();
-      if (ld_stage == 0) pos0 = p0;
-      else pos1 = p0;
       if (p0 >= 0) {
-        const unsigned dst = stg0 + (unsigned)(ld_stage * kStageBytes);
-        for (int g = cw; g < ngroups; g += kConvWarps) {
+        const unsigned to = stg0 + (unsigned)(ld_stage * kStageBytes);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int row = 8 * g + 2 * t + (lane >> 4), ch = lane & 15;
-            if (row <= c && row != kt)
-              cp_async16(dst + (unsigned)(row * kPitch + 16 * ch), a.ring + sh.tab[row] + p0 + 16 * ch);
-          }
-        }
+        for (int gi = 0; gi < kGroups; ++gi)
+#pragma unroll
+          for (int t = 0; t < 2; ++t)
+            if (src[gi][t]) cp_async16(to + dst[gi][t], src[gi][t] + p0);
       }
-      ld_stage ^= 1;
+      cp_async_commit();                     // one group per K-step, empty past the end
+      ld_stage = (ld_stage + 1 == kStages) ? 0 : ld_stage + 1;
     };
-    load_next();
-    cp_async_commit();
+    for (int s = 0; s < kStages - 1; ++s) load_next();
     int stage = 0;
     Ring tb;
     for (int s = 0; !*stop; ++s) {
-      const bool valid = !(ended && s >= nvalid);
       load_next();
-      cp_async_commit();
-      cp_async_wait<1>();                    // this lane's copies of K-step s have landed
+      const bool valid = !(ended && s >= nvalid);
+      cp_async_wait<kStages - 1>();          // this lane's copies of K-step s have landed
       __syncwarp();                          // ... and those of the other lanes
-      const int64_t p0 = (stage == 0) ? pos0 : pos1;
+      // the chunk's slot in sh.chunk is rewritten two chunks later, after every
+      // converter warp (at most kTiles K-steps behind) has passed this one
+      const int64_t p0 = ((int64_t)sh.chunk[(s / kStepsPerChunk) & 1] * kStepsPerChunk + s % kStepsPerChunk) * kKst;
       const uint8_t* sb = stg + stage * kStageBytes;
-      stage ^= 1;
+      stage = (stage + 1 == kStages) ? 0 : stage + 1;
       int ok = 1;
       if (lane == 0 && s >= kTiles) ok = mbar_wait(smem_u32(&sh.tile_free[tb.idx]), tb.phase ^ 1u);
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -252,12 +258,15 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
         break;
       }
       uint8_t* tile = tiles + tb.idx * kTileBytes;
-      for (int g = cw; g < ngroups; g += kConvWarps) {
+      const bool tail = p0 + kKst > a.n;     // positions past n contribute nothing
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const int row = 8 * g + (lane & 7), ch = (lane >> 3) + 4 * t;   // 16 positions 16 ch ..
-          if (row > c) continue;
-          const int64_t pos = p0 + 16 * ch;
+      for (int gi = 0; gi < kGroups; ++gi) {
+        const int g = cw + kConvWarps * gi, row = 8 * g + (lane & 7);
+        if (g >= ngroups) break;             // warp-uniform
+        if (row > c) continue;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const int ch = 4 * t + (lane >> 3);                  // 16 positions 16 ch ..
           uint4 lo, hi;
           if (row != kt) {
             const uint4 w = *reinterpret_cast<const uint4*>(sb + row * kPitch + 16 * ch);
@@ -273,7 +282,8 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
             lo = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
             hi = lo;
           }
-          if (pos + 16 > a.n) {              // positions past n contribute nothing
+          if (tail) {
+            const int64_t pos = p0 + 16 * ch;
             unsigned wv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -357,11 +367,28 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
     const int lq = warp & 3, half = warp >> 2;
     const int cols = npad / 2;                       // multiple of 8, <= 64
     const int col0 = half * cols;
-    long long sum[8][8];
+    int sum[8][8];
 #pragma unroll
     for (int pc = 0; pc < 8; ++pc)
 #pragma unroll
       for (int i = 0; i < 8; ++i) sum[pc][i] = 0;
+    // this CTA's partial G' (rows and columns 0 .. c; row/column c = sums)
+    const int row = 32 * lq + lane;
+    long long* P = a.partials + (int64_t)blockIdx.x * kRowsM * kRowsM + (int64_t)row * kRowsM + col0;
+    int periods = 0;
+    bool first = true;
+    auto flush = [&]() {
+#pragma unroll
+      for (int pc = 0; pc < 8; ++pc)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int col = col0 + 8 * pc + i;
+          if (8 * pc < cols && row <= c && col <= kt) P[8 * pc + i] = sum[pc][i] + (first ? 0ll : P[8 * pc + i]);
+          sum[pc][i] = 0;
+        }
+      first = false;
+      periods = 0;
+    };
     Ring acc;
     for (;;) {
       if (*stop) break;
@@ -384,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             asm volatile("" : "+r"(v[i]));
-            sum[pc][i] += (long long)__float2int_rn(__uint_as_float(v[i]));
+            sum[pc][i] += __float2int_rn(__uint_as_float(v[i]));
           }
         }
       }
@@ -392,17 +419,9 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&sh.acc_empty[acc.idx]));
       acc.next(2);
+      if (++periods == kFlush) flush();
     }
-    // this CTA's partial G' (rows and columns 0 .. c; row/column c = sums)
-    const int row = 32 * lq + lane;
-    long long* P = a.partials + (int64_t)blockIdx.x * kRowsM * kRowsM;
-#pragma unroll
-    for (int pc = 0; pc < 8; ++pc)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int col = col0 + 8 * pc + i;
-        if (8 * pc < cols && row <= c && col <= kt) P[(int64_t)row * kRowsM + col] = sum[pc][i];
-      }
+    if (periods > 0 || first) flush();
   }
   __syncthreads();
   fence_after();
@@ -411,36 +430,44 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
 }
 
 // G_ij = G'_ij + 128 (s_i + s_j) + 128^2 n from the per-CTA partials, for
-// every tile row i (one block each) and target j (threads), written to both
-// G[i][j] and G[j][i] at the physical slots.
-__global__ void reset_sched_kernel(unsigned* sched) { sched[0] = 0u; }   // ready for the next launch
-
-__global__ void gram_full_finish_kernel(GramFullArgs a, int ctas) {
-  __shared__ long long si_n[2];
+// every tile row i (one block each) and target j, written to both G[i][j] and
+// G[j][i] at the physical slots. s_j comes from the ones row (coalesced, the
+// same integers as its column). kFinSlices threads per column share the CTAs:
+// one thread per column walked 152 partials 128 KB apart in 56 us.
+constexpr int kFinSlices = 4;
+__global__ void __launch_bounds__(kRowsM * kFinSlices) gram_full_finish_kernel(GramFullArgs a, int ctas) {
+  __shared__ long long gi[kFinSlices][kRowsM], gs[kFinSlices][kRowsM];
   const int i = blockIdx.x, kt = a.k;
+  const int j = threadIdx.x % kRowsM, sl = threadIdx.x / kRowsM;
+  if (i == 0 && threadIdx.x == 0) a.sched[0] = 0u;   // ready for the next launch
   if (i == kt) return;                   // the ones row
-  if (threadIdx.x < 2) {                 // s_i = G'_i,kt and n = G'_kt,kt
-    const int rw = (threadIdx.x == 0) ? i : kt;
-    long long s = 0;
-    for (int b = 0; b < ctas; ++b) s += a.partials[((int64_t)b * kRowsM + rw) * kRowsM + kt];
-    si_n[threadIdx.x] = s;
-  }
-  __syncthreads();
-  const long long si = si_n[0], n = si_n[1];
-  const int ti = (i < kt) ? a.t_tgt + i : a.t_old + (i - kt - 1);
-  const int pi = (a.start + ti) % a.m;
-  for (int j = threadIdx.x; j < kt; j += blockDim.x) {
-    long long g = 0, sj = 0;
-    for (int b = 0; b < ctas; ++b) {
-      const long long* P = a.partials + (int64_t)b * kRowsM * kRowsM;
-      g += P[(int64_t)i * kRowsM + j];
-      sj += P[(int64_t)j * kRowsM + kt];
+  long long g = 0, s = 0;
+  if (j <= kt) {
+    const long long* P = a.partials + j;
+#pragma unroll 8
+    for (int b = sl; b < ctas; b += kFinSlices) {
+      g += P[((int64_t)b * kRowsM + i) * kRowsM];
+      s += P[((int64_t)b * kRowsM + kt) * kRowsM];
     }
-    const long long v = g + 128LL * (si + sj) + 16384LL * n;
-    const int pj = (a.start + a.t_tgt + j) % a.m;
-    a.G[(int64_t)pi * a.m + pj] = v;
-    a.G[(int64_t)pj * a.m + pi] = v;
   }
+  gi[sl][j] = g;
+  gs[sl][j] = s;
+  __syncthreads();
+  if (sl > 0 || j >= kt) return;
+  long long si = 0, n = 0;
+  g = s = 0;
+#pragma unroll
+  for (int q = 0; q < kFinSlices; ++q) {
+    g += gi[q][j];
+    s += gs[q][j];
+    si += gi[q][kt];                     // s_i = G'_i,kt and n = G'_kt,kt
+    n += gs[q][kt];
+  }
+  const int ti = (i < kt) ? a.t_tgt + i : a.t_old + (i - kt - 1);
+  const int pi = (a.start + ti) % a.m, pj = (a.start + a.t_tgt + j) % a.m;
+  const long long v = g + 128LL * (si + s) + 16384LL * n;
+  a.G[(int64_t)pi * a.m + pj] = v;
+  a.G[(int64_t)pj * a.m + pi] = v;
 }
 
 }  // namespace
@@ -476,10 +503,7 @@ cudaError_t launch_gram_full_tc(const GramFullArgs& base, int* ctas_out, cudaStr
       gram_full_tc_kernel<<<ctas, kThreads, kSmemBytes, st>>>(a);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
-      gram_full_finish_kernel<<<a.k + 1 + a.nold, 128, 0, st>>>(a, ctas);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-      reset_sched_kernel<<<1, 1, 0, st>>>(a.sched);
+      gram_full_finish_kernel<<<a.k + 1 + a.nold, kRowsM * kFinSlices, 0, st>>>(a, ctas);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
       o += a.nold;

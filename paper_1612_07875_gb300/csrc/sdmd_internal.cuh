@@ -317,8 +317,10 @@ struct SparseRowArgs {
 
 // CTAs a snapshot with nnz entries takes in the sparse row kernel.
 int sparse_chunks(int nnz);
+// The new snapshot's table entries; with ring_idx / ring_val also its copy into
+// the ring slot (idx, val in device memory).
 cudaError_t launch_sparse_scatter(const int* idx, const float2* val, int nnz, int64_t n, int stamp, int* tag,
-                                  float2* tval, int* status, cudaStream_t st);
+                                  float2* tval, int* ring_idx, float2* ring_val, int* status, cudaStream_t st);
 cudaError_t launch_sparse_row(const SparseRowArgs& a, cudaStream_t st);
 
 // Modes of a Fourier-sparse window in coefficient space (compressed Phi-hat).
@@ -334,7 +336,7 @@ struct FourierPhiArgs {
   const float* Mf;           // p x 2R (re, im) of M = V Sigma^-1 W
   int64_t n;                 // coefficients per snapshot
   unsigned* bitmap;          // ceil(n / 32) words
-  unsigned long long* prefix;// ceil(n / 32) exclusive popcount prefix
+  unsigned long long* prefix;// popcounts of the bitmap's blocks of words (at most ceil(n / 32) of them)
   unsigned long long* count; // union size
   int* idx_out;              // cap sorted coefficient indices
   float2* phi_out;           // cap x r complex64, column-major (leading dimension cap)
