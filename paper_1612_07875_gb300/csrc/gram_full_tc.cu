@@ -26,28 +26,28 @@
 // x positions 8 kg .. 8 kg + 7 at (kg * 16 + rg) * 128 bytes: LBO 2048 B
 // between K neighbours, SBO 128 B between row groups.
 //
-// Work: persistent CTAs take chunks of 4096 positions (32 K-steps of 128)
+// Work: persistent CTAs take chunks of 2048 positions (8 K-steps of 256)
 // from a global counter; the integer sums do not depend on which CTA took
 // which chunk. Per CTA:
 //   warps 9..16  load + convert: warp-private row groups (8 rows x 128 bytes
-//                per K-step), cp.async copies (a quarter warp = one row's 128
-//                bytes) into an 8-deep staging ring (row pitch 144 B: the
+//                per stage), cp.async copies (a quarter warp = one row's 128
+//                bytes) into a 5-deep staging ring (row pitch 144 B: the
 //                reads of 8 rows hit distinct banks), conversion with a byte
 //                permute (fp16 1024 + b) and one f16x2 subtraction of 1152,
-//                written into a 2-deep ring of fp16 tiles;
-//   warp 8       lane 0 issues 8 MMAs per K-step into one of two TMEM
-//                accumulators (128 x N FP32) and commits every 8 K-steps;
+//                branch-free, two stages into one tile of a 2-deep ring;
+//   warp 8       lane 0 issues 16 MMAs per K-step into one of two TMEM
+//                accumulators (128 x N FP32) and commits every 4 K-steps;
 //   warps 0..7   drain: each reads its 32 TMEM lanes x N/2 columns and adds
 //                the exact integers into int32 registers, which go to the
 //                CTA's int64 partial G' [CTA][128][128] after at most 96
 //                periods (96 x 2^24 < 2^31).
 // A second kernel sums the partials over CTAs and writes G (physical slots).
-// What bounds it: the loads in flight, then shared memory. HBM gives one SM
-// about 22 bytes a cycle, 600 cycles for a K-step of 104 rows; the ring keeps
-// 93 KB per SM on its way. Three converter warps with one K-step of 256
-// positions in flight (and L2 prefetches issued as they were needed) took 466
-// us for 8 new HD frames (c = 100), loads straight into registers, 28 KB in
-// flight, 692.
+// What bounds it: the converter warps' time per K-step (hand-over waits, the
+// copies' issue and the conversion), against about 1,200 cycles in which HBM
+// delivers 104 rows of 256 bytes to one SM; without any MMA the kernel takes
+// the same time. For 8 new HD frames (c = 100): three converter warps with one
+// K-step in flight 466 us; loads straight into registers, 28 KB in flight, 692;
+// eight warps, K-steps of 128 handed on one by one with branches per row 266.
 // Every wait is bounded; on expiry the status word gets kDevTimeout, all
 // roles stop, MMAs are waited for (bounded) and TMEM is freed.
 #include <cuda_runtime.h>
@@ -69,14 +69,16 @@ constexpr int kConvWarps = 8;
 constexpr int kThreads = 32 * (kConvWarp0 + kConvWarps);   // 544
 constexpr int kGroups = 16 / kConvWarps;  // row groups of 8 per converter warp, at most
 constexpr int kRowsM = 128;          // MMA M
-constexpr int kKst = 128;            // positions per K-step
-constexpr int kStepsPerChunk = 32;   // scheduling unit: 4096 positions
-constexpr int kStepsPerDrain = 8;    // 1024 positions per accumulator period
-constexpr int kStages = 8;           // staging ring (u8): seven K-steps in flight
+constexpr int kKst = 256;            // positions per K-step
+constexpr int kStepsPerChunk = 8;    // scheduling unit: 2048 positions
+constexpr int kStepsPerDrain = 4;    // 1024 positions per accumulator period
+constexpr int kHalf = 128;           // positions per staging stage
+constexpr int kHalves = kKst / kHalf;
+constexpr int kStages = 5;           // staging ring (u8): four stages in flight
 constexpr int kPitch = 144;          // staging row pitch, bytes
 constexpr int kTiles = 2;            // fp16 tile ring
 constexpr int kFlush = 96;           // accumulator periods between flushes of the int32 sums
-constexpr int kTileBytes = kRowsM * kKst * 2;              // 32768
+constexpr int kTileBytes = kRowsM * kKst * 2;              // 65536
 constexpr int kStageBytes = kRowsM * kPitch;               // 18432
 constexpr int kTmemCols = 256;       // two accumulators of <= 128 columns
 
@@ -160,6 +162,10 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
     if (row > c) *reinterpret_cast<uint4*>(tiles + t * kTileBytes + (kg * 16 + (row >> 3)) * 128 + (row & 7) * 16) =
                      make_uint4(0u, 0u, 0u, 0u);
   }
+  // the ones row (positions past n are cleared where they occur)
+  for (int idx = tid; idx < kTiles * (kKst / 8); idx += kThreads)
+    *reinterpret_cast<uint4*>(tiles + (idx / (kKst / 8)) * kTileBytes + ((idx % (kKst / 8)) * 16 + (kt >> 3)) * 128 + (kt & 7) * 16) =
+        make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
   fence_proxy_async();
   fence_before();
   __syncthreads();
@@ -171,83 +177,86 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
     const int cw = warp - kConvWarp0;
     const int ngroups = (c + 1 + 7) / 8;                       // row groups incl. the ones row
     const unsigned stg0 = smem_u32(stg);
-    // copies of group gi, half t: lane -> row 4 t + lane / 8, 16-byte chunk lane % 8
-    const uint8_t* src[kGroups][2];                            // nullptr: nothing to load
+    const int ng = (ngroups > cw + kConvWarps) ? 2 : (ngroups > cw ? 1 : 0);   // this warp's row groups
+    static_assert(kGroups == 2, "ng");
+    // copies of group gi, t = 0, 1: lane -> row 4 t + lane / 8, 16-byte chunk
+    // lane % 8; rows without a snapshot (the ones row, padding) copy row 0's
+    // bytes, which are not used, so that no lane branches
+    const uint8_t* src[kGroups][2];
     unsigned dst[kGroups][2];
 #pragma unroll
     for (int gi = 0; gi < kGroups; ++gi)
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const int row = 8 * (cw + kConvWarps * gi) + 4 * t + (lane >> 3);
-        src[gi][t] = (row <= c && row != kt) ? a.ring + sh.tab[row] + 16 * (lane & 7) : nullptr;
+        src[gi][t] = a.ring + sh.tab[(row <= c && row != kt) ? row : 0] + 16 * (lane & 7);
         dst[gi][t] = (unsigned)(row * kPitch + 16 * (lane & 7));
       }
-    // K-step sequence: chunk k covers K-steps 32 k .. 32 k + 31 of this CTA
-    int ld_count = 0, nvalid = 0x7fffffff, cbase = 0;
+    // conversion: lane -> row lane % 8 of the group, chunks lane / 8 and lane / 8 + 4
+    bool st_ok[kGroups];
+#pragma unroll
+    for (int gi = 0; gi < kGroups; ++gi) {
+      const int row = 8 * (cw + kConvWarps * gi) + (lane & 7);
+      st_ok[gi] = gi < ng && row <= c && row != kt;
+    }
+    // stage sequence: chunk k covers stages 16 k .. 16 k + 15 of this CTA, two a K-step
+    constexpr int kHalvesPerChunk = kStepsPerChunk * kHalves;
+    int ld_count = 0, nvalid = 0x7fffffff, cbase = 0, o = 0, ck = 0;
     bool ended = false;
-    // fix the position of K-step number ld_count (or -1 past the end)
+    // fix the position of stage number ld_count (or -1 past the end)
     auto fix_next = [&]() -> int64_t {
-      int64_t p0 = -1;
-      if (!ended) {
-        const int ck = ld_count / kStepsPerChunk, o = ld_count % kStepsPerChunk;
-        if (o == 0) {
-          const unsigned bar = smem_u32(&sh.chunk_bar[ck & 1]);
-          if (cw == 0 && lane == 0) {
-            sh.chunk[ck & 1] = (int)atomicAdd(a.sched, 1u);
-            mbar_arrive(bar);
-          }
-          int ok = 1;
-          if (lane == 0) ok = mbar_wait(bar, (unsigned)((ck >> 1) & 1));
-          ok = __shfl_sync(0xffffffffu, ok, 0);
-          __syncwarp();
-          if (ok) {
-            cbase = sh.chunk[ck & 1];
-          } else {
-            if (lane == 0) raise_timeout(a.status, stop);
-            cbase = (int)nchunks;
-          }
+      if (ended) return -1;
+      if (o == 0) {
+        const unsigned bar = smem_u32(&sh.chunk_bar[ck & 1]);
+        if (cw == 0 && lane == 0) {
+          sh.chunk[ck & 1] = (int)atomicAdd(a.sched, 1u);
+          mbar_arrive(bar);
         }
-        if (cbase < nchunks) {
-          p0 = ((int64_t)cbase * kStepsPerChunk + o) * kKst;
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait(bar, (unsigned)((ck >> 1) & 1));
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        if (ok) {
+          cbase = sh.chunk[ck & 1];
         } else {
+          if (lane == 0) raise_timeout(a.status, stop);
+          cbase = (int)nchunks;
+        }
+        if (cbase >= nchunks) {
           ended = true;
           nvalid = ld_count;
+          return -1;
         }
       }
+      const int64_t p0 = ((int64_t)cbase * kHalvesPerChunk + o) * kHalf;
       ++ld_count;
+      if (++o == kHalvesPerChunk) {
+        o = 0;
+        ++ck;
+      }
       return p0;
     };
-    int ld_stage = 0;
+    unsigned ld_to = stg0;
     auto load_next = [&]() {
       const int64_t p0 = fix_next();
       if (p0 >= 0) {
-        const unsigned to = stg0 + (unsigned)(ld_stage * kStageBytes);
 #pragma unroll
         for (int gi = 0; gi < kGroups; ++gi)
-#pragma unroll
-          for (int t = 0; t < 2; ++t)
-            if (src[gi][t]) cp_async16(to + dst[gi][t], src[gi][t] + p0);
+          if (gi < ng) {
+            cp_async16(ld_to + dst[gi][0], src[gi][0] + p0);
+            cp_async16(ld_to + dst[gi][1], src[gi][1] + p0);
+          }
       }
-      cp_async_commit();                     // one group per K-step, empty past the end
-      ld_stage = (ld_stage + 1 == kStages) ? 0 : ld_stage + 1;
+      cp_async_commit();                     // one group per stage, empty past the end
+      ld_to = (ld_to + kStageBytes == stg0 + kStages * kStageBytes) ? stg0 : ld_to + kStageBytes;
     };
     for (int s = 0; s < kStages - 1; ++s) load_next();
     int stage = 0;
     Ring tb;
     for (int s = 0; !*stop; ++s) {
-      load_next();
-      const bool valid = !(ended && s >= nvalid);
-      cp_async_wait<kStages - 1>();          // this lane's copies of K-step s have landed
-      __syncwarp();                          // ... and those of the other lanes
-      // the chunk's slot in sh.chunk is rewritten two chunks later, after every
-      // converter warp (at most kTiles K-steps behind) has passed this one
-      const int64_t p0 = ((int64_t)sh.chunk[(s / kStepsPerChunk) & 1] * kStepsPerChunk + s % kStepsPerChunk) * kKst;
-      const uint8_t* sb = stg + stage * kStageBytes;
-      stage = (stage + 1 == kStages) ? 0 : stage + 1;
-      int ok = 1;
-      if (lane == 0 && s >= kTiles) ok = mbar_wait(smem_u32(&sh.tile_free[tb.idx]), tb.phase ^ 1u);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
+      const bool valid = !(ended && kHalves * s >= nvalid);
+      const bool ok = s < kTiles || mbar_wait(smem_u32(&sh.tile_free[tb.idx]), tb.phase ^ 1u);
+      if (__any_sync(0xffffffffu, !ok)) {
         if (lane == 0) raise_timeout(a.status, stop);
         break;
       }
@@ -258,45 +267,66 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
         break;
       }
       uint8_t* tile = tiles + tb.idx * kTileBytes;
+      // the chunk's slot in sh.chunk is rewritten two chunks later, after every
+      // converter warp (at most kTiles K-steps behind) has passed this one
+      const int64_t p0 = ((int64_t)sh.chunk[(s / kStepsPerChunk) & 1] * kStepsPerChunk + s % kStepsPerChunk) * kKst;
       const bool tail = p0 + kKst > a.n;     // positions past n contribute nothing
 #pragma unroll
-      for (int gi = 0; gi < kGroups; ++gi) {
-        const int g = cw + kConvWarps * gi, row = 8 * g + (lane & 7);
-        if (g >= ngroups) break;             // warp-uniform
-        if (row > c) continue;
+      for (int hf = 0; hf < kHalves; ++hf) {
+        load_next();
+        cp_async_wait<kStages - 1>();        // this lane's copies of the stage have landed
+        __syncwarp();                        // ... and those of the other lanes
+        const uint8_t* sb = stg + stage * kStageBytes;
+        stage = (stage + 1 == kStages) ? 0 : stage + 1;
+        uint4 w[kGroups][2];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          const int ch = 4 * t + (lane >> 3);                  // 16 positions 16 ch ..
-          uint4 lo, hi;
-          if (row != kt) {
-            const uint4 w = *reinterpret_cast<const uint4*>(sb + row * kPitch + 16 * ch);
-            lo.x = f16x2_centred(w.x, 0x4140u);
-            lo.y = f16x2_centred(w.x, 0x4342u);
-            lo.z = f16x2_centred(w.y, 0x4140u);
-            lo.w = f16x2_centred(w.y, 0x4342u);
-            hi.x = f16x2_centred(w.z, 0x4140u);
-            hi.y = f16x2_centred(w.z, 0x4342u);
-            hi.z = f16x2_centred(w.w, 0x4140u);
-            hi.w = f16x2_centred(w.w, 0x4342u);
-          } else {                           // the ones row
-            lo = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
-            hi = lo;
+        for (int gi = 0; gi < kGroups; ++gi)
+          if (gi < ng) {
+            const uint8_t* r = sb + (8 * (cw + kConvWarps * gi) + (lane & 7)) * kPitch + 16 * (lane >> 3);
+            w[gi][0] = *reinterpret_cast<const uint4*>(r);
+            w[gi][1] = *reinterpret_cast<const uint4*>(r + 64);
           }
-          if (tail) {
-            const int64_t pos = p0 + 16 * ch;
-            unsigned wv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int64_t pa = pos + 2 * q;
-              if (pa >= a.n) wv[q] = 0u;
-              else if (pa + 1 >= a.n) wv[q] &= 0x0000FFFFu;   // element 0 is the low half
+        for (int gi = 0; gi < kGroups; ++gi) {
+          if (gi >= ng) break;               // warp-uniform
+          const int g = cw + kConvWarps * gi;
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const int ch = 8 * hf + 4 * t + (lane >> 3);         // positions 16 ch .. of the K-step
+            const uint4 x = w[gi][t];
+            uint4 lo, hi;
+            lo.x = f16x2_centred(x.x, 0x4140u);
+            lo.y = f16x2_centred(x.x, 0x4342u);
+            lo.z = f16x2_centred(x.y, 0x4140u);
+            lo.w = f16x2_centred(x.y, 0x4342u);
+            hi.x = f16x2_centred(x.z, 0x4140u);
+            hi.y = f16x2_centred(x.z, 0x4342u);
+            hi.z = f16x2_centred(x.w, 0x4140u);
+            hi.w = f16x2_centred(x.w, 0x4342u);
+            uint8_t* core = tile + (size_t)((2 * ch) * 16 + g) * 128 + (lane & 7) * 16;
+            bool store = st_ok[gi];
+            if (tail) {                      // masked; the ones row too
+              if (8 * g + (lane & 7) == kt) {
+                lo = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
+                hi = lo;
+                store = true;
+              }
+              const int64_t pos = p0 + 16 * ch;
+              unsigned wv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const int64_t pa = pos + 2 * q;
+                if (pa >= a.n) wv[q] = 0u;
+                else if (pa + 1 >= a.n) wv[q] &= 0x0000FFFFu;   // element 0 is the low half
+              }
+              lo = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+              hi = make_uint4(wv[4], wv[5], wv[6], wv[7]);
             }
-            lo = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            hi = make_uint4(wv[4], wv[5], wv[6], wv[7]);
+            if (store) {
+              *reinterpret_cast<uint4*>(core) = lo;
+              *reinterpret_cast<uint4*>(core + 16 * 128) = hi;   // kg + 1: 16 row groups further
+            }
           }
-          uint8_t* core = tile + (size_t)((2 * ch) * 16 + g) * 128 + (row & 7) * 16;
-          *reinterpret_cast<uint4*>(core) = lo;
-          *reinterpret_cast<uint4*>(core + 16 * 128) = hi;     // kg + 1: 16 row groups further
         }
       }
       fence_proxy_async();
@@ -432,36 +462,36 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
 // G_ij = G'_ij + 128 (s_i + s_j) + 128^2 n from the per-CTA partials, for
 // every tile row i (one block each) and target j, written to both G[i][j] and
 // G[j][i] at the physical slots. s_j comes from the ones row (coalesced, the
-// same integers as its column). kFinSlices threads per column share the CTAs:
-// one thread per column walked 152 partials 128 KB apart in 56 us.
-constexpr int kFinSlices = 4;
-__global__ void __launch_bounds__(kRowsM * kFinSlices) gram_full_finish_kernel(GramFullArgs a, int ctas) {
-  __shared__ long long gi[kFinSlices][kRowsM], gs[kFinSlices][kRowsM];
+// same integers as its column). The threads split into columns (cw of them, a
+// power of two past k) and slices of the CTAs: one thread per column walked 152
+// partials 128 KB apart in 56 us.
+constexpr int kFinThreads = 1024;
+__global__ void __launch_bounds__(kFinThreads) gram_full_finish_kernel(GramFullArgs a, int ctas, int cw) {
+  __shared__ long long gi[kFinThreads], gs[kFinThreads];   // [slice][cw]
   const int i = blockIdx.x, kt = a.k;
-  const int j = threadIdx.x % kRowsM, sl = threadIdx.x / kRowsM;
+  const int j = threadIdx.x % cw, sl = threadIdx.x / cw, slices = kFinThreads / cw;
   if (i == 0 && threadIdx.x == 0) a.sched[0] = 0u;   // ready for the next launch
   if (i == kt) return;                   // the ones row
   long long g = 0, s = 0;
   if (j <= kt) {
     const long long* P = a.partials + j;
-#pragma unroll 8
-    for (int b = sl; b < ctas; b += kFinSlices) {
+#pragma unroll 10
+    for (int b = sl; b < ctas; b += slices) {
       g += P[((int64_t)b * kRowsM + i) * kRowsM];
       s += P[((int64_t)b * kRowsM + kt) * kRowsM];
     }
   }
-  gi[sl][j] = g;
-  gs[sl][j] = s;
+  gi[threadIdx.x] = g;
+  gs[threadIdx.x] = s;
   __syncthreads();
   if (sl > 0 || j >= kt) return;
   long long si = 0, n = 0;
   g = s = 0;
-#pragma unroll
-  for (int q = 0; q < kFinSlices; ++q) {
-    g += gi[q][j];
-    s += gs[q][j];
-    si += gi[q][kt];                     // s_i = G'_i,kt and n = G'_kt,kt
-    n += gs[q][kt];
+  for (int q = 0; q < slices; ++q) {
+    g += gi[q * cw + j];
+    s += gs[q * cw + j];
+    si += gi[q * cw + kt];               // s_i = G'_i,kt and n = G'_kt,kt
+    n += gs[q * cw + kt];
   }
   const int ti = (i < kt) ? a.t_tgt + i : a.t_old + (i - kt - 1);
   const int pi = (a.start + ti) % a.m, pj = (a.start + a.t_tgt + j) % a.m;
@@ -503,7 +533,9 @@ cudaError_t launch_gram_full_tc(const GramFullArgs& base, int* ctas_out, cudaStr
       gram_full_tc_kernel<<<ctas, kThreads, kSmemBytes, st>>>(a);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
-      gram_full_finish_kernel<<<a.k + 1 + a.nold, kRowsM * kFinSlices, 0, st>>>(a, ctas);
+      int cw = 8;                          // columns 0 .. k, padded to a power of two
+      while (cw < a.k + 1) cw *= 2;
+      gram_full_finish_kernel<<<a.k + 1 + a.nold, kFinThreads, 0, st>>>(a, ctas, cw);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
       o += a.nold;
