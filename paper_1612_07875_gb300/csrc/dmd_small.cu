@@ -1898,9 +1898,17 @@ __global__ void __launch_bounds__(kThreads, 1) modes_batch_kernel(const __grid_c
 // FP64 two-sided Rayleigh quotients, M = vsi W, amplitudes and the
 // background index as for real windows. Outputs go to the same workspace
 // arrays (sig, lamout, Mf, bamp, r_dev); V (complex) to the cx region.
+//
+// FP64 runs at two lanes per cycle and SM, so the products of phases 3 and 5
+// (0.28 M FP64 operations at p = 63, r = 10) are spread over a cluster of
+// kCxCtas CTAs, every entry by one thread in the order it always had; the
+// rest is CTA 0's. With the handoff the eigenpairs come sorted and G_X is not
+// gathered. 470 us before, one CTA, a single thread sorting p values and the
+// background index mode by mode.
 constexpr int kCThreads = 512;
 constexpr int kCWarps = kCThreads / 32;
 constexpr int kJacobiMaxSweeps = 40;
+constexpr int kCxCtas = 8;
 
 struct C64d {
   double re, im;
@@ -1931,7 +1939,11 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
   __shared__ float cs[SDMD_MAX_M];
   __shared__ CF sn[SDMD_MAX_M];
   __shared__ int sh_int[4];
+  __shared__ double key_s[SDMD_MAX_M];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const bool lead = rank == 0;
   const int m = a.m, p = a.c - 1;
   const int R = a.r_req;
   double* ws = a.ws;
@@ -1958,23 +1970,28 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
   }
   __syncthreads();
   const int s_exp = sh_int[0];
-  for (int idx = tid; idx < p * p; idx += kCThreads) {
+  // the handoff of the embedded solve, if it passed its missed-eigenvalue check
+  const bool pre = a.cx_pre && reinterpret_cast<const double*>(At)[min(R, p)] == 1.0;
+  // G_XY (rows over the cluster), and without the handoff G_X
+  for (int idx = rank * kCThreads + tid; idx < p * p; idx += kCxCtas * kCThreads) {
     const int i = idx / p, j = idx - i * p;
     const int si = (a.start + i) % m, sj = (a.start + j) % m, sj1 = (a.start + j + 1) % m;
-    const double2 gx = G[(int64_t)si * m + sj], gxy = G[(int64_t)si * m + sj1];
-    Ac[idx] = {ldexp(gx.x, -s_exp), (i == j) ? 0.0 : ldexp(gx.y, -s_exp)};
+    const double2 gxy = G[(int64_t)si * m + sj1];
     Bc[idx] = {ldexp(gxy.x, -s_exp), ldexp(gxy.y, -s_exp)};
-    Vc[idx] = {(i == j) ? 1.0 : 0.0, 0.0};
+    if (!pre) {
+      const double2 gx = G[(int64_t)si * m + sj];
+      Ac[idx] = {ldexp(gx.x, -s_exp), (i == j) ? 0.0 : ldexp(gx.y, -s_exp)};
+      Vc[idx] = {(i == j) ? 1.0 : 0.0, 0.0};
+    }
   }
-  __syncthreads();
+  cl.sync();                                       // (also: every CTA has read the handoff flag)
+  if (lead) {
 
   // ---- 1. cyclic Jacobi: A <- J^H A J, V <- V J, J = diag(1, e^{-i phi}) R
   //         with R the real rotation that zeroes |a_ij| (round-robin pairs,
   //         all disjoint pairs of a step at once)
   const int P2 = p + (p & 1);
   const int npairs = P2 / 2;
-  // the handoff of the embedded solve, if it passed its missed-eigenvalue check
-  const bool pre = a.cx_pre && reinterpret_cast<const double*>(At)[min(R, p)] == 1.0;
   for (int sweep = 0; !pre && sweep < kJacobiMaxSweeps; ++sweep) {
     double off = 0.0, tot = 0.0;
     for (int idx = tid; idx < p * p; idx += kCThreads) {
@@ -2048,42 +2065,54 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     }
   }
 
-  // ---- 1'. (cx_pre, check passed) the eigenpairs handed over by the real
-  //          df64 solver of the embedding: lambda_k at the start of the A~
-  //          array, x_k in the sorted-V array; the other diagonal entries sort
-  //          last, below the rank threshold
-  if (pre) {
-    const int K = min(R, p);
-    const double* lam_h = reinterpret_cast<const double*>(At);
-    for (int idx = tid; idx < p * p; idx += kCThreads) {
-      const int i = idx / p, k = idx - i * p;
-      Vc[idx] = (k < K) ? Vo[(int64_t)k * p + i] : C64d{(i == k) ? 1.0 : 0.0, 0.0};
-    }
-    for (int i = tid; i < p; i += kCThreads) Ac[(int64_t)i * p + i].re = (i < K) ? ldexp(lam_h[i], -s_exp) : -1.0;
-    __syncthreads();
+  // ---- 2. eigenvalues sorted descending, rank, sigma, V, vsi. The handoff's
+  //         (cx_pre, check passed) come sorted: lambda_k at the start of the A~
+  //         array, x_k in the sorted-V array.
+  const int np = pre ? min(R, p) : p;              // eigenvalues at hand
+  const double* lam_h = reinterpret_cast<const double*>(At);
+  for (int i = tid; i < np; i += kCThreads) {
+    lam_s[i] = pre ? ldexp(lam_h[i], -s_exp) : Ac[(int64_t)i * p + i].re;
+    ord[i] = i;
   }
-
-  // ---- 2. eigenvalues (real diagonal) sorted descending, rank, sigma, V, vsi
-  for (int i = tid; i < p; i += kCThreads) lam_s[i] = Ac[(int64_t)i * p + i].re;
   __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < p; ++i) ord[i] = i;
-    for (int i = 0; i < p; ++i) {
-      int best = i;
-      for (int q = i + 1; q < p; ++q)
-        if (lam_s[ord[q]] > lam_s[ord[best]]) best = q;
-      const int t = ord[i];
-      ord[i] = ord[best];
-      ord[best] = t;
+  if (warp == 0) {
+    // selection sort, descending: the first largest of the rest, by a warp reduction
+    for (int i = 0; !pre && i + 1 < np; ++i) {
+      double best = -INFINITY;
+      int at = np;
+      for (int q = i + lane; q < np; q += 32) {
+        const double v = lam_s[ord[q]];
+        if (at == np || v > best) {
+          best = v;
+          at = q;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, best, o);
+        const int vat = __shfl_xor_sync(0xffffffffu, at, o);
+        if (vat < np && (at == np || v > best || (!(best > v) && vat < at))) {
+          best = v;
+          at = vat;
+        }
+      }
+      if (lane == 0) {
+        const int t = ord[i];
+        ord[i] = ord[at];
+        ord[at] = t;
+      }
+      __syncwarp();
     }
-    const int rw = min(R, p);
-    int k = 0;
-    const double l0 = lam_s[ord[0]];
-    if (l0 > 0.0) {
-      const double thr = l0 * kRankRtol * (double)p * kEps;
-      while (k < rw && lam_s[ord[k]] > thr) ++k;
+    if (lane == 0) {
+      const int rw = min(R, p);
+      int k = 0;
+      const double l0 = lam_s[ord[0]];
+      if (l0 > 0.0) {
+        const double thr = l0 * kRankRtol * (double)p * kEps;
+        while (k < rw && lam_s[ord[k]] > thr) ++k;
+      }
+      sh_int[1] = k;
     }
-    sh_int[1] = k;
   }
   __syncthreads();
   const int re = sh_int[1];
@@ -2091,17 +2120,22 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     ws[L.sig + k] = (k < re) ? sqrt(ldexp(lam_s[ord[k]], s_exp)) : 0.0;
   for (int idx = tid; idx < R * p; idx += kCThreads) {
     const int k = idx / p, i = idx - k * p;
-    const C64d v = (k < re) ? Vc[(int64_t)i * p + ord[k]] : C64d{0.0, 0.0};
+    const C64d v = (k < re) ? (pre ? Vo[idx] : Vc[(int64_t)i * p + ord[k]]) : C64d{0.0, 0.0};
     Vo[idx] = v;
     const double inv = (k < re) ? 1.0 / sqrt(lam_s[ord[k]]) : 0.0;
     vsi[(int64_t)i * R + k] = {v.re * inv, v.im * inv};
   }
   __syncthreads();
 
-  // ---- 3. A~ = vsi^H (G_XY vsi)
-  for (int idx = tid; idx < p * re; idx += kCThreads) {
+  }
+  cl.sync();                                       // vsi is complete; the rank from CTA 0
+  const int re = cl.map_shared_rank(sh_int, 0)[1];
+
+  // ---- 3. A~ = vsi^H (G_XY vsi), entries over the cluster
+  for (int idx = rank * kCThreads + tid; idx < p * re; idx += kCxCtas * kCThreads) {
     const int i = idx / re, k = idx - i * re;
     C64d s = {0.0, 0.0};
+#pragma unroll 4
     for (int j = 0; j < p; ++j) {
       const C64d t = zmul(Bc[(int64_t)i * p + j], vsi[(int64_t)j * R + k]);
       s.re += t.re;
@@ -2109,15 +2143,16 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     }
     Ac[(int64_t)i * R + k] = s;                  // Y = G_XY vsi, p x re (stride R)
   }
-  __syncthreads();
+  cl.sync();
   CF* Hc = reinterpret_cast<CF*>(ws + L.lu);
   CF* Qc = Hc + re * re;
   CF* Wc = Qc + re * re;
   CF* Uc = Wc + re * re;
   CF* yc = Uc + re * re;
-  for (int idx = tid; idx < re * re; idx += kCThreads) {
+  for (int idx = rank * kCThreads + tid; idx < re * re; idx += kCxCtas * kCThreads) {
     const int k = idx / re, l = idx - k * re;
     C64d s = {0.0, 0.0};
+#pragma unroll 4
     for (int i = 0; i < p; ++i) {
       const C64d t = zcmul(vsi[(int64_t)i * R + k], Ac[(int64_t)i * R + l]);
       s.re += t.re;
@@ -2126,29 +2161,44 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     At[idx] = s;
     Hc[idx] = {(float)s.re, (float)s.im};
   }
-  __syncthreads();
+  cl.sync();
+  if (lead) {
 
   // ---- 4. eig(A~): FP32 complex Schur, then FP64 two-sided Rayleigh quotients
   if (warp == 0 && re > 0) {
     const bool ok = warp_schur32(Hc, Qc, yc, re, cs, sn);
     if (!ok && lane == 0) atomicOr(a.status, kDevRank);
-    warp_right32(Hc, Qc, Wc, yc, re);
-    warp_left32(Hc, Qc, Uc, yc, re);
+  }
+  __syncthreads();
+  // both vector sets at once: the left ones' scratch in A~'s array past A~
+  // when it fits
+  const bool two = 2 * (int64_t)re * re <= (int64_t)p * p;
+  if (re > 0) {
+    if (warp == 0) warp_right32(Hc, Qc, Wc, yc, re);
+    if (!two) __syncthreads();
+    if (warp == 1) warp_left32(Hc, Qc, Uc, two ? reinterpret_cast<CF*>(At + re * re) : yc, re);
   }
   __syncthreads();
   double* lam_tmp = ws + L.Y;
+  // the products A~ w_k, one (i, k) per thread (G_XY's array is free), then the quotients
+  C64d* aw = Bc;
+  for (int idx = tid; idx < re * re; idx += kCThreads) {
+    const int i = idx / re, k = idx - i * re;
+    C64d s = {0.0, 0.0};
+    for (int j = 0; j < re; ++j) {
+      const CF wj = Wc[j * re + k];
+      const C64d t = zmul(At[i * re + j], C64d{wj.re, wj.im});
+      s.re += t.re;
+      s.im += t.im;
+    }
+    aw[idx] = s;
+  }
+  __syncthreads();
   for (int k = tid; k < re; k += kCThreads) {
     C64d num = {0.0, 0.0}, den = {0.0, 0.0};
     for (int i = 0; i < re; ++i) {
-      C64d aw = {0.0, 0.0};
-      for (int j = 0; j < re; ++j) {
-        const CF wj = Wc[j * re + k];
-        const C64d t = zmul(At[i * re + j], C64d{wj.re, wj.im});
-        aw.re += t.re;
-        aw.im += t.im;
-      }
       const CF ui = Uc[i * re + k], wi = Wc[i * re + k];
-      const C64d un = zcmul(C64d{ui.re, ui.im}, aw);
+      const C64d un = zcmul(C64d{ui.re, ui.im}, aw[i * re + k]);
       const C64d ud = zcmul(C64d{ui.re, ui.im}, C64d{wi.re, wi.im});
       num.re += un.re;
       num.im += un.im;
@@ -2156,19 +2206,23 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
       den.im += ud.im;
     }
     const double q = den.re * den.re + den.im * den.im;
-    lam_tmp[2 * k] = (q > 0.0) ? (num.re * den.re + num.im * den.im) / q : 0.0;
-    lam_tmp[2 * k + 1] = (q > 0.0) ? (num.im * den.re - num.re * den.im) / q : 0.0;
+    const double lr = (q > 0.0) ? (num.re * den.re + num.im * den.im) / q : 0.0;
+    const double li = (q > 0.0) ? (num.im * den.re - num.re * den.im) / q : 0.0;
+    lam_tmp[2 * k] = lr;
+    lam_tmp[2 * k + 1] = li;
+    key_s[k] = lr * lr + li * li;
   }
   __syncthreads();
   if (tid == 0) {
+    const long long* ikey = reinterpret_cast<const long long*>(key_s);   // >= 0: ordered as their bits
     for (int k = 0; k < re; ++k) ord[k] = k;
     for (int k = 0; k < re; ++k) {
       int best = k;
       for (int q = k + 1; q < re; ++q) {
-        const double br = lam_tmp[2 * ord[best]], bi = lam_tmp[2 * ord[best] + 1];
-        const double qr = lam_tmp[2 * ord[q]], qi = lam_tmp[2 * ord[q] + 1];
-        const double mb = br * br + bi * bi, mq = qr * qr + qi * qi;
-        if (mq > mb || (mq == mb && atan2(qi, qr) < atan2(bi, br))) best = q;
+        const long long mb = ikey[ord[best]], mq = ikey[ord[q]];
+        if (mq > mb || (mq == mb && atan2(lam_tmp[2 * ord[q] + 1], lam_tmp[2 * ord[q]]) <
+                                        atan2(lam_tmp[2 * ord[best] + 1], lam_tmp[2 * ord[best]])))
+          best = q;
       }
       const int t = ord[k];
       ord[k] = ord[best];
@@ -2182,14 +2236,19 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
   }
   __syncthreads();
 
-  // ---- 5. M = vsi W, FP32 out in true units (vsi carries 2^{s/2})
+  }
+  cl.sync();                                       // W and the order, from CTA 0
+  const int* order = cl.map_shared_rank(ord, 0);
+
+  // ---- 5. M = vsi W, FP32 out in true units (vsi carries 2^{s/2}), entries
+  //         over the cluster
   float* Mf = reinterpret_cast<float*>(ws + L.Mf);
   const double unscale = exp2(-0.5 * s_exp);
-  for (int idx = tid; idx < p * R; idx += kCThreads) {
+  for (int idx = rank * kCThreads + tid; idx < p * R; idx += kCxCtas * kCThreads) {
     const int row = idx / R, k = idx - row * R;
     C64d s = {0.0, 0.0};
     if (k < re) {
-      const int kk = ord[k];
+      const int kk = order[k];
       for (int l = 0; l < re; ++l) {
         const CF wv = Wc[l * re + kk];
         const C64d t = zmul(vsi[(int64_t)row * R + l], C64d{wv.re, wv.im});
@@ -2200,6 +2259,8 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     Mf[2 * idx] = (float)(s.re * unscale);
     Mf[2 * idx + 1] = (float)(s.im * unscale);
   }
+  cl.sync();                                       // CTA 0's order has been read
+  if (!lead) return;
 
   // ---- 6. amplitudes b_k = u_k^H alpha_1 / (lambda_k u_k^H w_k), alpha_1[i] =
   //         sigma_i conj(V[0][i]); background index argmin |log lambda|
@@ -2231,17 +2292,19 @@ __global__ void __launch_bounds__(kCThreads, 1) modes_complex_kernel(ModesArgs a
     ws[L.bamp + 2 * k] = br;
     ws[L.bamp + 2 * k + 1] = bi;
   }
+  for (int k = tid - 32; k >= 0 && k < re; k += kCThreads - 32) {   // warps without an amplitude
+    const double lr = ws[L.lamout + 2 * k], li = ws[L.lamout + 2 * k + 1];
+    const double lm = 0.5 * log(lr * lr + li * li), th = atan2(li, lr);
+    key_s[k] = lm * lm + th * th;
+  }
   __syncthreads();
   if (tid == 0) {
     int best = -1;
     double bv = 0.0;
     for (int k = 0; k < re; ++k) {
-      const double lr = ws[L.lamout + 2 * k], li = ws[L.lamout + 2 * k + 1];
-      const double lm = 0.5 * log(lr * lr + li * li), th = atan2(li, lr);
-      const double v = lm * lm + th * th;
-      if (best < 0 || v < bv) {
+      if (best < 0 || key_s[k] < bv) {
         best = k;
-        bv = v;
+        bv = key_s[k];
       }
     }
     ws[L.bamp + 2 * (a.ws_m - 1 > 1 ? a.ws_m - 1 : 1)] = (double)best;
@@ -2385,8 +2448,17 @@ cudaError_t launch_modes_batch(const ModesBatch& b, cudaStream_t st) {
 
 cudaError_t launch_modes_complex(const ModesArgs& a, cudaStream_t st) {
   if (a.c - 1 > SDMD_MAX_M - 1) return cudaErrorNotSupported;
-  modes_complex_kernel<<<1, kCThreads, 0, st>>>(a, modes_layout(a.ws_m));
-  return cudaGetLastError();
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kCxCtas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCxCtas);
+  cfg.blockDim = dim3(kCThreads);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, modes_complex_kernel, a, modes_layout(a.ws_m));
 }
 
 }  // namespace sdmd
