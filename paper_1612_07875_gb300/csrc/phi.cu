@@ -4,12 +4,18 @@
 // matrix produced by the FP64 kernel, rounded to FP32 here.
 //
 // A CTA owns a tile of kPos positions and streams the p slots of X' through
-// shared memory in chunks of kSlots slots with cp.async double buffering
-// (each chunk row is kPos contiguous elements of one slot: 16-byte copies,
-// fully coalesced). Each thread owns kPos / 256 positions and KT modes and
-// accumulates 2*KT FP32 sums per position against M broadcast from shared
-// memory; gridDim.y tiles the modes. Columns beyond the kept rank have M = 0
-// and come out as zeros.
+// shared memory in 32 KiB stages of kSlots slots (each row kPos contiguous
+// elements of one slot, 16-byte cp.async copies), three stages in a ring, one
+// block barrier per stage. Each thread owns kPer positions (groups of
+// consecutive ones) and KT modes and accumulates kPer x KT sums (2 x for
+// complex modes) against M broadcast from shared memory; gridDim.y tiles the
+// modes. Columns beyond the kept rank have M = 0 and come out as zeros.
+//
+// What bounds it: a slot's row of M is read once per thread whatever kPer, so
+// with one position per thread (two for uint8) the broadcasts took as many
+// shared-memory cycles as the FMAs; four positions (eight for uint8) leave the
+// FMA pipe (FP32 modes, r = 10: 20 FP32 cycles per 512 bytes against 23 of
+// HBM time). Every sum is taken slot by slot, as before.
 //
 // The same kernel with a real p x r matrix and real output, reading X
 // (columns 0..c-2) instead of X', gives the POD modes U = X V Sigma^-1
@@ -26,23 +32,26 @@ namespace {
 
 constexpr int kPhiThreads = 256;
 
-template <typename T>
+// positions per thread: kGrp groups of kVec consecutive ones, at most 80 sums
+template <typename T, bool kReal, int KT>
 struct PhiTraits;
-template <>
-struct PhiTraits<uint8_t> {
-  static constexpr int kPos = 512;  // positions per tile (2 per thread)
-  static constexpr int kSlots = 32; // slots per staged chunk
+template <bool kReal, int KT>
+struct PhiTraits<uint8_t, kReal, KT> {
+  static constexpr int kVec = (kReal || KT <= 10) ? 4 : 2;
+  static constexpr int kGrp = (kReal && KT <= 10) ? 2 : 1;
 };
-template <>
-struct PhiTraits<float> {
-  static constexpr int kPos = 256;  // positions per tile (1 per thread)
-  static constexpr int kSlots = 32;
+template <bool kReal, int KT>
+struct PhiTraits<float, kReal, KT> {
+  static constexpr int kVec = (kReal || KT <= 10) ? 4 : 2;
+  static constexpr int kGrp = 1;
 };
-template <>
-struct PhiTraits<float2> {          // complex64 (re, im)
-  static constexpr int kPos = 256;
-  static constexpr int kSlots = 16; // 2 x 16 x 2 KB staged: two CTAs per SM
+template <int KT>
+struct PhiTraits<float2, false, KT> {            // complex64 (re, im)
+  static constexpr int kVec = 2;
+  static constexpr int kGrp = 1;
 };
+constexpr int kStageBytes = 32768;
+constexpr int kStages = 3;
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -50,37 +59,36 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_le1() { asm volatile("cp.async.wait_group 1;\n" ::); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
 
-// Stage slots [a0, a0 + ns) of the position tile starting at i0 (elements).
-template <typename T>
-__device__ __forceinline__ void stage_chunk(const PhiArgs& a, uint8_t* buf, int a0, int ns, int64_t i0) {
-  constexpr int kPos = PhiTraits<T>::kPos;
-  constexpr int kRowBytes = kPos * (int)sizeof(T);
-  constexpr int kVec = kRowBytes / 16;
-  for (int idx = threadIdx.x; idx < ns * kVec; idx += kPhiThreads) {
-    const int s = idx / kVec, v = idx - s * kVec;
-    const int slot = (a.start + a.xoff + a0 + s) % a.m;
-    const uint8_t* src = a.ring + (int64_t)slot * a.slot_bytes + i0 * (int64_t)sizeof(T) + 16 * v;
-    cp_async16(buf + s * kRowBytes + 16 * v, src);
+// Stage slots [a0, a0 + ns) of the position tile starting at byte b0.
+template <int kRowBytes>
+__device__ __forceinline__ void stage_chunk(const PhiArgs& a, uint8_t* buf, int a0, int ns, int64_t b0) {
+  constexpr int kVecs = kRowBytes / 16;
+  for (int idx = threadIdx.x; idx < ns * kVecs; idx += kPhiThreads) {
+    const int s = idx / kVecs, v = idx - s * kVecs;
+    int slot = a.start + a.xoff + a0 + s;
+    if (slot >= a.m) slot -= a.m;
+    cp_async16(buf + s * kRowBytes + 16 * v, a.ring + (int64_t)slot * a.slot_bytes + b0 + 16 * v);
   }
 }
 
 template <typename T, int KT, bool kReal>
 __global__ void __launch_bounds__(kPhiThreads, 2) phi_tile_kernel(PhiArgs a) {
-  constexpr int kPos = PhiTraits<T>::kPos;
-  constexpr int kPer = kPos / kPhiThreads;               // positions per thread
-  constexpr int kRowBytes = kPos * (int)sizeof(T);
+  constexpr bool kCx = sizeof(T) == 8;                   // complex snapshots
+  constexpr int kVec = PhiTraits<T, kReal, KT>::kVec, kGrp = PhiTraits<T, kReal, KT>::kGrp;
+  constexpr int kPer = kVec * kGrp;                      // positions per thread
+  constexpr int kPos = kPer * kPhiThreads;               // positions per tile
+  constexpr int kRowBytes = kPos * (int)sizeof(T);       // at most 4096: slots are padded to 4 KiB
+  static_assert(kRowBytes <= 4096 && 4096 % kRowBytes == 0, "a tile's row stays within the padded slot");
+  constexpr int kSlots = kStageBytes / kRowBytes;
   constexpr int kW = kReal ? KT : 2 * KT;                // sums per position
-  constexpr int kSlots = PhiTraits<T>::kSlots;
+  constexpr int kWp = (kW + 3) & ~3;                     // row of M, padded to 16 bytes
   extern __shared__ __align__(16) uint8_t smem[];
-  uint8_t* buf0 = smem;
-  uint8_t* buf1 = smem + kSlots * kRowBytes;
-  float* Ms = reinterpret_cast<float*>(smem + 2 * kSlots * kRowBytes);   // p x kW
+  float* Ms = reinterpret_cast<float*>(smem + kStages * kStageBytes);   // p x kWp
   const int k0 = blockIdx.y * KT;
   const int kt = min(KT, a.r - k0);
-  for (int idx = threadIdx.x; idx < a.p * kW; idx += kPhiThreads) {
-    const int row = idx / kW, q = idx - row * kW;
+  for (int idx = threadIdx.x; idx < a.p * kWp; idx += kPhiThreads) {
+    const int row = idx / kWp, q = idx - row * kWp;
     if constexpr (kReal)
       Ms[idx] = (q < kt) ? a.Mf[(int64_t)row * a.r + k0 + q] : 0.f;
     else
@@ -88,94 +96,120 @@ __global__ void __launch_bounds__(kPhiThreads, 2) phi_tile_kernel(PhiArgs a) {
   }
   const int64_t ntiles = (a.n + kPos - 1) / kPos;
   const int nchunks = (a.p + kSlots - 1) / kSlots;
+  // stage sequence over the tiles of this CTA: chunk c of tile blockIdx.x + i gridDim.x
+  int64_t ld_tile = blockIdx.x;
+  int ld_c = 0, ld_buf = 0;
+  auto load_next = [&]() {
+    if (ld_tile < ntiles) {
+      stage_chunk<kRowBytes>(a, smem + ld_buf * kStageBytes, ld_c * kSlots, min(kSlots, a.p - ld_c * kSlots),
+                             ld_tile * kRowBytes);
+      if (++ld_c == nchunks) {
+        ld_c = 0;
+        ld_tile += gridDim.x;
+      }
+    }
+    cp_async_commit();                                   // one group per stage, empty past the end
+    ld_buf = (ld_buf + 1 == kStages) ? 0 : ld_buf + 1;
+  };
+  load_next();
+  load_next();
+  int buf = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t i0 = tile * kPos;
     float acc[kPer][kW];
 #pragma unroll
     for (int u = 0; u < kPer; ++u)
 #pragma unroll
       for (int q = 0; q < kW; ++q) acc[u][q] = 0.f;
-    __syncthreads();   // previous tile's buffers are free
-    stage_chunk<T>(a, buf0, 0, min(kSlots, a.p), i0);
-    cp_async_commit();
     for (int c = 0; c < nchunks; ++c) {
-      uint8_t* cur = (c & 1) ? buf1 : buf0;
-      uint8_t* nxt = (c & 1) ? buf0 : buf1;
-      const int a0 = c * kSlots;
-      const int ns = min(kSlots, a.p - a0);
-      if (c + 1 < nchunks) {
-        stage_chunk<T>(a, nxt, a0 + kSlots, min(kSlots, a.p - a0 - kSlots), i0);
-        cp_async_commit();
-        cp_async_wait_le1();
-      } else {
-        cp_async_wait_all();
-      }
-      __syncthreads();
-      for (int s = 0; s < ns; ++s) {
-        if constexpr (sizeof(T) == 8) {   // complex64: phi += x m, 4 FMAs per mode
-          const float2 xc = *reinterpret_cast<const float2*>(cur + s * kRowBytes + 8 * threadIdx.x);
-          const float4* mrow = reinterpret_cast<const float4*>(Ms + (a0 + s) * kW);
+      cp_async_wait_le1();                               // this thread's copies of the stage have landed
+      __syncthreads();                                   // ... everyone's; and the stage before is free
+      load_next();
+      const uint8_t* cur = smem + buf * kStageBytes;
+      buf = (buf + 1 == kStages) ? 0 : buf + 1;
+      const int ns = min(kSlots, a.p - c * kSlots);
+      const float* mrow = Ms + c * kSlots * kWp;
+#pragma unroll 2
+      for (int s = 0; s < ns; ++s, cur += kRowBytes, mrow += kWp) {
+        float m[kWp];
 #pragma unroll
-          for (int q2 = 0; q2 < KT / 2; ++q2) {
-            const float4 mv = mrow[q2];            // modes 2 q2 and 2 q2 + 1: (re, im, re, im)
-            acc[0][4 * q2 + 0] = fmaf(-xc.y, mv.y, fmaf(xc.x, mv.x, acc[0][4 * q2 + 0]));
-            acc[0][4 * q2 + 1] = fmaf(xc.y, mv.x, fmaf(xc.x, mv.y, acc[0][4 * q2 + 1]));
-            acc[0][4 * q2 + 2] = fmaf(-xc.y, mv.w, fmaf(xc.x, mv.z, acc[0][4 * q2 + 2]));
-            acc[0][4 * q2 + 3] = fmaf(xc.y, mv.z, fmaf(xc.x, mv.w, acc[0][4 * q2 + 3]));
-          }
-          continue;
+        for (int q = 0; q < kWp; q += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(mrow + q);
+          m[q] = v.x;
+          m[q + 1] = v.y;
+          m[q + 2] = v.z;
+          m[q + 3] = v.w;
         }
-        float x[kPer];
-        if constexpr (sizeof(T) == 1) {
-          const unsigned short v = *reinterpret_cast<const unsigned short*>(cur + s * kRowBytes + 2 * threadIdx.x);
-          x[0] = (float)(v & 0xffu);
-          x[1] = (float)(v >> 8);
+        if constexpr (kCx) {                             // complex64: phi += x m, 4 FMAs per mode
+          const float4 v = *reinterpret_cast<const float4*>(cur + 16 * threadIdx.x);
+          const float xr[2] = {v.x, v.z}, xi[2] = {v.y, v.w};
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int q = 0; q < KT; ++q) {
+              acc[u][2 * q] = fmaf(-xi[u], m[2 * q + 1], fmaf(xr[u], m[2 * q], acc[u][2 * q]));
+              acc[u][2 * q + 1] = fmaf(xi[u], m[2 * q], fmaf(xr[u], m[2 * q + 1], acc[u][2 * q + 1]));
+            }
         } else {
-          x[0] = *reinterpret_cast<const float*>(cur + s * kRowBytes + 4 * threadIdx.x);
-        }
-        if constexpr (kReal) {
-          const float2* mrow = reinterpret_cast<const float2*>(Ms + (a0 + s) * kW);
+          float x[kPer];
 #pragma unroll
-          for (int q2 = 0; q2 < KT / 2; ++q2) {
-            const float2 mv = mrow[q2];
+          for (int g = 0; g < kGrp; ++g) {
+            if constexpr (sizeof(T) == 1) {
+              const uint8_t* at = cur + kVec * (threadIdx.x + kPhiThreads * g);
+              unsigned v;
+              if constexpr (kVec == 4) v = *reinterpret_cast<const unsigned*>(at);
+              else v = *reinterpret_cast<const unsigned short*>(at);
 #pragma unroll
-            for (int u = 0; u < kPer; ++u) {
-              acc[u][2 * q2 + 0] = fmaf(x[u], mv.x, acc[u][2 * q2 + 0]);
-              acc[u][2 * q2 + 1] = fmaf(x[u], mv.y, acc[u][2 * q2 + 1]);
+              for (int b = 0; b < kVec; ++b)             // 0x4B0000bb = 2^23 + byte, exact
+                x[kVec * g + b] = __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7650u | (unsigned)b)) - 8388608.f;
+            } else if constexpr (kVec == 4) {
+              const float4 v = *reinterpret_cast<const float4*>(cur + 16 * threadIdx.x);
+              x[0] = v.x;
+              x[1] = v.y;
+              x[2] = v.z;
+              x[3] = v.w;
+            } else {
+              const float2 v = *reinterpret_cast<const float2*>(cur + 8 * threadIdx.x);
+              x[0] = v.x;
+              x[1] = v.y;
             }
           }
-        } else {
-          const float4* mrow = reinterpret_cast<const float4*>(Ms + (a0 + s) * kW);
 #pragma unroll
-          for (int q4 = 0; q4 < KT / 2; ++q4) {
-            const float4 mv = mrow[q4];
+          for (int u = 0; u < kPer; ++u)
 #pragma unroll
-            for (int u = 0; u < kPer; ++u) {
-              acc[u][4 * q4 + 0] = fmaf(x[u], mv.x, acc[u][4 * q4 + 0]);
-              acc[u][4 * q4 + 1] = fmaf(x[u], mv.y, acc[u][4 * q4 + 1]);
-              acc[u][4 * q4 + 2] = fmaf(x[u], mv.z, acc[u][4 * q4 + 2]);
-              acc[u][4 * q4 + 3] = fmaf(x[u], mv.w, acc[u][4 * q4 + 3]);
-            }
-          }
+            for (int q = 0; q < kW; ++q) acc[u][q] = fmaf(x[u], m[q], acc[u][q]);
         }
       }
-      __syncthreads();   // `cur` may be overwritten by the next stage
     }
-    // write: mode k, positions i0 + kPer*tid + u (complex64, or FP32 when real)
-    const int64_t ibase = i0 + (int64_t)kPer * threadIdx.x;
+    // write: mode k, groups of kVec positions (complex64, or FP32 when real),
+    // 16 bytes at a time where the column allows it
 #pragma unroll
-    for (int q = 0; q < KT; ++q) {
-      if (q < kt) {
+    for (int g = 0; g < kGrp; ++g) {
+      const int64_t i0 = tile * kPos + (int64_t)kVec * (threadIdx.x + kPhiThreads * g);
+#pragma unroll
+      for (int q = 0; q < KT; ++q) {
+        if (q >= kt) continue;
         if constexpr (kReal) {
-          float* col = a.phi + (int64_t)(k0 + q) * a.n;
+          float* o = a.phi + (int64_t)(k0 + q) * a.n + i0;
+          if (i0 + kVec <= a.n && (reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
+            *reinterpret_cast<float4*>(o) = make_float4(acc[kVec * g][q], acc[kVec * g + 1][q],
+                                                        acc[kVec * g + 2][q], acc[kVec * g + 3][q]);
+          } else {
 #pragma unroll
-          for (int u = 0; u < kPer; ++u)
-            if (ibase + u < a.n) col[ibase + u] = acc[u][q];
+            for (int u = 0; u < kVec; ++u)
+              if (i0 + u < a.n) o[u] = acc[kVec * g + u][q];
+          }
         } else {
-          float2* col = reinterpret_cast<float2*>(a.phi) + (int64_t)(k0 + q) * a.n;
+          float2* o = reinterpret_cast<float2*>(a.phi) + (int64_t)(k0 + q) * a.n + i0;
+          if (i0 + kVec <= a.n && (reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
 #pragma unroll
-          for (int u = 0; u < kPer; ++u)
-            if (ibase + u < a.n) col[ibase + u] = make_float2(acc[u][2 * q], acc[u][2 * q + 1]);
+            for (int u = 0; u < kVec; u += 2)
+              *reinterpret_cast<float4*>(o + u) = make_float4(acc[kVec * g + u][2 * q], acc[kVec * g + u][2 * q + 1],
+                                                              acc[kVec * g + u + 1][2 * q], acc[kVec * g + u + 1][2 * q + 1]);
+          } else {
+#pragma unroll
+            for (int u = 0; u < kVec; ++u)
+              if (i0 + u < a.n) o[u] = make_float2(acc[kVec * g + u][2 * q], acc[kVec * g + u][2 * q + 1]);
+          }
         }
       }
     }
@@ -184,9 +218,9 @@ __global__ void __launch_bounds__(kPhiThreads, 2) phi_tile_kernel(PhiArgs a) {
 
 template <typename T, int KT, bool kReal>
 cudaError_t launch_t(const PhiArgs& a, cudaStream_t st, int sms) {
-  constexpr int kPos = PhiTraits<T>::kPos;
-  constexpr int kSlots = PhiTraits<T>::kSlots;
-  const size_t smem = 2 * kSlots * kPos * sizeof(T) + (size_t)a.p * (kReal ? KT : 2 * KT) * sizeof(float);
+  constexpr int kPos = PhiTraits<T, kReal, KT>::kVec * PhiTraits<T, kReal, KT>::kGrp * kPhiThreads;
+  constexpr int kWp = ((kReal ? KT : 2 * KT) + 3) & ~3;
+  const size_t smem = kStages * kStageBytes + (size_t)a.p * kWp * sizeof(float);
   {
     const cudaError_t e = smem_optin(reinterpret_cast<const void*>(phi_tile_kernel<T, KT, kReal>), smem);
     if (e != cudaSuccess) return e;
