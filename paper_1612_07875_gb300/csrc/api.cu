@@ -1359,6 +1359,7 @@ int sdmd_modes(sdmd_t h, int32_t r, void* phi, void* lambda, int32_t* r_out, voi
   a.ws = h->ws;
   a.status = h->status;
   a.r_dev = h->r_dev;
+  a.spread = 1;
   {
     TraceScope ts(h, SDMD_K_MODES, st);
     if (cplx) {

@@ -1252,7 +1252,7 @@ struct SmemPlan {
 constexpr int64_t kSmemDynUnits = (216 * 1024) / 8;
 constexpr int kEigUnits = 8;   // H, Q, W, U, two y (complex float) and the products A~ w (two df64) per r x r
 
-__host__ __device__ inline SmemPlan smem_plan(int p, int r) {
+__host__ __device__ inline SmemPlan smem_plan(int p, int r, int cl) {
   SmemPlan s;
   s.P = (p + 3) & ~3;
   // d, e, rn, pv (two: provisional eigenvalues), lam (df64) + d32, e2_32 (float) + 32 df64 scalars
@@ -1260,7 +1260,7 @@ __host__ __device__ inline SmemPlan smem_plan(int p, int r) {
   s.rr_dim = (r + kClusterExt < p) ? r + kClusterExt : p;
   s.rr_in_smem = (s.rr_dim <= kRRMax);
   s.rr_units = s.rr_in_smem ? 2 * (int64_t)s.rr_dim * s.rr_dim : 0;
-  s.cl = (p <= kSmemMaxP) ? 1 : kClusterCtas;
+  s.cl = cl;
   const int64_t room = kSmemDynUnits - s.vec_units - s.rr_units;
   const int64_t rows = s.cl == 1 ? p : 2 * ((p + 7) / 8);
   const int64_t tri = rows * p + tri_units(s.P, s.cl);
@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   // embed_cx: the 2pc x 2pc real embedding of a complex pc x pc G_X
   const int m = a.m, pc = a.c - 1, p = a.embed_cx ? 2 * pc : pc;
   const int rw = min(a.r_req, p);
-  const SmemPlan plan = smem_plan(p, a.r_req);
+  const SmemPlan plan = smem_plan(p, a.r_req, kCl);
   const int64_t P = plan.P;
   dd* base = reinterpret_cast<dd*>(smem_d);
   dd* d = base;
@@ -1340,8 +1340,10 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   const int s_exp = sh_int[0];
   // complex G_X = B0 + i B1 embedded as [[B0, -B1], [B1, B0]] (symmetric:
   // G_X is Hermitian, its diagonal imaginary parts taken as zero)
-  for (int idx = tid; a.embed_cx && idx < p * p; idx += kThreads) {
-    const int i = idx / p, j = idx - i * p;
+  const int nrows = kCl > 1 ? (p >> 3) * 2 + min(max((p & 7) - 2 * rank, 0), 2) : p;   // stored rows of this CTA
+  for (int idx = tid; a.embed_cx && idx < nrows * p; idx += kThreads) {
+    const int li = idx / p, j = idx - li * p;
+    const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
     const int bi = i >= pc, bj = j >= pc, ii = i - bi * pc, jj = j - bj * pc;
     const double2 g = static_cast<const double2*>(a.G)[(int64_t)((a.start + ii) % m) * m + (a.start + jj) % m];
     const double v = (bi == bj) ? g.x : ((ii == jj) ? 0.0 : (bi ? g.y : -g.y));
@@ -1355,7 +1357,6 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   // 6 reads it with consecutive rows over the lanes. A cluster's CTA takes the
   // rows it owns.
   constexpr int kGatherBatch = 4;
-  const int nrows = kCl > 1 ? (p >> 3) * 2 + min(max((p & 7) - 2 * rank, 0), 2) : p;   // stored rows of this CTA
   for (int li = warp; !a.embed_cx && li < nrows; li += kWarps) {
     const int i = kCl > 1 ? (li >> 1) * 8 + 2 * rank + (li & 1) : li;
     int si = a.start + i;
@@ -1391,7 +1392,8 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
 
   // ---- 1. tridiagonalise G_X (df64)
   if constexpr (kCl > 1) {
-    tridiagonalize<kCl, 8>(A, p, d, e, tri_ws, plan.P, HV);
+    if (p <= 128) tridiagonalize<kCl, 4>(A, p, d, e, tri_ws, plan.P, HV);
+    else tridiagonalize<kCl, 8>(A, p, d, e, tri_ws, plan.P, HV);
   } else {
     if (p <= 32) tridiagonalize<1, 1>(A, p, d, e, tri_ws, plan.P, HV);
     else if (p <= 64) tridiagonalize<1, 2>(A, p, d, e, tri_ws, plan.P, HV);
@@ -1869,8 +1871,9 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   }
 }
 
-// Windows of p <= kSmemMaxP snapshot pairs: one CTA; longer ones: a cluster of
-// kClusterCtas (blockIdx.x / kClusterCtas is the job).
+// Windows of p <= kSmemMaxP snapshot pairs: one CTA; longer ones, and those of
+// at least kSpreadP pairs in a call that waits for one eigensolver: a cluster
+// of kClusterCtas (blockIdx.x / kClusterCtas is the job).
 template <int kCl>
 __global__ void __launch_bounds__(kThreads, 1) modes_small_kernel(ModesArgs a, ModesLayout L) {
   modes_small_body<kCl>(a, L);
@@ -2373,14 +2376,23 @@ bool modes_embed_ok(int c, int r) {
   return (int64_t)rr * 6 * p <= 6 * pp + 64 && (int64_t)rr * p <= pp;
 }
 
+// CTAs of one eigensolver. Alone, a window of kSpreadP pairs or more is faster
+// over a cluster: the trailing updates, bound by one SM's FP32 rate, split four
+// ways for one cluster barrier a step.
+constexpr int kSpreadP = 64;
+static int modes_ctas(const ModesArgs& a) {
+  const int p = a.embed_cx ? 2 * (a.c - 1) : a.c - 1;
+  return p > kSmemMaxP || (a.spread && p >= kSpreadP) ? kClusterCtas : 1;
+}
+
 static size_t modes_smem_bytes(const ModesArgs& a) {
-  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req);
+  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req, modes_ctas(a));
   return (size_t)(plan.vec_units + plan.rr_units + plan.pool_units) * 8;
 }
 
 cudaError_t launch_modes_small(const ModesArgs& a, cudaStream_t st) {
   const size_t bytes = modes_smem_bytes(a);
-  const bool cluster = !a.embed_cx && a.c - 1 > kSmemMaxP;
+  const bool cluster = modes_ctas(a) > 1;
   const void* f = cluster ? reinterpret_cast<const void*>(modes_small_kernel<kClusterCtas>)
                           : reinterpret_cast<const void*>(modes_small_kernel<1>);
   const cudaError_t e = smem_optin(f, bytes);

@@ -238,8 +238,12 @@ cudaError_t launch_t(const PhiArgs& a, cudaStream_t st, int sms) {
 
 template <typename T, bool kReal>
 cudaError_t launch_for_type(const PhiArgs& a, cudaStream_t st, int sms) {
-  // modes per pass: the smallest even tile >= r, at most 16
-  const int kt = a.r >= 16 ? 16 : ((a.r + 1) / 2) * 2;
+  // modes per pass: the smallest even tile >= r, at most 16; fewer while the
+  // position tiles (about 1024 positions) leave half of the SMs idle (a 64 x
+  // 64 field, r = 10: four CTAs 11 us)
+  int kt = a.r >= 16 ? 16 : ((a.r + 1) / 2) * 2;
+  const int64_t tiles = (a.n + 1023) / 1024;
+  while (kt > 2 && 2 * tiles * ((a.r + kt - 1) / kt) < sms) kt -= 2;
   switch (kt) {
     case 2: return launch_t<T, 2, kReal>(a, st, sms);
     case 4: return launch_t<T, 4, kReal>(a, st, sms);

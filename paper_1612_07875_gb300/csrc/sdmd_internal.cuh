@@ -197,6 +197,10 @@ struct ModesArgs {
   // kernel take them instead of running its Jacobi sweeps.
   int32_t embed_cx = 0;
   int32_t cx_pre = 0;
+  // 1: the call waits for this one eigensolver, so windows of some length take
+  // a cluster's SMs for it; 0: it runs beside other work and keeps to one SM
+  // where its G_X fits one
+  int32_t spread = 0;
 };
 
 // Doubles of workspace needed by the modes kernel for window length m.
