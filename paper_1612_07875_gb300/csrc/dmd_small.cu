@@ -490,7 +490,7 @@ __device__ int sturm_below_dd(const dd* __restrict__ d, const dd* __restrict__ e
 // ---------------------------------------------------------------- phase 3 --
 // LU with partial pivoting of the df64 tridiagonal T - mu I. Row i of U has
 // (1/u0, u1, u2) on columns (i, i+1, i+2) (diagonal stored as reciprocal);
-// mult / piv (0 or 1) describe L. Pivots below `tiny` are raised to it.
+// mult / piv (0 or 1, a byte) describe L. Pivots below `tiny` are raised to it.
 // Branch-free (selects), so the lanes of a warp that factor different shifts
 // never diverge.
 // b is eliminated forward on the way (the first solve's forward pass: its
@@ -500,8 +500,8 @@ __device__ int sturm_below_dd(const dd* __restrict__ d, const dd* __restrict__ e
 // warp would otherwise wait for each of them in turn.
 __device__ __forceinline__ void tri_lu_forward_dd(const dd* __restrict__ d, const dd* __restrict__ e, int p, dd mu,
                                                   float tiny, dd* __restrict__ u0, dd* __restrict__ u1,
-                                                  dd* __restrict__ u2, dd* __restrict__ mult, dd* __restrict__ piv,
-                                                  dd* __restrict__ b) {
+                                                  dd* __restrict__ u2, dd* __restrict__ mult,
+                                                  unsigned char* __restrict__ piv, dd* __restrict__ b) {
   const dd zero = {0.f, 0.f};
   dd cd = dd_sub(d[0], mu), c1 = (p > 1) ? e[0] : zero;
   dd bi = b[0];
@@ -524,7 +524,7 @@ __device__ __forceinline__ void tri_lu_forward_dd(const dd* __restrict__ d, cons
     u0[i] = rp;
     u1[i] = dd_sel(sw, nd, c1);
     u2[i] = dd_sel(sw, n1, zero);
-    piv[i] = {sw ? 1.f : 0.f, 0.f};
+    piv[i] = sw ? 1 : 0;
     mult[i] = m;
     const dd keep = dd_sel(sw, bn, bi), elim = dd_sel(sw, bi, bn);
     b[i] = keep;
@@ -544,15 +544,15 @@ __device__ __forceinline__ void tri_lu_forward_dd(const dd* __restrict__ d, cons
   b[p - 1] = bi;
 }
 
-__device__ __forceinline__ void tri_forward_dd(int p, const dd* __restrict__ mult, const dd* __restrict__ piv,
-                                               dd* __restrict__ b) {
+__device__ __forceinline__ void tri_forward_dd(int p, const dd* __restrict__ mult,
+                                               const unsigned char* __restrict__ piv, dd* __restrict__ b) {
   dd bi = b[0];
   dd bn = b[p > 1 ? 1 : 0], m = mult[0];
-  bool sw = p > 1 && piv[0].hi != 0.f;
+  bool sw = p > 1 && piv[0] != 0;
   for (int i = 0; i + 1 < p; ++i) {   // branch-free: b_i is carried in registers
     const int nx = (i + 2 < p) ? i + 2 : i + 1;
     const dd bnn = b[nx], mn = mult[nx - 1];
-    const bool swn = piv[nx - 1].hi != 0.f;
+    const bool swn = piv[nx - 1] != 0;
     const dd keep = dd_sel(sw, bn, bi), elim = dd_sel(sw, bi, bn);
     b[i] = keep;
     bi = dd_sub(elim, dd_mul(m, keep));
@@ -1236,7 +1236,7 @@ __device__ void warp_left32(const CF* H, const CF* Q, CF* U, CF* ycol, int r) {
 // Shared-memory plan (dynamic), in 8-byte units: the vectors, the
 // Rayleigh-Ritz matrices, and a pool that the phases use one after another:
 //   1     A (or this CTA's rows of it) and the tridiagonalisation's workspace
-//   3, 4  LU factors (5p per vector; Ritz scratch in the same place) and the
+//   3, 4  LU factors (about 4p per vector; Ritz scratch in the same place) and the
 //         vectors Z, which stay; the recurrences are chains of dependent
 //         loads and stores, so they belong on chip when they fit
 //   6..9  behind Z: G_XY vsi, A~, the small eigenproblem, G_XY transposed
@@ -1250,6 +1250,10 @@ struct SmemPlan {
 // Dynamic shared memory the plan may use (8-byte units): the SM's 227 KiB
 // less the kernel's static arrays, with margin.
 constexpr int64_t kSmemDynUnits = (216 * 1024) / 8;
+// LU factors of one vector: 1 / u0, u1, u2, multipliers (p each), the row swaps
+// (bytes). 4 1/8 p units and not 5 p, so 20 vectors of 255 pairs fit the pool:
+// 64 calls of 255 pairs together 6678 us, 7184 us with their LU off chip.
+__host__ __device__ constexpr int lu_units(int p) { return 4 * p + (p + 7) / 8; }
 constexpr int kEigUnits = 8;   // H, Q, W, U, two y (complex float) and the products A~ w (two df64) per r x r
 
 __host__ __device__ inline SmemPlan smem_plan(int p, int r, int cl) {
@@ -1264,7 +1268,7 @@ __host__ __device__ inline SmemPlan smem_plan(int p, int r, int cl) {
   const int64_t room = kSmemDynUnits - s.vec_units - s.rr_units;
   const int64_t rows = s.cl == 1 ? p : 2 * ((p + 7) / 8);
   const int64_t tri = rows * p + tri_units(s.P, s.cl);
-  const int64_t inv = (int64_t)s.rr_dim * 6 * p;
+  const int64_t inv = (int64_t)s.rr_dim * (lu_units(p) + p);
   const int64_t small = (int64_t)s.rr_dim * p + (int64_t)r * p + (1 + kEigUnits) * (int64_t)r * r + (int64_t)p * p;
   s.pool_units = tri;
   if (inv > s.pool_units) s.pool_units = inv < room ? inv : room;
@@ -1482,8 +1486,8 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
   const int rwe = (rw > 0) ? sh_int[2] : 0;
   for (int i = tid; i < rwe; i += kThreads) pv[i] = lam[i];   // the FP32 values, for phase 3'
   // inverse iteration: the vectors Z (later the eigenvectors, then vsi) and
-  // LU factors (5p per vector; the Ritz scratch takes their place)
-  const bool inv_in_smem = (int64_t)rwe * 6 * p <= plan.pool_units;
+  // LU factors (the Ritz scratch takes their place)
+  const bool inv_in_smem = (int64_t)rwe * (lu_units(p) + p) <= plan.pool_units;
   dd* Z = inv_in_smem ? pool : w.Z;
   if (tid == 0) w.clk[3] = clock64();
 
@@ -1554,15 +1558,16 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
         // vector i on lane i / 16 of warp i % 16: the factorisations and solves
         // are serial recurrences, so they are spread over all warps' issue slots
         for (int i = warp + kWarps * lane; i < rwe; i += kThreads) {
-          dd* u0 = LU + (int64_t)i * 5 * p;
+          dd* u0 = LU + (int64_t)i * lu_units(p);
+          unsigned char* piv = reinterpret_cast<unsigned char*>(u0 + 4 * p);
           dd* z = Z + (int64_t)i * p;
           if (it == 0) {
             dd shift = lam[i];
             for (int q = 0; q < i; ++q)    // (numerically) equal shifts: separate them slightly
               if (fabsf(lam[q].hi - shift.hi) <= sep) shift = dd_sub(shift, dd_make(sep));
-            tri_lu_forward_dd(d, e, p, shift, tiny, u0, u0 + p, u0 + 2 * p, u0 + 3 * p, u0 + 4 * p, z);
+            tri_lu_forward_dd(d, e, p, shift, tiny, u0, u0 + p, u0 + 2 * p, u0 + 3 * p, piv, z);
           } else {
-            tri_forward_dd(p, u0 + 3 * p, u0 + 4 * p, z);
+            tri_forward_dd(p, u0 + 3 * p, piv, z);
           }
           tri_backward_dd(p, u0, u0 + p, u0 + 2 * p, z);
         }
