@@ -527,8 +527,9 @@ SDMD_API int sdmd_modes_phase_cycles(sdmd_t h, int64_t *cycles, int32_t count, v
 /*
  * sdmd_modes_many -- the small algebra of exact DMD (as sdmd_modes, Sec. 2.2,
  * Eqs. 7-8; Algorithm 2: eig of G_X, rank, sigma, V, A~, eig(A~), the
- * amplitudes) for `count` <= 64 real dense handles in one launch, one CTA per
- * handle, each on its own G and workspace: the eigenvalues, rank and every
+ * amplitudes) for `count` <= 64 real dense handles side by side, one CTA per
+ * handle (four for windows of more than 145 snapshots), each on its own G and
+ * workspace: the eigenvalues, rank and every
  * later sdmd_svd / sdmd_amplitudes / sdmd_reconstruct of a handle are the
  * same bits as after sdmd_modes(hs[i], r[i], NULL, ...). Serves many streams
  * whose frames arrive together (the serving loop), where one-CTA launches

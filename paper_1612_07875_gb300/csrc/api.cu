@@ -179,6 +179,18 @@ PtrKind ptr_kind(const void* p) {
   }
 }
 
+// Whether a kernel on GPU `device` may use p directly: that GPU's own device
+// memory. Another GPU's memory (which a kernel reaches only with peer access)
+// and managed memory are left to cudaMemcpyAsync.
+bool on_gpu(const void* p, int device) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+
 // Copy `bytes` from device memory to a caller buffer of any kind; pageable
 // destinations make the call wait for the stream.
 int copy_out(void* dst, const void* src_dev, size_t bytes, cudaStream_t st) {
@@ -672,7 +684,7 @@ int sdmd_push_sparse(sdmd_t h, int32_t nnz, const int32_t* idx, const void* vals
   const int32_t s = h->head;
   int* sidx = h->idx_ring + (int64_t)s * h->nnz_max;
   float2* sval = h->val_ring + (int64_t)s * h->nnz_max;
-  const bool from_device = nnz > 0 && ptr_kind(idx) == kDevice && ptr_kind(vals) == kDevice &&
+  const bool from_device = nnz > 0 && on_gpu(idx, h->device) && on_gpu(vals, h->device) &&
                            (reinterpret_cast<uintptr_t>(idx) & 3u) == 0 && (reinterpret_cast<uintptr_t>(vals) & 7u) == 0;
   if (nnz > 0 && !from_device) {         // a snapshot in device memory is copied by the scatter kernel
     TraceScope ts(h, SDMD_K_INGEST, st);
@@ -790,10 +802,10 @@ int ingest(sdmd_s* h, const void* x, cudaStream_t st) {
 }
 
 // Whether the Gram-row kernel can take the snapshot from the caller's buffer
-// (bulk copies need 16-byte aligned device memory); other sources go through
-// ingest().
-bool row_ingests(const void* x) {
-  return (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && ptr_kind(x) == kDevice;
+// (bulk copies need 16-byte aligned memory of this GPU); other sources go
+// through ingest().
+bool row_ingests(const void* x, int device) {
+  return (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && on_gpu(x, device);
 }
 
 // Gram row of the newest snapshot, in slot `s` (x = nullptr) or still in the
@@ -834,7 +846,7 @@ int sdmd_push(sdmd_t h, const void* x, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = flush_pending(h, st);
   if (rc != SDMD_OK) return rc;
-  if (row_ingests(x)) {
+  if (row_ingests(x, h->device)) {
     rc = wait_ring_readers(h, st);
     return rc == SDMD_OK ? gram_row_and_advance(h, h->head, st, x) : rc;
   }
@@ -929,7 +941,7 @@ int sdmd_push_batch(sdmd_t h, int32_t k, const void* X, int64_t ld, void* stream
   const int64_t count0 = h->count;
   int copied = 0;
   cudaError_t e = cudaSuccess;
-  if (ptr_kind(X) == kDevice) {                            // ingest only
+  if (on_gpu(X, h->device)) {                              // ingest only
     TraceScope ts(h, SDMD_K_INGEST, st);
     const int64_t bytes = h->n * h->elem;
     int64_t bx = (bytes + 16 * 256 * 4 - 1) / (16 * 256 * 4);        // four vectors a thread
@@ -1066,11 +1078,11 @@ int sdmd_push_many(const sdmd_t* hs, const void* const* xs, int32_t count, void*
   if (rc != SDMD_OK) return rc;
   int copied = 0;
   cudaError_t e = cudaSuccess;
-  // one launch when every snapshot is aligned device memory, else a copy each
+  // one launch when every snapshot is aligned memory of this GPU, else a copy each
   bool all_dev = true;
   int64_t most = 0;
   for (int i = 0; i < plan.ncopies; ++i) {
-    all_dev = all_dev && row_ingests(plan.src[i]);
+    all_dev = all_dev && row_ingests(plan.src[i], hs[0]->device);
     if ((int64_t)plan.bytes[i] > most) most = (int64_t)plan.bytes[i];
   }
   if (all_dev) {
@@ -1259,22 +1271,36 @@ int sdmd_modes_many(const sdmd_t* hs, int32_t count, const int32_t* r, void* con
     TraceScope ts(hs[0], SDMD_K_MODES, st);
     CK(launch_modes_batch(b, st));
   }
-  // the results: one launch for those to device memory, a copy each for
-  // pinned host memory
-  const bool r_dev = r_out && ptr_kind(r_out) == kDevice;
+  // the results: one launch for those to this GPU's memory (buffers that do
+  // not overlap, so the order of the copies does not matter), a copy each for
+  // the others
+  const int device = hs[0]->device;
+  const bool r_dev = r_out && on_gpu(r_out, device);
+  bool apart = true;
+  for (int i = 0; lambda && i < count; ++i) {
+    if (!lambda[i]) continue;
+    const uintptr_t b0 = reinterpret_cast<uintptr_t>(lambda[i]), e0 = b0 + (size_t)r[i] * 16;
+    const uintptr_t q0 = reinterpret_cast<uintptr_t>(r_out);
+    apart = apart && !(r_out && b0 < q0 + (size_t)count * 4 && q0 < e0);
+    for (int j = 0; j < i; ++j) {
+      if (!lambda[j]) continue;
+      const uintptr_t b1 = reinterpret_cast<uintptr_t>(lambda[j]);
+      apart = apart && !(b0 < b1 + (size_t)r[j] * 16 && b1 < e0);
+    }
+  }
   CopyJobs jobs[2];                      // eigenvalues, ranks
   int nj[2] = {0, 0};
   for (int i = 0; i < count; ++i) {
     sdmd_s* h = hs[i];
     const ModesLayout L = modes_layout(h->m);
     auto put = [&](int q, const void* src, void* dst, size_t bytes, bool dev) -> cudaError_t {
-      if (!dev || (reinterpret_cast<uintptr_t>(dst) & 3u)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
+      if (!apart || !dev || (reinterpret_cast<uintptr_t>(dst) & 3u)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
       jobs[q].src[nj[q]] = src;
       jobs[q].dst[nj[q]] = dst;
       jobs[q].bytes[nj[q]++] = (int64_t)bytes;
       return cudaSuccess;
     };
-    if (lambda && lambda[i]) CK(put(0, h->ws + L.lamout, lambda[i], (size_t)r[i] * 16, ptr_kind(lambda[i]) == kDevice));
+    if (lambda && lambda[i]) CK(put(0, h->ws + L.lamout, lambda[i], (size_t)r[i] * 16, on_gpu(lambda[i], device)));
     if (r_out) CK(put(1, h->r_dev, r_out + i, sizeof(int32_t), r_dev));
     h->last_r = r[i];
     h->last_p = resident(h) - 1;

@@ -1,6 +1,6 @@
 // Small dense algebra of the exact DMD step (Sec. 2.1 Eqs. 3-4, Sec. 2.2
 // Eqs. 7-9; Algorithm 1's eig/sort and Algorithm 2's vsi, A~, eig, vsi*W),
-// one CTA of 256 threads per call.
+// one CTA of 512 threads per call, or a cluster of four (rule at modes_ctas).
 //
 // Precision plan. GB300 executes FP64 at about 1/64 of the FP32 rate, and an
 // FP64 instruction costs the same whether one lane or 32 are active. So the
@@ -12,19 +12,22 @@
 //  0. gather  G_X = G[0:p, 0:p], G_XY = G[0:p, 1:p+1] in time order from the
 //     ring-indexed physical G (p = c-1), converted to df64 and scaled by an
 //     exact power of two so that the largest diagonal entry is in [0.5, 1).
-//  1. Householder tridiagonalisation of G_X in df64: Q^T G_X Q = T (d, e),
-//     reflectors kept down the columns of G_X's storage, one block barrier
-//     per Householder step (the rank-2 update deferred into the next step).
+//  1. Householder tridiagonalisation of G_X in df64: Q^T G_X Q = T (d, e);
+//     the rank-2 update of a step runs in the next one, beside that step's
+//     scalar chain (over the shared memory of four CTAs for long windows).
 //  2. the r largest eigenvalues of T by Sturm-count multisection in FP32
 //     (one warp per eigenvalue, 32 points per round): shifts accurate to
 //     ~eps32 * |T|.
 //  3. df64 inverse iteration on T with those shifts (one thread per vector,
-//     LU with partial pivoting), classical Gram-Schmidt over all wanted
-//     vectors after every solve, then a Rayleigh-Ritz step (Z^T T Z
-//     diagonalised by parallel cyclic Jacobi in df64); a second round uses
-//     the Ritz values as shifts. Clusters of close eigenvalues are resolved
-//     by the Gram-Schmidt / Rayleigh-Ritz steps.
-//  4. back-transform z -> Q z in df64 (warp per vector) = columns of V.
+//     vectors spread over the warps; LU with partial pivoting, loads one step
+//     ahead of the recurrences), classical Gram-Schmidt over all wanted
+//     vectors after every solve (two barriers a vector), then a Rayleigh-Ritz
+//     step (Z^T T Z diagonalised by parallel cyclic Jacobi in df64, its 2 x 2
+//     blocks rotated by one thread each); a second round uses the Ritz values
+//     as shifts. Clusters of close eigenvalues are resolved by the
+//     Gram-Schmidt / Rayleigh-Ritz steps.
+//  4. back-transform z -> Q z in df64 = columns of V; a spare warp meanwhile
+//     checks by a Sturm count that no eigenvalue was missed.
 //  5. numerical rank, sigma = sqrt(lambda), vsi = V Sigma^-1.
 //  6. A~ = vsi^T (G_XY vsi) in df64.
 //  7. eig(A~): FP32 complex Householder-Hessenberg, shifted QR (Wilkinson
@@ -35,6 +38,13 @@
 //     eigenvectors; eigenpairs ordered by descending |lambda| then angle.
 //  8. M = vsi W in df64, written in FP32 (scaled back) for the Phi kernel;
 //     lambda, sigma and V written out in FP64.
+//
+// Bound by dependent latency: block barriers (43 cycles), df64 divisions (173
+// cycles of IEEE division) and chains of FADD (4.9 cycles each). Thousand
+// cycles per phase (gather, 1, 2, 3, 4, 6, 7, 8) with r = 10: p = 31 18 / 84 /
+// 25 / 354 / 16 / 15 / 187 / 21; p = 119 (four CTAs) 19 / 528 / 79 / 647 / 150 /
+// 78 / 231 / 34. One call, p = 31 / 119: 459 / 1,277 us with 8 warps that
+// repeated the scalar chains, 357 / 850 us now.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <float.h>
@@ -167,7 +177,7 @@ __device__ WS carve(double* base, const ModesLayout& L) {
 //
 // Measured, p = 99 / 126 / 255: 712 / 1,103 / 8,400 thousand cycles when eight
 // warps repeated the scalar chain, took whole rows and (p > 144) kept A in L2;
-// see the phase clocks for the present figures.
+// 517 now for p = 99 in one CTA, 528 / 1,940 for p = 119 / 255 over four.
 //
 // Workspace tw (8-byte units): part[kCl > 1 ? 2 : 1][kParts][P], u, v, w, pv
 // [P], dot[kParts], inv[2].
@@ -2383,8 +2393,10 @@ bool modes_embed_ok(int c, int r) {
 
 // CTAs of one eigensolver. Alone, a window of kSpreadP pairs or more is faster
 // over a cluster: the trailing updates, bound by one SM's FP32 rate, split four
-// ways for one cluster barrier a step.
-constexpr int kSpreadP = 64;
+// ways for one cluster barrier a step. Four CTAs against one, r = 10: p = 64
+// 493 / 480 us, 72 544 / 550, 80 569 / 585, 100 684 / 734, 120 789 / 884, 144
+// 983 / 1160. Many windows at once fill the SMs with one CTA each.
+constexpr int kSpreadP = 72;
 static int modes_ctas(const ModesArgs& a) {
   const int p = a.embed_cx ? 2 * (a.c - 1) : a.c - 1;
   return p > kSmemMaxP || (a.spread && p >= kSpreadP) ? kClusterCtas : 1;
