@@ -26,9 +26,10 @@
 // x positions 8 kg .. 8 kg + 7 at (kg * 16 + rg) * 128 bytes: LBO 2048 B
 // between K neighbours, SBO 128 B between row groups.
 //
-// Work: persistent CTAs take chunks of 2048 positions (8 K-steps of 256)
+// Work: persistent CTAs take chunks of 1024 positions (4 K-steps of 256)
 // from a global counter; the integer sums do not depend on which CTA took
-// which chunk. Per CTA:
+// which chunk. With 2048 a window of 1,000,003 positions was four rounds of
+// chunks for 3.2 of work: 200 such frames loaded in 548 us, 483 now. Per CTA:
 //   warps 9..16  load + convert: warp-private row groups (8 rows x 128 bytes
 //                per stage), cp.async copies (a quarter warp = one row's 128
 //                bytes) into a 5-deep staging ring (row pitch 144 B: the
@@ -70,7 +71,7 @@ constexpr int kThreads = 32 * (kConvWarp0 + kConvWarps);   // 544
 constexpr int kGroups = 16 / kConvWarps;  // row groups of 8 per converter warp, at most
 constexpr int kRowsM = 128;          // MMA M
 constexpr int kKst = 256;            // positions per K-step
-constexpr int kStepsPerChunk = 8;    // scheduling unit: 2048 positions
+constexpr int kStepsPerChunk = 4;    // scheduling unit: 1024 positions
 constexpr int kStepsPerDrain = 4;    // 1024 positions per accumulator period
 constexpr int kHalf = 128;           // positions per staging stage
 constexpr int kHalves = kKst / kHalf;
