@@ -29,7 +29,8 @@
 // Work: persistent CTAs take chunks of 1024 positions (4 K-steps of 256)
 // from a global counter; the integer sums do not depend on which CTA took
 // which chunk. With 2048 a window of 1,000,003 positions was four rounds of
-// chunks for 3.2 of work: 200 such frames loaded in 548 us, 483 now. Per CTA:
+// chunks for 3.2 of work: 200 such frames loaded in 548 us against 484; chunks
+// of 512 lose to their hand-overs (491 us; 8 HD frames 229 against 221). Per CTA:
 //   warps 9..16  load + convert: warp-private row groups (8 rows x 128 bytes
 //                per stage), cp.async copies (a quarter warp = one row's 128
 //                bytes) into a 5-deep staging ring (row pitch 144 B: the
@@ -172,6 +173,8 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
   __syncthreads();
   fence_after();
   const unsigned tbase = sh.tmem_base;
+  // the setup above runs while the launch before this one ends
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
 
   if (warp >= kConvWarp0) {
     // ---------------- load + convert ----------------
@@ -469,6 +472,10 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
 constexpr int kFinThreads = 1024;
 __global__ void __launch_bounds__(kFinThreads) gram_full_finish_kernel(GramFullArgs a, int ctas, int cw) {
   __shared__ long long gi[kFinThreads], gs[kFinThreads];   // [slice][cw]
+  // the partials are complete; the next launch may set itself up (it waits for
+  // this one before it takes a chunk)
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int i = blockIdx.x, kt = a.k;
   const int j = threadIdx.x % cw, sl = threadIdx.x / cw, slices = kFinThreads / cw;
   if (i == 0 && threadIdx.x == 0) a.sched[0] = 0u;   // ready for the next launch
@@ -520,6 +527,13 @@ cudaError_t launch_gram_full_tc(const GramFullArgs& base, int* ctas_out, cudaStr
   // blocks of 127 - kg rows. A window of at most 127 fits one tile: one
   // launch whatever k.
   const int gmax = (c + 1 <= kRowsM) ? k : kGramFullMaxTargets;
+  // programmatic launches: every kernel waits itself for the one before it, so
+  // its launch and setup hide behind that one's end: the load of 200 frames of
+  // 1,000,003 positions (seven pairs of launches) 488 -> 445 us, 8 HD frames
+  // (one pair) 221 -> 215
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
   for (int hi = c; hi > c - k;) {
     const int lo = (hi - gmax > c - k) ? hi - gmax : c - k;
     const int kg = hi - lo;
@@ -531,13 +545,21 @@ cudaError_t launch_gram_full_tc(const GramFullArgs& base, int* ctas_out, cudaStr
       a.k = kg;
       a.t_old = o;
       a.nold = (lo - o < blk) ? lo - o : blk;
-      gram_full_tc_kernel<<<ctas, kThreads, kSmemBytes, st>>>(a);
-      cudaError_t e = cudaGetLastError();
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)ctas);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = kSmemBytes;
+      cfg.stream = st;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      cudaError_t e = cudaLaunchKernelEx(&cfg, gram_full_tc_kernel, a);
       if (e != cudaSuccess) return e;
       int cw = 8;                          // columns 0 .. k, padded to a power of two
       while (cw < a.k + 1) cw *= 2;
-      gram_full_finish_kernel<<<a.k + 1 + a.nold, kFinThreads, 0, st>>>(a, ctas, cw);
-      e = cudaGetLastError();
+      cfg.gridDim = dim3((unsigned)(a.k + 1 + a.nold));
+      cfg.blockDim = dim3(kFinThreads);
+      cfg.dynamicSmemBytes = 0;
+      e = cudaLaunchKernelEx(&cfg, gram_full_finish_kernel, a, ctas, cw);
       if (e != cudaSuccess) return e;
       o += a.nold;
     } while (o < lo);
