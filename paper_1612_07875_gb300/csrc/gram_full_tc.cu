@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
             w[gi][0] = *reinterpret_cast<const uint4*>(r);
             w[gi][1] = *reinterpret_cast<const uint4*>(r + 64);
           }
+        __syncwarp();                        // every lane has read the stage: the next load refills it
 #pragma unroll
         for (int gi = 0; gi < kGroups; ++gi) {
           if (gi >= ng) break;               // warp-uniform
