@@ -181,7 +181,9 @@ PtrKind ptr_kind(const void* p) {
 
 // Whether a kernel on GPU `device` may use p directly: that GPU's own device
 // memory. Another GPU's memory (which a kernel reaches only with peer access)
-// and managed memory are left to cudaMemcpyAsync.
+// and managed memory are left to cudaMemcpyAsync: snapshots, Gram rows and
+// eigenvalues. (Phi, POD modes, reconstructions and Fourier modes are written
+// by kernels wherever they lie.)
 bool on_gpu(const void* p, int device) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -221,13 +223,14 @@ __global__ void __launch_bounds__(256) ingest_copy_kernel(const uint4* __restric
     reinterpret_cast<uint8_t*>(dst + n16)[threadIdx.x] = reinterpret_cast<const uint8_t*>(src + n16)[threadIdx.x];
 }
 
-// Copy one snapshot (`bytes`) into a ring slot on `st`: the SM kernel above
-// for device sources with both addresses 16-byte aligned, else
-// cudaMemcpyAsync (host sources, unaligned device pointers).
-cudaError_t copy_snapshot(void* dst, const void* src, size_t bytes, int num_sms, cudaStream_t st) {
+// Copy one snapshot (`bytes`) into a ring slot of GPU `device` on `st`: the SM
+// kernel above for sources in that GPU's memory with both addresses 16-byte
+// aligned, else cudaMemcpyAsync (host, managed and other GPUs' memory,
+// unaligned device pointers).
+cudaError_t copy_snapshot(void* dst, const void* src, size_t bytes, int device, int num_sms, cudaStream_t st) {
   if (bytes == 0) return cudaSuccess;
   const bool aligned = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0;
-  if (!aligned || ptr_kind(src) != kDevice) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
+  if (!aligned || !on_gpu(src, device)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
   const int64_t n16 = (int64_t)(bytes / 16);
   const int tail = (int)(bytes - (size_t)n16 * 16);
   int64_t blocks = (n16 + 4 * 256 - 1) / (4 * 256);
@@ -788,7 +791,7 @@ int ingest(sdmd_s* h, const void* x, cudaStream_t st) {
     }
     TraceScope ts(h, SDMD_K_INGEST, st);
     CK(cudaStreamWaitEvent(st, h->ev_h2d, 0));
-    CK(copy_snapshot(h->ring + (int64_t)h->head * h->slot_bytes, sb, bytes, h->num_sms, st));
+    CK(copy_snapshot(h->ring + (int64_t)h->head * h->slot_bytes, sb, bytes, h->device, h->num_sms, st));
     CK(cudaEventRecord(h->ev_stage_free[b], st));
     return SDMD_OK;
   }
@@ -797,7 +800,8 @@ int ingest(sdmd_s* h, const void* x, cudaStream_t st) {
     if (rc != SDMD_OK) return rc;
   }
   TraceScope ts(h, SDMD_K_INGEST, st);
-  CK(copy_snapshot(h->ring + (int64_t)h->head * h->slot_bytes, x, (size_t)(h->n * h->elem), h->num_sms, st));
+  CK(copy_snapshot(h->ring + (int64_t)h->head * h->slot_bytes, x, (size_t)(h->n * h->elem), h->device, h->num_sms,
+                   st));
   return SDMD_OK;
 }
 
@@ -956,7 +960,7 @@ int sdmd_push_batch(sdmd_t h, int32_t k, const void* X, int64_t ld, void* stream
   for (int j = copied; j < k && e == cudaSuccess; ++j) {
     TraceScope ts(h, SDMD_K_INGEST, st);
     e = copy_snapshot(h->ring + (int64_t)((head0 + j) % h->cap) * h->slot_bytes, src + (size_t)j * ld * elem_bytes,
-                      (size_t)(h->n * h->elem), h->num_sms, st);
+                      (size_t)(h->n * h->elem), h->device, h->num_sms, st);
     if (e == cudaSuccess) ++copied;
   }
   if (e == cudaSuccess) {
@@ -1217,7 +1221,7 @@ int sdmd_gram(sdmd_t h, void* G, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int c = resident(h);
   if (c == 0) return SDMD_OK;
-  const bool direct = ptr_kind(G) == kDevice;
+  const bool direct = on_gpu(G, h->device);
   uint64_t* dst = direct ? static_cast<uint64_t*>(G) : static_cast<uint64_t*>(h->gtmp);
   gather_gram_kernel<<<(c * c + 255) / 256, 256, 0, st>>>(static_cast<const uint64_t*>(h->G), h->cap, c,
                                                            oldest_slot(h), (int)(h->gsz / 8), dst);
@@ -1325,7 +1329,7 @@ int sdmd_newest_row(sdmd_t h, void* row, void* stream) {
   const int c = resident(h);
   if (c == 0) return fail(SDMD_ERR_NOT_READY, "sdmd_newest_row: no snapshot pushed yet");
   const int32_t s_new = (int32_t)((h->head + h->cap - 1) % h->cap);
-  const bool direct = ptr_kind(row) == kDevice;
+  const bool direct = on_gpu(row, h->device);
   uint64_t* dst = direct ? static_cast<uint64_t*>(row) : static_cast<uint64_t*>(h->gtmp);
   newest_row_kernel<<<(c + 127) / 128, 128, 0, st>>>(static_cast<const uint64_t*>(h->G), h->cap, c, oldest_slot(h),
                                                       s_new, (int)(h->gsz / 8), dst);
@@ -1346,7 +1350,7 @@ int sdmd_set_newest_row(sdmd_t h, const void* row, void* stream) {
   if (c == 0) return fail(SDMD_ERR_NOT_READY, "sdmd_set_newest_row: no snapshot pushed yet");
   const int32_t s_new = (int32_t)((h->head + h->cap - 1) % h->cap);
   const uint64_t* src = static_cast<const uint64_t*>(row);
-  if (ptr_kind(row) != kDevice) {      // staged through the gather scratch, in stream order
+  if (!on_gpu(row, h->device)) {       // staged through the gather scratch, in stream order
     CK(cudaMemcpyAsync(h->gtmp, row, (size_t)c * h->gsz, cudaMemcpyDefault, st));
     src = static_cast<const uint64_t*>(h->gtmp);
   }
