@@ -31,7 +31,7 @@
 // 14.3 us.
 //
 //  - uint8: __dp4a (4 u8 x u8 products into u32). A lane sums at most
-//    32 KiB / 32 = 1024 products (< 2^32 / 255^2) before the value goes to
+//    24 KiB / 32 = 768 products (< 2^32 / 255^2) before the value goes to
 //    int64, so the result is exact and independent of order.
 //  - float32: four FP32 FMA chains of 8 products per piece per lane, then the
 //    piece's sum is added in FP64; cross-lane and cross-CTA sums are FP64 in a
@@ -41,7 +41,10 @@
 //
 // Every mbarrier wait is bounded (about one second of SM clock); on expiry
 // the kernel raises kDevTimeout in the handle's status word, stops issuing
-// copies, waits (bounded) for the copies it has in flight, and finishes.
+// copies, waits (bounded) for the copies it has in flight, and finishes. The
+// row is then incomplete, but the snapshot is not: with x_src the CTAs that
+// gave up still copy it into its slot (plain loads and stores, nothing to wait
+// for), so a rebuild of the window restores G.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -56,7 +59,18 @@ namespace {
 constexpr int kStages = 4;
 constexpr int kPiece = 4096;                       // bytes per bulk copy
 constexpr int kXSub = 24576;                       // largest chunk (x_new bytes staged per chunk)
-constexpr long long kWaitCycles = 2000000000LL;    // ~1 s at 2 GHz
+static_assert(kXSub / 32 * 255LL * 255LL < (1LL << 32), "a lane's uint8 sum over a chunk stays in 32 bits");
+// Bound of a wait, ~1 s at 2 GHz. A test compiles this file with a short bound
+// and with the x_new barrier of every CTA's item number SDMD_GR_STARVED_ITEM
+// told to expect 16 bytes that nobody sends, so that its wait expires.
+#ifndef SDMD_GR_WAIT_CYCLES
+#define SDMD_GR_WAIT_CYCLES 2000000000LL
+#endif
+#ifndef SDMD_GR_STARVED_ITEM
+#define SDMD_GR_STARVED_ITEM -1
+#endif
+constexpr long long kWaitCycles = SDMD_GR_WAIT_CYCLES;
+constexpr int kStarvedItem = SDMD_GR_STARVED_ITEM;
 
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
@@ -263,6 +277,30 @@ __device__ __forceinline__ void finish_slot(const void* partials, int nblk, int 
   }
 }
 
+// After an expired wait (the whole CTA): the chunks of the snapshot that
+// belong to the items at hand (it0, it1) and to those nobody has taken yet go
+// from the caller's buffer to the ring slot. Chunks that were stored already
+// get the same bytes again.
+__device__ void ingest_rest(const GramRowArgs& a, Smem& sm, int it0, int it1, int nitems) {
+  uint8_t* slot = const_cast<uint8_t*>(a.ring) + (int64_t)a.s_new * a.slot_bytes;
+  for (int q = 0;; ++q) {
+    int it = q == 0 ? it0 : it1;
+    if (q >= 2) {
+      __syncthreads();
+      if (threadIdx.x == 0) sm.iq[0] = (int)atomicAdd(a.ticket + 1, 1u);
+      __syncthreads();
+      it = sm.iq[0];
+      if (it >= nitems) return;
+    }
+    if (it >= nitems || it % a.groups != 0) continue;
+    const int64_t off = (int64_t)(it / a.groups) * a.chunk, len = min(a.chunk, a.x_bytes - off);
+    const int64_t nv = len > 0 ? len / 16 : 0;
+    for (int64_t v = threadIdx.x; v < nv; v += kGrThreads)
+      reinterpret_cast<uint4*>(slot + off)[v] = reinterpret_cast<const uint4*>(a.x_src + off)[v];
+    for (int64_t b = 16 * nv + threadIdx.x; b < len; b += kGrThreads) slot[off + b] = a.x_src[off + b];
+  }
+}
+
 template <int kMode>
 __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArgs a) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -298,7 +336,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
     const int ch = it / S;
     const unsigned xb = smem_u32(&sm.xbar[k & 1]);
     const int len = bulk_len(ch);
-    mbar_expect_tx(xb, (unsigned)len);
+    mbar_expect_tx(xb, (unsigned)len + (kStarvedItem >= 0 && k == kStarvedItem ? 16u : 0u));
     if (len > 0) bulk_g2s(smem_u32(sm.xs[k & 1]), xnew + (int64_t)ch * a.chunk, (unsigned)len, xb);
   };
   if (threadIdx.x == 0) {
@@ -350,7 +388,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
       }
     }
   };
-  int gprev = -1;                      // group of the item before
+  int gprev = -1, itprev = -1;         // group and index of the item before
   for (int k = 0;; ++k) {
     __syncthreads();                   // item k - 1 consumed, its partials written: xs[(k + 1) & 1] is free
     if (threadIdx.x == 0) {
@@ -382,12 +420,17 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
       // is released (bounded waits); then stop
       if (lane == 0)
         for (unsigned gk = consumed; gk < issued; ++gk) mbar_wait(smem_u32(&sm.bar[warp][gk % kStages]), (gk / kStages) & 1);
-      if (threadIdx.x == 0 && it < nitems) mbar_wait(smem_u32(&sm.xbar[k & 1]), (unsigned)((k >> 1) & 1));
+      if (threadIdx.x == 0) {          // (item k - 1's may be the wait that expired)
+        mbar_wait(smem_u32(&sm.xbar[(k - 1) & 1]), (unsigned)(((k - 1) >> 1) & 1));
+        if (it < nitems) mbar_wait(smem_u32(&sm.xbar[k & 1]), (unsigned)((k >> 1) & 1));
+      }
+      if (src) ingest_rest(a, sm, itprev, it, nitems);
       break;
     }
     if (it >= nitems) break;
     const int ch = it / S, g = it - ch * S;
     gprev = g;
+    itprev = it;
     const int np = chunk_len(ch) / kPiece, rows = rows_of(g);
     uint8_t* xs = sm.xs[k & 1];
     top_up(k);
