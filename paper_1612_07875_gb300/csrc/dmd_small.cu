@@ -2402,14 +2402,32 @@ static int modes_ctas(const ModesArgs& a) {
   return p > kSmemMaxP || (a.spread && p >= kSpreadP) ? kClusterCtas : 1;
 }
 
-static size_t modes_smem_bytes(const ModesArgs& a) {
-  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req, modes_ctas(a));
+// Dynamic shared memory of an eigensolver over `ctas` CTAs.
+static size_t modes_smem_bytes(const ModesArgs& a, int ctas) {
+  const SmemPlan plan = smem_plan(a.embed_cx ? 2 * (a.c - 1) : a.c - 1, a.r_req, ctas);
   return (size_t)(plan.vec_units + plan.rr_units + plan.pool_units) * 8;
 }
 
+cudaError_t modes_batch_split(const ModesBatch& b, ModesBatch (&part)[2], size_t (&bytes)[2]) {
+  part[0].count = part[1].count = 0;
+  bytes[0] = bytes[1] = 0;
+  if (b.count < 1 || b.count > kMaxModesJobs) return cudaErrorInvalidValue;
+  for (int i = 0; i < b.count; ++i) {
+    ModesArgs a = b.job[i];
+    if (a.embed_cx) return cudaErrorInvalidValue;   // real windows only
+    a.spread = 0;                                   // the jobs run side by side
+    const int ctas = modes_ctas(a), q = ctas > 1;
+    part[q].job[part[q].count++] = a;
+    const size_t jb = modes_smem_bytes(a, ctas);
+    if (jb > bytes[q]) bytes[q] = jb;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_modes_small(const ModesArgs& a, cudaStream_t st) {
-  const size_t bytes = modes_smem_bytes(a);
-  const bool cluster = modes_ctas(a) > 1;
+  const int ctas = modes_ctas(a);
+  const size_t bytes = modes_smem_bytes(a, ctas);
+  const bool cluster = ctas > 1;
   const void* f = cluster ? reinterpret_cast<const void*>(modes_small_kernel<kClusterCtas>)
                           : reinterpret_cast<const void*>(modes_small_kernel<1>);
   const cudaError_t e = smem_optin(f, bytes);
@@ -2433,18 +2451,11 @@ cudaError_t launch_modes_small(const ModesArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_modes_batch(const ModesBatch& b, cudaStream_t st) {
-  if (b.count < 1 || b.count > kMaxModesJobs) return cudaErrorInvalidValue;
-  ModesBatch part[2];                    // [0] one-CTA windows, [1] cluster windows
-  size_t bytes[2] = {0, 0};
-  part[0].count = part[1].count = 0;
-  for (int i = 0; i < b.count; ++i) {
-    const int q = b.job[i].c - 1 > kSmemMaxP;
-    part[q].job[part[q].count++] = b.job[i];
-    const size_t jb = modes_smem_bytes(b.job[i]);
-    if (jb > bytes[q]) bytes[q] = jb;
-  }
+  ModesBatch part[2];
+  size_t bytes[2];
+  cudaError_t e = modes_batch_split(b, part, bytes);
+  if (e != cudaSuccess) return e;
   const int paired = part[0].count > 0 && part[1].count > 0;
-  cudaError_t e = cudaSuccess;
   if (part[0].count > 0) e = smem_optin(reinterpret_cast<const void*>(modes_batch_kernel<1>), bytes[0]);
   if (e == cudaSuccess && part[1].count > 0)
     e = smem_optin(reinterpret_cast<const void*>(modes_batch_kernel<kClusterCtas>), bytes[1]);

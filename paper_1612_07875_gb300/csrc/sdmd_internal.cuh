@@ -218,14 +218,19 @@ struct ModesLayout {
 __host__ __device__ ModesLayout modes_layout(int m);
 
 cudaError_t launch_modes_small(const ModesArgs& a, cudaStream_t st);
-// The real-window eigensolvers of several handles in one launch (one CTA per
-// job; each job exactly as launch_modes_small would run it alone).
+// The real-window eigensolvers of several handles side by side (one CTA per
+// job, a cluster for the longest windows; each job exactly as
+// launch_modes_small would run it alone). cudaErrorInvalidValue for a bad
+// count or an embedded complex window.
 constexpr int kMaxModesJobs = 64;
 struct ModesBatch {
   ModesArgs job[kMaxModesJobs];
   int32_t count;
 };
 cudaError_t launch_modes_batch(const ModesBatch& b, cudaStream_t st);
+// Its two launches: [0] the one-CTA jobs, [1] the cluster ones, and the
+// dynamic shared memory of each (the CTAs of a job decide both).
+cudaError_t modes_batch_split(const ModesBatch& b, ModesBatch (&part)[2], size_t (&bytes)[2]);
 // The same outputs for complex windows (G complex128 Hermitian): FP64 Jacobi
 // for G_X, complex A~, W, M and amplitudes.
 cudaError_t launch_modes_complex(const ModesArgs& a, cudaStream_t st);
