@@ -723,7 +723,7 @@ int sdmd_push_sparse(sdmd_t h, int32_t nnz, const int32_t* idx, const void* vals
     CK(launch_sparse_scatter(from_device ? idx : sidx, from_device ? static_cast<const float2*>(vals) : sval, nnz, h->n,
                              h->stamp, h->tag, h->tval, from_device ? sidx : nullptr, from_device ? sval : nullptr,
                              h->status, st));
-    CK(launch_sparse_row(a, st));
+    CK(launch_sparse_row(a, h->num_sms, st));
   }
   h->head = (s + 1) % h->cap;
   h->count += 1;
@@ -1187,7 +1187,7 @@ int sdmd_rebuild(sdmd_t h, void* stream) {
       TraceScope ts(h, SDMD_K_GRAM_ROW, st);
       CK(launch_sparse_scatter(h->idx_ring + (int64_t)s * h->nnz_max, h->val_ring + (int64_t)s * h->nnz_max,
                                h->nnz[s], h->n, h->stamp, h->tag, h->tval, nullptr, nullptr, h->status, st));
-      CK(launch_sparse_row(a, st));
+      CK(launch_sparse_row(a, h->num_sms, st));
     } else {
       GramRowArgs a;
       a.ring = h->ring;

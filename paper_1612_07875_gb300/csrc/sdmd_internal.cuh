@@ -330,7 +330,7 @@ int sparse_chunks(int nnz);
 // the ring slot (idx, val in device memory).
 cudaError_t launch_sparse_scatter(const int* idx, const float2* val, int nnz, int64_t n, int stamp, int* tag,
                                   float2* tval, int* ring_idx, float2* ring_val, int* status, cudaStream_t st);
-cudaError_t launch_sparse_row(const SparseRowArgs& a, cudaStream_t st);
+cudaError_t launch_sparse_row(const SparseRowArgs& a, int num_sms, cudaStream_t st);
 
 // Modes of a Fourier-sparse window in coefficient space (compressed Phi-hat).
 struct FourierPhiArgs {

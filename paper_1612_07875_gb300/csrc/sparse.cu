@@ -17,8 +17,15 @@
 //     at most 8 terms, CTA and cross-CTA sums in FP64 in a fixed order; the
 //     last CTA (atomic ticket, no waiting) writes row/column s_new of the
 //     Hermitian G. The kernel is three dependent gathers deep (index, tag,
-//     values), so a thread has its eight entries of each in flight together:
-//     26 us one entry after the other at c = 64, nnz = 10,486.
+//     values), so a thread has its eight entries of each in flight together
+//     (26 us one entry after the other at c = 64, nnz = 10,486), and in launches
+//     of one short wave it loads the values before it knows the tags (a push
+//     of that size 29.1 us, 30.5 after the tags). Larger launches are bound by
+//     the gathers' sectors, where values of coefficients that the new snapshot
+//     lacks cost more than they save: nnz = 167,772 of n = 2^24, 1 % shared, a
+//     push 254 us with them, 106 without, 133 one entry after the other. Tables
+//     of several hundred megabytes are gathered best one after the other: nnz =
+//     671,088 of n = 2^26, 90 % shared, 985 us, 1,087 together.
 // Indices outside [0, n) are skipped and raise kDevRange in the status word.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -56,6 +63,12 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// How a thread takes its eight entries: one after the other, together, or
+// together with the values loaded beside the tags whether or not the new
+// snapshot has the coefficient. The sums are the same.
+enum { kSerial = 0, kTogether = 1, kAhead = 2 };
+
+template <int kHow>
 __global__ void __launch_bounds__(kThreads) sparse_row_kernel(SparseRowArgs a) {
   __shared__ double red[2][kThreads / 32];
   __shared__ bool last;
@@ -74,34 +87,53 @@ __global__ void __launch_bounds__(kThreads) sparse_row_kernel(SparseRowArgs a) {
   const float2* val = a.val_ring + (int64_t)slot * a.nnz_max;
   const int e0 = q * kChunk, e1 = min(nnz, e0 + kChunk);
   constexpr int kPer = kChunk / kThreads;
-  // every load is unconditional (entries past the end and indices outside
-  // [0, n) read entry or table position 0 and do not count)
-  int k[kPer], tg[kPer];
-  float2 x[kPer], y[kPer];
-  bool in[kPer];
-#pragma unroll
-  for (int u = 0; u < kPer; ++u) {
-    const int e = e0 + threadIdx.x + u * kThreads;
-    in[u] = e < e1;
-    k[u] = __ldg(idx + (in[u] ? e : 0));
-    x[u] = __ldg(val + (in[u] ? e : 0));
-  }
-#pragma unroll
-  for (int u = 0; u < kPer; ++u) {
-    in[u] = in[u] && k[u] >= 0 && (int64_t)k[u] < a.n;
-    k[u] = in[u] ? k[u] : 0;
-    tg[u] = __ldcg(a.tag + k[u]);
-    y[u] = __ldcg(a.tval + k[u]);
-  }
-#pragma unroll
-  for (int u = 0; u < kPer; ++u) in[u] = in[u] && tg[u] == a.stamp;
   float sr = 0.f, si = 0.f;
-#pragma unroll
-  for (int u = 0; u < kPer; ++u)
-    if (in[u]) {
-      sr = fmaf(x[u].x, y[u].x, fmaf(x[u].y, y[u].y, sr));     // conj(x) * y
-      si = fmaf(x[u].x, y[u].y, fmaf(-x[u].y, y[u].x, si));
+  if constexpr (kHow == kSerial) {
+    for (int e = e0 + threadIdx.x; e < e1; e += kThreads) {
+      const int k = __ldg(idx + e);
+      if (k < 0 || (int64_t)k >= a.n) continue;
+      if (__ldcg(a.tag + k) != a.stamp) continue;
+      const float2 x = __ldg(val + e), y = __ldcg(a.tval + k);
+      sr = fmaf(x.x, y.x, fmaf(x.y, y.y, sr));       // conj(x) * y
+      si = fmaf(x.x, y.y, fmaf(-x.y, y.x, si));
     }
+  } else {
+    // a thread's eight loads of a kind are in flight together (entries past the
+    // end and indices outside [0, n) read entry or table position 0 and do not
+    // count)
+    int k[kPer], tg[kPer];
+    float2 x[kPer], y[kPer];
+    bool in[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int e = e0 + threadIdx.x + u * kThreads;
+      in[u] = e < e1;
+      k[u] = __ldg(idx + (in[u] ? e : 0));
+      x[u] = y[u] = make_float2(0.f, 0.f);
+      if (kHow == kAhead) x[u] = __ldg(val + (in[u] ? e : 0));
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      in[u] = in[u] && k[u] >= 0 && (int64_t)k[u] < a.n;
+      k[u] = in[u] ? k[u] : 0;
+      tg[u] = __ldcg(a.tag + k[u]);
+      if (kHow == kAhead) y[u] = __ldcg(a.tval + k[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      in[u] = in[u] && tg[u] == a.stamp;
+      if (kHow != kAhead && in[u]) {
+        y[u] = __ldcg(a.tval + k[u]);
+        x[u] = __ldg(val + e0 + threadIdx.x + u * kThreads);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      if (in[u]) {
+        sr = fmaf(x[u].x, y[u].x, fmaf(x[u].y, y[u].y, sr));     // conj(x) * y
+        si = fmaf(x[u].x, y[u].y, fmaf(-x[u].y, y[u].x, si));
+      }
+  }
   double dr = warp_sum((double)sr), di = warp_sum((double)si);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
@@ -323,8 +355,18 @@ cudaError_t launch_sparse_scatter(const int* idx, const float2* val, int nnz, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_sparse_row(const SparseRowArgs& a, cudaStream_t st) {
-  sparse_row_kernel<<<a.nblk, kThreads, 0, st>>>(a);
+// Values ahead of the tags: at most four CTAs an SM, and lookup tables (12
+// bytes a coefficient) that the L2 holds.
+constexpr int kAheadCtas = 4;
+constexpr int64_t kAheadN = 1 << 22, kSerialN = 1 << 25;
+
+cudaError_t launch_sparse_row(const SparseRowArgs& a, int num_sms, cudaStream_t st) {
+  if (a.n > kSerialN)
+    sparse_row_kernel<kSerial><<<a.nblk, kThreads, 0, st>>>(a);
+  else if (a.n <= kAheadN && a.nblk <= kAheadCtas * num_sms)
+    sparse_row_kernel<kAhead><<<a.nblk, kThreads, 0, st>>>(a);
+  else
+    sparse_row_kernel<kTogether><<<a.nblk, kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
