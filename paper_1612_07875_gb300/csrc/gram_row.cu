@@ -20,15 +20,18 @@
 // completes a group's last chunk (atomic count, no waiting) sums its partials
 // in a fixed order and writes its entries of row and column `s_new` of G, so
 // the result depends neither on which CTA took which item nor on the number
-// of groups.
+// of groups. The count's fence and round trip would lengthen every hand-over
+// between two items, so its answer is looked at one item later (n = 2^28 bytes:
+// 16 slots 819 -> 770 us, 8 slots 509 -> 465).
 //
 // The new snapshot. With x_src set (a 16-byte aligned device buffer) the
 // kernel also is the ingest: x_new's chunks come from x_src, the items of
 // group 0 write them to the ring slot, and <x_new, x_new> is formed from the
 // staged chunk, so the snapshot is read once and its slot not at all. Against
-// a copy kernel before this one a push of one HD frame (m = 100) went from 126
-// to 117 us, one of a 64 x 64 FP32 field (m = 32, launches only) from 22.5 to
-// 14.3 us.
+// a copy kernel before this one a push of one HD frame (m = 100) went from 124
+// to 114 us, one of a 64 x 64 FP32 field (m = 32, launches only) from 22.5 to
+// 14.3 us. (Snapshots of 2^28 bytes in windows of 64 and more slots, 17 GB, are
+// the exception: 2,545 us with the copy, 2,578.)
 //
 //  - uint8: __dp4a (4 u8 x u8 products into u32). A lane sums at most
 //    24 KiB / 32 = 768 products (< 2^32 / 255^2) before the value goes to
@@ -121,6 +124,8 @@ __device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
+
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;\n" ::: "memory"); }
 
 // Bounded wait on phase `parity` of barrier `bar`; false on expiry.
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
@@ -388,7 +393,14 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
       }
     }
   };
+  auto finish_group = [&](int g) {     // a group whose chunks are all in: its entries of G
+    if (g < 0) return;
+    for (int jj = warp + kGrWarps * g; jj < a.c; jj += kGrWarps * S)
+      finish_slot<kMode>(a.partials, a.nblk, jj, a.G, a.s_first, a.s_new, a.m, lane);
+  };
   int gprev = -1, itprev = -1;         // group and index of the item before
+  int counted = -1;                    // (thread 32) group of the count on its way
+  unsigned count = 0;
   for (int k = 0;; ++k) {
     __syncthreads();                   // item k - 1 consumed, its partials written: xs[(k + 1) & 1] is free
     if (threadIdx.x == 0) {
@@ -401,19 +413,20 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
         if (src) bulk_store_wait_read(); // the store that still reads that buffer
         issue_x(k + 1, nx);
       }
-    } else if (threadIdx.x == 32) {    // count item k - 1 (the barrier ordered its partials before the fence)
-      int last = -1;
-      if (gprev >= 0 && !sm.fail) {
-        __threadfence();
-        if (atomicAdd(a.ticket + kGrTicketGroups + gprev, 1u) == (unsigned)a.nblk - 1u) last = gprev;
-        __threadfence();
+    } else if (threadIdx.x == 32) {
+      // item k - 2's count, asked for an item ago, is in by now
+      const int last = (counted >= 0 && count == (unsigned)a.nblk - 1u) ? counted : -1;
+      counted = -1;
+      if (gprev >= 0 && !sm.fail) {    // count item k - 1 (the barrier ordered its partials before the fence)
+        fence_acq_rel();
+        count = atomicAdd(a.ticket + kGrTicketGroups + gprev, 1u);
+        counted = gprev;
       }
+      if (last >= 0) fence_acq_rel();
       sm.last = last;
     }
     __syncthreads();
-    if (sm.last >= 0)                  // this group's chunks are all in: its entries of G
-      for (int jj = warp + kGrWarps * sm.last; jj < a.c; jj += kGrWarps * S)
-        finish_slot<kMode>(a.partials, a.nblk, jj, a.G, a.s_first, a.s_new, a.m, lane);
+    finish_group(sm.last);
     const int it = sm.iq[k & 1];
     if (sm.quit) {
       // copies issued but not consumed must land before the shared memory
@@ -427,7 +440,16 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_row_bulk_kernel(GramRowArg
       if (src) ingest_rest(a, sm, itprev, it, nitems);
       break;
     }
-    if (it >= nitems) break;
+    if (it >= nitems) {                // the count of this CTA's last item
+      __syncthreads();
+      if (threadIdx.x == 32) {
+        sm.last = (counted >= 0 && count == (unsigned)a.nblk - 1u) ? counted : -1;
+        fence_acq_rel();
+      }
+      __syncthreads();
+      finish_group(sm.last);
+      break;
+    }
     const int ch = it / S, g = it - ch * S;
     gprev = g;
     itprev = it;
