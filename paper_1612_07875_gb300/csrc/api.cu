@@ -288,37 +288,69 @@ __global__ void __launch_bounds__(256) ingest_rows_kernel(const uint8_t* __restr
   }
 }
 
-// Up to 64 copies between device buffers in one launch (job blockIdx.y; 16
-// bytes at a time where both ends are 16-byte aligned, else 4): the ingest of
-// a batched push and the results of a batched eigensolver. As copies of their
-// own 64 ingests and 128 results took 0.9 ms of a 64-stream tick.
+// Up to 64 copies between device buffers in one launch: the ingest of a
+// batched push and the results of a batched eigensolver. As copies of their
+// own 64 ingests and 128 results took 0.9 ms of a 64-stream tick. Block
+// blockIdx.x copies one span of one job (16 bytes at a time where both ends are
+// 16-byte aligned, else 4), so every job has blocks by its bytes: with the same
+// number for all jobs a push of one 256 MB snapshot beside 63 small ones took
+// 1,047 us (935 as 64 copies), now 570.
 struct CopyJobs {
   const void* src[kMaxBatchJobs];
   void* dst[kMaxBatchJobs];
   int64_t bytes[kMaxBatchJobs];
+  int32_t first[kMaxBatchJobs];          // first block of each job (set by launch_copy_jobs)
+  int64_t span;                          // bytes per block, a multiple of 16
+  int32_t count;
 };
+constexpr int64_t kCopySpan = 16 * 256 * 4;   // four vectors a thread
 __global__ void __launch_bounds__(256) copy_jobs_kernel(const __grid_constant__ CopyJobs a) {
-  const uint8_t* s = static_cast<const uint8_t*>(a.src[blockIdx.y]);
-  uint8_t* d = static_cast<uint8_t*>(a.dst[blockIdx.y]);
-  const int64_t bytes = a.bytes[blockIdx.y];
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  int lo = 0, hi = a.count - 1;          // the last job whose first block is not past this one
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.first[mid] <= (int)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const int64_t at = (int64_t)((int)blockIdx.x - a.first[lo]) * a.span;
+  const uint8_t* s = static_cast<const uint8_t*>(a.src[lo]) + at;
+  uint8_t* d = static_cast<uint8_t*>(a.dst[lo]) + at;
+  const int64_t bytes = min(a.span, a.bytes[lo] - at), t = threadIdx.x;
   if (((reinterpret_cast<uintptr_t>(s) | reinterpret_cast<uintptr_t>(d)) & 15u) == 0) {
     const uint4* sv = reinterpret_cast<const uint4*>(s);
     uint4* dv = reinterpret_cast<uint4*>(d);
     const int64_t nv = bytes / 16;
     int64_t i = t;
-    for (; i + 3 * stride < nv; i += 4 * stride) {
-      const uint4 w = sv[i], x = sv[i + stride], y = sv[i + 2 * stride], z = sv[i + 3 * stride];
+    for (; i + 768 < nv; i += 1024) {
+      const uint4 w = sv[i], x = sv[i + 256], y = sv[i + 512], z = sv[i + 768];
       dv[i] = w;
-      dv[i + stride] = x;
-      dv[i + 2 * stride] = y;
-      dv[i + 3 * stride] = z;
+      dv[i + 256] = x;
+      dv[i + 512] = y;
+      dv[i + 768] = z;
     }
-    for (; i < nv; i += stride) dv[i] = sv[i];
+    for (; i < nv; i += 256) dv[i] = sv[i];
     if (t < bytes % 16) d[16 * nv + t] = s[16 * nv + t];
   } else {
-    for (int64_t i = t; i < bytes / 4; i += stride) reinterpret_cast<unsigned*>(d)[i] = reinterpret_cast<const unsigned*>(s)[i];
+    for (int64_t i = t; i < bytes / 4; i += 256) reinterpret_cast<unsigned*>(d)[i] = reinterpret_cast<const unsigned*>(s)[i];
   }
+}
+
+// Fills in the spans of a (count jobs) and launches it: kCopySpan bytes a
+// block, more once that would be eight blocks an SM.
+cudaError_t launch_copy_jobs(CopyJobs* a, int count, int num_sms, cudaStream_t st) {
+  int64_t total = 0;
+  for (int i = 0; i < count; ++i) total += a->bytes[i];
+  const int64_t most = 8 * (int64_t)(num_sms > 0 ? num_sms : 1);
+  const int64_t times = (total + kCopySpan * most - 1) / (kCopySpan * most);
+  a->span = kCopySpan * (times > 1 ? times : 1);
+  a->count = count;
+  int32_t blocks = 0;
+  for (int i = 0; i < count; ++i) {
+    a->first[i] = blocks;
+    const int64_t b = (a->bytes[i] + a->span - 1) / a->span;
+    blocks += b > 1 ? (int32_t)b : 1;
+  }
+  copy_jobs_kernel<<<(unsigned)blocks, 256, 0, st>>>(*a);
+  return cudaGetLastError();
 }
 
 // Time-ordered copy of the physical G; `words` 8-byte words per entry.
@@ -1084,11 +1116,7 @@ int sdmd_push_many(const sdmd_t* hs, const void* const* xs, int32_t count, void*
   cudaError_t e = cudaSuccess;
   // one launch when every snapshot is aligned memory of this GPU, else a copy each
   bool all_dev = true;
-  int64_t most = 0;
-  for (int i = 0; i < plan.ncopies; ++i) {
-    all_dev = all_dev && row_ingests(plan.src[i], hs[0]->device);
-    if ((int64_t)plan.bytes[i] > most) most = (int64_t)plan.bytes[i];
-  }
+  for (int i = 0; i < plan.ncopies; ++i) all_dev = all_dev && row_ingests(plan.src[i], hs[0]->device);
   if (all_dev) {
     CopyJobs cj;
     for (int i = 0; i < plan.ncopies; ++i) {
@@ -1096,13 +1124,8 @@ int sdmd_push_many(const sdmd_t* hs, const void* const* xs, int32_t count, void*
       cj.dst[i] = plan.dst[i];
       cj.bytes[i] = (int64_t)plan.bytes[i];
     }
-    int64_t bx = (most + 256 * 64 - 1) / (256 * 64);               // four vectors a thread for the longest
-    const int64_t lim = (8 * (int64_t)hs[0]->num_sms + count - 1) / count;
-    if (bx > lim) bx = lim;
-    if (bx < 1) bx = 1;
     TraceScope ts(hs[0], SDMD_K_INGEST, st);
-    copy_jobs_kernel<<<dim3((unsigned)bx, (unsigned)count), 256, 0, st>>>(cj);
-    e = cudaGetLastError();
+    e = launch_copy_jobs(&cj, plan.ncopies, hs[0]->num_sms, st);
     if (e == cudaSuccess) copied = plan.ncopies;
   }
   for (int i = copied; i < plan.ncopies && e == cudaSuccess; ++i) {
@@ -1312,8 +1335,7 @@ int sdmd_modes_many(const sdmd_t* hs, int32_t count, const int32_t* r, void* con
   }
   for (int q = 0; q < 2; ++q) {
     if (nj[q] == 0) continue;
-    copy_jobs_kernel<<<dim3(1, (unsigned)nj[q]), 256, 0, st>>>(jobs[q]);
-    CK(cudaGetLastError());
+    CK(launch_copy_jobs(&jobs[q], nj[q], hs[0]->num_sms, st));
   }
   return SDMD_OK;
 }
