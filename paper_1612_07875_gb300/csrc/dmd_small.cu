@@ -1686,6 +1686,14 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     return at;
   };
   const int64_t re2 = (int64_t)re * re;
+  // The Schur iteration is one warp's chain of dependent accesses to H and Q:
+  // when the whole eigenproblem does not fit, those two come first (phase 7, r
+  // = 100 of 199 pairs: 125 million cycles with them in global memory, whose L1
+  // is what the kernel's shared memory leaves, 36 on chip)
+  const int64_t y_units = (used + (int64_t)re * p <= plan.pool_units) ? (int64_t)re * p : 0;
+  const bool whole = used + y_units + (1 + kEigUnits) * re2 <= plan.pool_units;
+  CF* Hc = whole ? nullptr : reinterpret_cast<CF*>(take(re2, nullptr));
+  CF* Qc = whole ? nullptr : reinterpret_cast<CF*>(take(re2, nullptr));
   dd* Yb = take((int64_t)re * p, w.Y);
   dd* At = take((1 + kEigUnits) * re2, nullptr);   // re x re df64, then the eigenproblem
   const bool eig_on_chip = At != nullptr;
@@ -1720,9 +1728,10 @@ __device__ __forceinline__ void modes_small_body(const ModesArgs& a, const Modes
     Yb[idx] = dd_add(s0, s1);
   }
   __syncthreads();
-  CF* Hc = reinterpret_cast<CF*>(At + re2);
-  CF* Qc = Hc + re2;
-  CF* Wc = Qc + re2;
+  CF* eig = reinterpret_cast<CF*>(At + re2);       // H, Q, W, U, y
+  if (!Hc) Hc = eig;
+  if (!Qc) Qc = eig + re2;
+  CF* Wc = eig + 2 * re2;
   CF* Uc = Wc + re2;
   CF* yc = Uc + re2;
   for (int idx = tid; idx < re * re; idx += kThreads) {
@@ -2360,7 +2369,7 @@ __host__ __device__ ModesLayout modes_layout(int m) {
   L.sig = take(p);
   L.lamout = take(2 * p);
   L.tmp = 0;
-  L.lu = take(6 * p2 + 64); // off chip: tridiagonal LU per vector (5 r p) or Ritz scratch (r p); A~ and eig (6 r^2)
+  L.lu = take(6 * p2 + 64); // off chip: tridiagonal LU per vector (4 1/8 r p) or Ritz scratch (r p); A~ and eig (6 r^2)
   L.clk = take(16);
   L.bamp = take(2 * p + 2);  // b (re, im) per mode, then [2p] = background index
   L.urec = take(p);          // 2p floats
