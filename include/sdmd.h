@@ -482,10 +482,17 @@ SDMD_API int sdmd_set_option(sdmd_t h, int32_t option, int64_t value);
 
 /* Kernel classes for tracing. */
 enum {
-    SDMD_K_INGEST = 0,    /* snapshot copy into its ring slot (sdmd_push from
-                             16-byte aligned device memory: part of the row)  */
+    SDMD_K_INGEST = 0,    /* copy of snapshots into their ring slots: one record
+                             per copy, or for the launch that copies several
+                             (sdmd_push_batch and sdmd_push_many from device
+                             memory; sdmd_push_many records it on every handle).
+                             Part of the row, and not recorded: sdmd_push and
+                             sdmd_push_batch's single pushes from this GPU's
+                             memory, 16-byte aligned, and sdmd_push_sparse from
+                             this GPU's memory                                 */
     SDMD_K_GRAM_ROW = 1,  /* Gram-row multi-dot + symmetric insert            */
-    SDMD_K_MODES = 2,     /* FP64 eigensolvers / small products (one CTA)     */
+    SDMD_K_MODES = 2,     /* eigensolvers and small products (one CTA, or a
+                             cluster of CTAs for long and complex windows)    */
     SDMD_K_PHI = 3,       /* Phi = X' (V Sigma^-1 W)                          */
     SDMD_K_FRAME = 4,     /* one sdmd_step frame: call start to outputs done  */
     SDMD_K_FUSED = 5,     /* Phi of an earlier frame + this snapshot's Gram row in one pass */

@@ -1124,7 +1124,8 @@ int sdmd_push_many(const sdmd_t* hs, const void* const* xs, int32_t count, void*
       cj.dst[i] = plan.dst[i];
       cj.bytes[i] = (int64_t)plan.bytes[i];
     }
-    TraceScope ts(hs[0], SDMD_K_INGEST, st);
+    std::deque<TraceScope> ts;           // every handle's ingest is this launch
+    for (int i = 0; i < count; ++i) ts.emplace_back(hs[i], SDMD_K_INGEST, st);
     e = launch_copy_jobs(&cj, plan.ncopies, hs[0]->num_sms, st);
     if (e == cudaSuccess) copied = plan.ncopies;
   }
