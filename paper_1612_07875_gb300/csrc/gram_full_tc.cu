@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
       const int row = 8 * (cw + kConvWarps * gi) + (lane & 7);
       st_ok[gi] = gi < ng && row <= c && row != kt;
     }
-    // stage sequence: chunk k covers stages 16 k .. 16 k + 15 of this CTA, two a K-step
+    // stage sequence: chunk k covers stages kHalvesPerChunk k .. of this CTA, two a K-step
     constexpr int kHalvesPerChunk = kStepsPerChunk * kHalves;
     int ld_count = 0, nvalid = 0x7fffffff, cbase = 0, o = 0, ck = 0;
     bool ended = false;
@@ -277,6 +277,9 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
       const bool tail = p0 + kKst > a.n;     // positions past n contribute nothing
 #pragma unroll
       for (int hf = 0; hf < kHalves; ++hf) {
+        // the load refills the stage of the half before: every lane has read it
+        // (the K-step's last one: the warp barrier before the hand-over)
+        if (hf > 0) __syncwarp();
         load_next();
         cp_async_wait<kStages - 1>();        // this lane's copies of the stage have landed
         __syncwarp();                        // ... and those of the other lanes
@@ -290,7 +293,6 @@ __global__ void __launch_bounds__(kThreads, 1) gram_full_tc_kernel(GramFullArgs 
             w[gi][0] = *reinterpret_cast<const uint4*>(r);
             w[gi][1] = *reinterpret_cast<const uint4*>(r + 64);
           }
-        __syncwarp();                        // every lane has read the stage: the next load refills it
 #pragma unroll
         for (int gi = 0; gi < kGroups; ++gi) {
           if (gi >= ng) break;               // warp-uniform
