@@ -131,6 +131,8 @@ SDMD_API int sdmd_destroy(sdmd_t h);
  * overwritten, not moved. Before the window is full nothing is evicted
  * (ramp-up, Sec. 5). FP32: products in FP32 over short runs, sums in FP64,
  * fixed reduction order (deterministic for a given n and GPU). U8: exact.
+ * If a device wait gives up (sdmd_status: SDMD_ERR_TIMEOUT) the row of G is
+ * incomplete, but the snapshot is in its slot: sdmd_rebuild restores G.
  */
 SDMD_API int sdmd_push(sdmd_t h, const void *x, void *stream);
 

@@ -1261,8 +1261,9 @@ struct SmemPlan {
 // less the kernel's static arrays, with margin.
 constexpr int64_t kSmemDynUnits = (216 * 1024) / 8;
 // LU factors of one vector: 1 / u0, u1, u2, multipliers (p each), the row swaps
-// (bytes). 4 1/8 p units and not 5 p, so 20 vectors of 255 pairs fit the pool:
-// 64 calls of 255 pairs together 6678 us, 7184 us with their LU off chip.
+// (bytes). 4 1/8 p units and not 5 p, so 20 vectors of 255 pairs fit the pool: a
+// tick of 64 streams with windows of 16 to 256 snapshots, rows and eigensolvers,
+// 6,678 us, 7,184 with the longest windows' LU off chip.
 __host__ __device__ constexpr int lu_units(int p) { return 4 * p + (p + 7) / 8; }
 constexpr int kEigUnits = 8;   // H, Q, W, U, two y (complex float) and the products A~ w (two df64) per r x r
 
@@ -2382,10 +2383,14 @@ __host__ __device__ ModesLayout modes_layout(int m) {
 int64_t modes_ws_doubles(int m) { return modes_layout(m).total; }
 
 // The complex windows whose G_X goes through the embedding: 2p <= 144, at most
-// 32 Ritz vectors (2K plus the cluster extension), and a working set (G_X, 40
-// vectors, the Ritz matrices, seven vectors per wanted eigenpair) within one
-// SM, or else within the workspace that is laid out for p. The line was drawn
-// where the embedded solver's accuracy and time were measured.
+// 32 Ritz vectors (2K plus the cluster extension), and a sum of shared memory
+// by an earlier layout of the kernel, or else of workspace. Under smem_plan
+// every window within the first two limits fits on chip; the sum stays because
+// it decides which algorithm a window gets (df64 on the embedding or FP64
+// Jacobi), so its rounding too. It takes windows of up to 71 snapshots for r <=
+// 8; for r = 9 up to 47 and 53 to 71, for r = 10 up to 45 and 57 to 71, for r =
+// 11 up to 44 and 61 to 70, for r = 12 up to 42 and 65 to 70; beyond r = 12 up to
+// 17. The gaps take the Jacobi sweeps (r = 10: 7.0 ms at 50 snapshots, 1.7 at 64).
 bool modes_embed_ok(int c, int r) {
   const int pc = c - 1, K = (r < pc) ? r : pc, p = 2 * pc;
   const int P = (p + 3) & ~3;

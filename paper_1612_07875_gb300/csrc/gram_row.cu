@@ -28,8 +28,8 @@
 // kernel also is the ingest: x_new's chunks come from x_src, the items of
 // group 0 write them to the ring slot, and <x_new, x_new> is formed from the
 // staged chunk, so the snapshot is read once and its slot not at all. Against
-// a copy kernel before this one a push of one HD frame (m = 100) went from 124
-// to 114 us, one of a 64 x 64 FP32 field (m = 32, launches only) from 22.5 to
+// a copy kernel before this one a push of one HD frame (m = 100) went from 125
+// to 116 us, one of a 64 x 64 FP32 field (m = 32, launches only) from 22.5 to
 // 14.3 us. (Snapshots of 2^28 bytes in windows of 64 and more slots, 17 GB, are
 // the exception: 2,545 us with the copy, 2,578.)
 //

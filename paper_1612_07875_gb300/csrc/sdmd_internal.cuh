@@ -234,8 +234,8 @@ cudaError_t modes_batch_split(const ModesBatch& b, ModesBatch (&part)[2], size_t
 // The same outputs for complex windows (G complex128 Hermitian): FP64 Jacobi
 // for G_X, complex A~, W, M and amplitudes.
 cudaError_t launch_modes_complex(const ModesArgs& a, cudaStream_t st);
-// Whether a complex window of c snapshots and rank r can take the embedded
-// df64 path (its working set fits what that path may use).
+// Whether a complex window of c snapshots and rank r takes the embedded df64
+// path.
 bool modes_embed_ok(int c, int r);
 
 struct PhiArgs {
